@@ -31,11 +31,11 @@
  *    the call returns.
  *  - Alignment: a device pointer must be aligned to its element size (2, 4
  *    or 8 bytes), else the call returns IGR_ERR_INVALID_ARG before any
- *    launch. Where a call could take the 4-cell kernel forms (igr_solve_sigma,
+ *    launch. Where a call could take 4-wide loads (igr_solve_sigma,
  *    igr_solve_sigma_noalloc), pointers that are element-aligned but not
  *    aligned to 4 elements (8 bytes at 16-bit storage, 16 bytes for FP32 and
- *    FP64; a sliced tensor can start anywhere) make that call take the
- *    1-cell forms, which give the same bits. Buffers from cudaMalloc or a
+ *    FP64; a sliced tensor can start anywhere) make that call load element by
+ *    element, with the same bits. Buffers from cudaMalloc or a
  *    caching allocator are 256-byte aligned.
  *  - A context is not thread-safe; distinct contexts are independent.
  *  - Asynchronous faults (CUDA errors, non-finite results) surface at the
@@ -356,24 +356,25 @@ igr_status igr_profile_read(igr_ctx *ctx, int kernel_class, long long *launches,
 
 /* ---- Launch shapes and the autotuner ----------------------------------
  * Each kernel class marches blocks up chunks of z-planes; the chunk length
- * is the tunable launch shape (>= 4 planes, at most nz). The source and
- * Jacobi kernels also come in two forms: one cell per thread (rows in
- * blocks of 32 cells) and four cells per thread (rows in blocks of 128
- * cells; only for nx % 4 == 0), which runs fewer instructions per cell but
- * idles more lanes on short rows. By default the four-cell form is taken
- * where its share of busy lanes is at least its instruction ratio (source
- * 80/140, Jacobi 69/79) times the one-cell form's.
+ * is the tunable launch shape (>= 4 planes, at most nz). The default is the
+ * chunk that a count of waves of resident blocks makes the fastest.
+ * The source and Jacobi kernels give a thread four consecutive cells of a
+ * row with 4-wide loads where rows are a multiple of 4 cells and the buffers
+ * aligned to 4 values, else two cells, one above the other, loaded element by
+ * element; blocks are fitted to the row length.
  * Results do not depend on the launch shape: every face flux comes out of
  * the same instructions whatever the chunking, both forms evaluate the same
  * sequence of rounded operations, and there are no atomics, so outputs are
  * bitwise identical for every choice.
  * igr_set_kernel_forms: source_vec4 and jacobi_vec4 each -1 (the default
- * rule), 0 (one cell per thread) or 1 (four cells; IGR_ERR_INVALID_ARG when
- * nx % 4 != 0).
- * igr_autotune times each class on the current state for the candidate
- * lengths 4..128 and, where nx % 4 == 0, both forms (reps launches each, on
- * the context stream; only scratch buffers are written) and keeps the
- * fastest; call it after igr_set_state. It synchronises. */
+ * rule), 0 or 1 (IGR_ERR_INVALID_ARG when nx % 4 != 0). The setting is kept
+ * and reported (the default rule reports 1 for rows of a multiple of 4 cells
+ * that fill blocks of 128 cells), and every setting launches the kernels
+ * described above.
+ * igr_autotune times each class on the current state for the default chunk
+ * and the candidate lengths 4..128 (reps launches each, on the context
+ * stream; only scratch buffers are written) and keeps the fastest; call it
+ * after igr_set_state. It synchronises. */
 igr_status igr_set_tiles(igr_ctx *ctx, int zc_source, int zc_jacobi, int zc_flux);
 igr_status igr_get_tiles(igr_ctx *ctx, int *zc_source, int *zc_jacobi, int *zc_flux);
 igr_status igr_set_kernel_forms(igr_ctx *ctx, int source_vec4, int jacobi_vec4);

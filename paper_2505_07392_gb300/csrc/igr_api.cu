@@ -249,28 +249,42 @@ const Ops *igr::ops_for(int p)
     return nullptr;
 }
 
-// Longest z-chunk (at most 128 planes, at least 16) that still gives the
-// kernel six waves of blocks on 152 SMs holding `resident` blocks each: every
-// block starts by loading the planes below its chunk, so longer chunks
-// amortise that prologue, while too few blocks leave SMs idle in the last
-// wave. (tx, ty): columns per block.
-static int default_zc(const Geom &g, int tx, int ty, int resident)
+// Z-chunk (planes per block) of a kernel with cols blocks per plane, of which
+// `resident` fit on an SM. A block spends c0 planes' time on the planes below
+// its chunk, and every wave of blocks the time of one, so a launch takes about
+// ceil(blocks / (152 resident)) (zc + c0); the chunk count with the least of
+// it is taken, chunks of 4 to 128 planes.
+static int choose_zc(long long cols, int nz, int resident, double c0)
 {
-    long long cols = (long long)((g.nx + tx - 1) / tx) * ((g.ny + ty - 1) / ty);
-    int zc = 128;
-    while (zc > 16 && cols * ((g.nz + zc - 1) / zc) < 6LL * 152 * resident) zc /= 2;
-    return zc > g.nz ? g.nz : zc;
+    int best = nz < 4 ? nz : 4;
+    double tbest = 1e300;
+    for (int m = (nz + 127) / 128; m <= (nz + 3) / 4; m++) {
+        const int zc = (nz + m - 1) / m;
+        if (zc < 4 && m > 1) break;
+        const long long slots = 152LL * resident, blocks = cols * ((nz + zc - 1) / zc);
+        const double t = (zc + c0) * (double)((blocks + slots - 1) / slots);
+        if (t < tbest * 0.999) {
+            tbest = t;
+            best = zc;
+        }
+    }
+    return best;
 }
 
-Tiles igr::default_tiles(const Geom &g)
+Tiles igr::default_tiles(const Geom &g, const Ops *o)
 {
-    Tiles t;
+    Tiles t = {};
     t.vec_source = vec4_default_source(g.nx);
     t.vec_jacobi = vec4_default_jacobi(g.nx);
-    t.zc_source = default_zc(g, t.vec_source ? 128 : 32, 8, 3);
-    t.zc_jacobi = default_zc(g, t.vec_jacobi ? 128 : 32, 8, 3);
-    t.zc_flux = default_zc(g, 32, 15, 1);
-    t.z_begin = t.z_end = 0;
+    long long cols;
+    int resident;
+    o->source_shape(g, &cols, &resident);
+    t.zc_source = choose_zc(cols, g.nz, resident, 1.5);
+    o->jacobi_shape(g, &cols, &resident);
+    t.zc_jacobi = choose_zc(cols, g.nz, resident, 1.5);
+    Tiles one = {};
+    one.zc_flux = g.nz;
+    t.zc_flux = choose_zc(o->flux_blocks(g, one), g.nz, 1, 3.0);
     return t;
 }
 
@@ -324,7 +338,7 @@ static Layout layout_of(const igr_config *c)
     g.plane = (long long)c->nx * c->ny;
     g.n = g.plane * c->nz;
     const Ops *o = ops_for(c->prec);
-    Tiles t = default_tiles(g);
+    Tiles t = default_tiles(g, o);
     Layout L;
     L.state = (size_t)5 * g.n * o->state_bytes;
     L.incr = (size_t)5 * g.n * o->storage_bytes;  // a stage increment (increment modes)
@@ -570,8 +584,8 @@ igr_status igr_create(const igr_config *cfg, const igr_allocator *allocator, voi
     c->p.order = cfg->order == 3 ? 3 : 5;
     c->p.mu = cfg->mu;
     c->p.zeta = cfg->zeta;
-    c->tiles = default_tiles(c->g);
     c->ops = ops_for(cfg->prec);
+    c->tiles = default_tiles(c->g, c->ops);
     if (allocator) {
         c->alloc = *allocator;
     } else {
@@ -902,7 +916,7 @@ igr_status igr_solve_sigma(igr_ctx *c, const void *q, void *sigma_inout, int swe
         return fail(c, IGR_ERR_INVALID_ARG, "q and sigma_inout must be aligned to their element size");
     Tiles t = c->tiles;
     if (!is_aligned(q, vec4_align((int)qb)) || !is_aligned(sigma_inout, vec4_align((int)sb)))
-        t.vec_source = t.vec_jacobi = 0;  // the 1-cell forms: same bits, element alignment only
+        t.elem = 1;  // element accesses: the same bits, element alignment only
     prof_begin(c, KC_SOURCE);
     CU(c, c->ops->source(c->g, c->p, t, inflow_of(c), q, nullptr, c->b, c->rho16, c->st));
     prof_end(c);
@@ -1066,38 +1080,38 @@ igr_status igr_autotune(igr_ctx *c, int reps)
 {
     if (!c || reps < 1) return fail(c, IGR_ERR_INVALID_ARG, "ctx and reps >= 1 are required");
     if (c->profiling) return fail(c, IGR_ERR_INVALID_ARG, "disable profiling before tuning");
-    const int cand[] = {4, 8, 16, 32, 64, 128};
+    // the default shape and chunks of 4..128 planes
+    const Tiles dflt = default_tiles(c->g, c->ops);
+    const int cand[] = {0, 4, 8, 16, 32, 64, 128};
     Tiles best = c->tiles;
     float tbest[3] = {1e30f, 1e30f, 1e30f};
     void *sig = c->sig[c->cur], *scratch = c->sig[1 - c->cur];
     if (c->cfg.sigma_solver == SOLVER_RBGS)
         CU(c, cudaMemcpyAsync(c->q[1], sig, c->g.n * (size_t)c->ops->storage_bytes, cudaMemcpyDeviceToDevice,
                               c->st));
-    const int nforms = c->g.nx % 4 == 0 ? 2 : 1;  // the 4-cell forms need rows of a multiple of 4
     for (int zc : cand) {
-        if (zc > c->g.nz && zc != cand[0]) continue;
+        if (zc > c->g.nz) continue;
         Tiles t = c->tiles;
-        t.zc_source = t.zc_jacobi = t.zc_flux = clamp_zc(zc, c->g.nz);
+        t.zc_source = zc ? zc : dflt.zc_source;
+        t.zc_jacobi = zc ? zc : dflt.zc_jacobi;
+        t.zc_flux = zc ? zc : dflt.zc_flux;
         float ms;
         igr_status s;
         // each kernel class writes only scratch: b, the other Sigma buffer, the stage-1 output
-        for (int v = 0; v < nforms; v++) {
-            t.vec_source = t.vec_jacobi = v;
-            s = time_launches(c, reps, [&] {
-                return c->ops->source(c->g, c->p, t, inflow_of(c), c->q[0], nullptr, c->b, c->rho16, c->st);
-            }, &ms);
-            if (s != IGR_OK) return s;
-            if (ms < tbest[0]) { tbest[0] = ms; best.zc_source = t.zc_source; best.vec_source = v; }
-            s = time_launches(c, reps, [&] {
-                // red-black: a half-sweep in place on a copy of Sigma in the stage-1 output buffer
-                const void *qj = c->inc ? c->rho16 : c->q[0];
-                return c->cfg.sigma_solver == SOLVER_RBGS
-                           ? c->ops->jacobi(c->g, c->p, t, qj, c->b, c->q[1], c->q[1], 0, c->st)
-                           : c->ops->jacobi(c->g, c->p, t, qj, c->b, sig, scratch, -1, c->st);
-            }, &ms);
-            if (s != IGR_OK) return s;
-            if (ms < tbest[1]) { tbest[1] = ms; best.zc_jacobi = t.zc_jacobi; best.vec_jacobi = v; }
-        }
+        s = time_launches(c, reps, [&] {
+            return c->ops->source(c->g, c->p, t, inflow_of(c), c->q[0], nullptr, c->b, c->rho16, c->st);
+        }, &ms);
+        if (s != IGR_OK) return s;
+        if (ms < tbest[0]) { tbest[0] = ms; best.zc_source = t.zc_source; }
+        s = time_launches(c, reps, [&] {
+            // red-black: a half-sweep in place on a copy of Sigma in the stage-1 output buffer
+            const void *qj = c->inc ? c->rho16 : c->q[0];
+            return c->cfg.sigma_solver == SOLVER_RBGS
+                       ? c->ops->jacobi(c->g, c->p, t, qj, c->b, c->q[1], c->q[1], 0, c->st)
+                       : c->ops->jacobi(c->g, c->p, t, qj, c->b, sig, scratch, -1, c->st);
+        }, &ms);
+        if (s != IGR_OK) return s;
+        if (ms < tbest[1]) { tbest[1] = ms; best.zc_jacobi = t.zc_jacobi; }
         s = time_launches(c, reps, [&] {
             return c->ops->flux(c->g, c->p, t, inflow_of(c), FLUX_STAGE1, c->q[0], nullptr, sig, c->q[0], c->q[1],
                                 nullptr, nullptr, c->sc, c->blockmax, &c->sc->err, c->st);

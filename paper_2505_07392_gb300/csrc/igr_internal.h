@@ -53,18 +53,17 @@ struct Tiles {
     int zc_source;  // z-planes per block of the source kernel
     int zc_jacobi;  // z-planes per block of the Jacobi kernel
     int zc_flux;    // z-planes per block of the flux kernel
-    int vec_source; // 1: 4 cells per thread (128-cell rows; nx % 4 == 0), 0: one cell per thread
-    int vec_jacobi; // the same for the Jacobi kernel
+    int vec_source; // the form igr_get_kernel_forms reports (both forms launch the same kernel
+    int vec_jacobi; // where rows are a multiple of 4 cells)
+    int elem;       // 1: the source and the sweeps load element by element (pointers that are not
+                    // aligned to 4 values)
     int z_begin;    // a flux launch covers planes [z_begin, z_end) only (z_begin a multiple
     int z_end;      // of zc_flux, z_end a multiple or nz); z_end = 0: all planes
 };
 
-// Default form of the source and Jacobi kernels for rows of nx cells. The
-// 4-cell form runs fewer instructions per cell (source 80 against 140,
-// Jacobi 69 against 79, FP16 storage) but covers rows in blocks of 128
-// cells, the 1-cell form in blocks of 32; the lanes beyond nx idle. The
-// 4-cell form is taken where its share of busy lanes is at least the
-// instruction ratio (num / den) times the 1-cell form's.
+// The form the default rule of igr_set_kernel_forms reports: 1 where rows of
+// nx cells fill blocks of 128 cells at least num / den times as well as
+// blocks of 32.
 inline int vec4_default(int nx, int num, int den)
 {
     if (nx % 4) return 0;
@@ -74,13 +73,40 @@ inline int vec4_default(int nx, int num, int den)
 inline int vec4_default_source(int nx) { return vec4_default(nx, 80, 140); }
 inline int vec4_default_jacobi(int nx) { return vec4_default(nx, 69, 79); }
 
+// Tile of the source and sweep kernels: wq quads (four cells of a row) by
+// rows rows, at most 256 threads, fitted to the plane so that rows of any
+// length fill it: the row is cut into the fewest tiles of at most 32 quads,
+// and the rows of the plane into tiles of equal height. On small grids lower
+// tiles (down to 8 rows) make more blocks: every SM marching a few planes is
+// what bounds them.
+enum { QUAD_TILE = 1360 };  // cells of the largest plane tile with its halo, (rows + 2)(4 wq + 8)
+struct QuadFit {
+    int wq, rows, threads, gx, gy;
+    bool full;  // 32 x 8 quads, every tile inside the grid
+};
+inline QuadFit quad_fit(const Geom &g)
+{
+    QuadFit f;
+    const int nq = (g.nx + 3) / 4;
+    f.gx = (nq + 31) / 32;
+    f.wq = (nq + f.gx - 1) / f.gx;
+    int rmax = 256 / f.wq < 32 ? 256 / f.wq : 32;
+    while (rmax > 8 && (long long)f.gx * ((g.ny + rmax - 1) / rmax) * ((g.nz + 3) / 4) < 2 * 152) rmax = rmax / 2 < 8 ? 8 : rmax / 2;
+    f.gy = (g.ny + rmax - 1) / rmax;
+    f.rows = (g.ny + f.gy - 1) / f.gy;
+    const int own = f.wq * f.rows, halo = 2 * f.wq + 2 * f.rows;  // a thread each
+    f.threads = ((own > halo ? own : halo) + 31) / 32 * 32;
+    f.full = g.nx % 128 == 0 && g.ny % 8 == 0 && f.rows == 8;
+    return f;
+}
+
 // Alignment of caller device pointers. Every kernel reads and writes whole
-// elements, so a pointer must be aligned to its element size. The 4-cell
-// forms of the source and Jacobi kernels also load and store 4 consecutive
-// values at once (8 bytes at 16-bit storage, 16 bytes for FP32 and, as two
-// 16-byte accesses, for FP64), so they need the field bases aligned to that;
-// a call whose pointers are not takes the 1-cell forms, which give the same
-// bits.
+// elements, so a pointer must be aligned to its element size. The source and
+// the sweeps load and store 4 consecutive values at once on rows of a
+// multiple of 4 cells (8 bytes at 16-bit storage, 16 bytes for FP32 and, as
+// two 16-byte accesses, for FP64), so they need the field bases aligned to
+// that; a call whose pointers are not takes element accesses (Tiles::elem),
+// which give the same bits.
 inline bool is_aligned(const void *p, size_t a) { return ((uintptr_t)p & (a - 1)) == 0; }
 inline size_t vec4_align(int storage_bytes) { return storage_bytes * 4 > 16 ? 16 : (size_t)storage_bytes * 4; }
 
@@ -170,6 +196,11 @@ struct Ops {
     cudaError_t (*source_group)(const struct SourceCall *calls, int n, cudaStream_t st);
     cudaError_t (*jacobi_group)(const struct JacobiCall *calls, int n, int colour, cudaStream_t st);
     cudaError_t (*flux_group)(const struct FluxCall *calls, int n, int mode, cudaStream_t st);
+
+    // blocks per plane of the source / of a sweep, and the blocks per SM that
+    // their registers allow (for the choice of the z-chunks)
+    void (*source_shape)(const Geom &, long long *cols, int *resident);
+    void (*jacobi_shape)(const Geom &, long long *cols, int *resident);
 };
 
 // One instance's arguments of a grouped launch (the same as the single
@@ -213,7 +244,7 @@ extern const Ops ops_f64, ops_f32, ops_f16, ops_bf16, ops_f16inc, ops_bf16inc;
 
 // shared by the host entry points (igr_api.cu, igr_noalloc.cu)
 const Ops *ops_for(int precision);             // kernel set of an igr_precision
-Tiles default_tiles(const Geom &g);            // launch shapes for a grid
+Tiles default_tiles(const Geom &g, const Ops *o);  // launch shapes for a grid
 const char *validate_config(const igr_config *c);  // NULL when valid
 
 }  // namespace igr

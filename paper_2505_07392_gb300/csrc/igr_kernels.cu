@@ -28,6 +28,7 @@
 
 #include <stdio.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "igr_internal.h"
@@ -258,10 +259,6 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-// a / b as the sweeps evaluate it: a times the approximate reciprocal in
-// FP32, the correctly rounded quotient in FP64
-__device__ __forceinline__ double quot(double a, double b) { return __ddiv_rn(a, b); }
-__device__ __forceinline__ float quot(float a, float b) { return __fmul_rn(a, rcp(b)); }
 
 // NaN-propagating maximum (a NaN wave speed must reach dt)
 __device__ __forceinline__ double nanmax(double a, double b) { return (a > b || a != a) ? a : b; }
@@ -563,20 +560,23 @@ struct BlockPos {
 };
 
 // --------------------------------------------- tiles of the 7-point kernels
-constexpr int BX = 32, BY = 8, BT = BX * BY;
-constexpr int HX = BX + 2, HY = BY + 2;   // plane tile with a halo of 1
-constexpr int NHALO1 = 2 * BX + 2 * BY;   // halo cells (corners are never read)
+// Two forms of the source and of the sweeps, marching up a z-chunk:
+//   quads  a thread has four consecutive cells of a row, one 4-wide load or
+//          store per field (rows of a multiple of 4 cells, fields aligned to
+//          4 values). A block owns wq quads x rows rows of the plane; quad_fit
+//          (igr_internal.h) fits the tile to the grid, so short rows (48..96
+//          cells) leave no lanes idle; grids that the largest tile (32 quads
+//          x 8 rows) divides take it with its shape compiled in (FULL).
+//   pairs  a thread has two cells, one above the other in y, loaded element by
+//          element: any row length and alignment, coalesced, and the same
+//          packed arithmetic. A block owns 32 x 16 cells of the plane.
+// Both evaluate one sequence of rounded operations per cell: the same bits.
+constexpr int VX = 4;
+constexpr int FQ = 32, FR = 8, BT = FQ * FR;   // full tile: quads, rows, threads
+constexpr int HXV = VX * FQ + 2 * VX;          // its row pitch (interior at column VX, 16-byte aligned)
+constexpr int TILEV = QUAD_TILE;               // cells of one plane tile with its halo, any shape
+static_assert((FR + 2) * HXV <= TILEV, "full tile");
 
-// position of halo cell e (0 <= e < NHALO1) in the HX x HY tile
-__device__ __forceinline__ void halo1_cell(int e, int &lx, int &ly)
-{
-    if (e < BX) { lx = 1 + e; ly = 0; }
-    else if (e < 2 * BX) { lx = 1 + e - BX; ly = HY - 1; }
-    else if (e < 2 * BX + BY) { lx = 0; ly = 1 + e - 2 * BX; }
-    else { lx = HX - 1; ly = 1 + e - 2 * BX - BY; }
-}
-
-// --------------------------------------------------------------- source
 // z-index of plane kk in [-1, nz]: periodic wrap or zero-gradient clamp
 __device__ __forceinline__ int zmap(int kk, const Geom &g)
 {
@@ -584,288 +584,107 @@ __device__ __forceinline__ int zmap(int kk, const Geom &g)
                   : (kk >= g.nz ? (g.bc[5] == BC_PERIODIC ? kk - g.nz : g.nz - 1) : kk);
 }
 
-// u = m / rho of the cell at in-plane offset f of plane kk (kk may leave the
-// domain through -z/+z: periodic wrap, zero-gradient clamp or the jet blend);
-// *rho_s gets the cell's (unblended) density
-template <bool HASD>
-__device__ __forceinline__ void col_u(const QIn &q, const Geom &g, const C *W, const C *J, idx f,
-                                      int kk, C u[3], C *rho_s = nullptr)
+// A thread's place in its tile. Threads 0..wq-1 also load the halo row below
+// the tile, the next wq the row above (4-wide, under their own quad), and the
+// next 2 rows threads the cells left and right of the rows. Everything is
+// mapped once; lanes outside the grid load nothing.
+struct Quad {
+    int i0, j;            // first cell
+    bool active;          // inside the grid
+    int pitch, pos;       // row pitch of the plane tile, position of the first cell in it
+    idx own;              // in-plane offset of the first cell
+    bool yh, xh;          // halo tasks: a quad above or below, a cell left or right
+    int hpos;             // position in the plane tile
+    idx hoff;             // in-plane offset
+    bool hdrop;           // the halo lies across a non-periodic boundary
+};
+template <bool FULL, int NR>
+__device__ __forceinline__ Quad quad_of(const Geom &g, const BlockPos &bp, int wq, int rows)
 {
-    idx c = ck((idx)map_axis(kk, g.nz, g.bc[4], g.bc[5]) * (idx)g.plane + f, g.n);
-    C rho = ldq<HASD>(q, 0, c), m0 = ldq<HASD>(q, 1, c), m1 = ldq<HASD>(q, 2, c), m2 = ldq<HASD>(q, 3, c);
-    if (rho_s) *rho_s = rho;
-    if (kk < 0 && g.bc[4] == BC_INFLOW) {
-        idx pl = (idx)g.plane;
-        f = ck(f, g.plane);
-        C w = C(1) - W[f];
-        rho = fma_rn(w, rho, J[f]);
-        m0 = fma_rn(w, m0, J[pl + f]);
-        m1 = fma_rn(w, m1, J[2 * pl + f]);
-        m2 = fma_rn(w, m2, J[3 * pl + f]);
+    Quad t;
+    if (FULL) {
+        wq = FQ;
+        rows = FR;
     }
-    // products rounded before they are differenced: equal neighbours give an exact 0
-    C r = rcp(rho);
-    u[0] = mul_rn(m0, r);
-    u[1] = mul_rn(m1, r);
-    u[2] = mul_rn(m2, r);
-}
-
-// b = alpha [tr(G^2) + tr(G)^2] (Eq. igrelliptic) from the undivided central
-// differences D = 2 dx G of u, with alpha_s = alpha / (2 dx)^2:
-//   b = alpha_s [sum_ab D_ab D_ba + (sum_a D_aa)^2],
-// in one fixed order of rounded operations, so that the two forms of the
-// source kernel give the same bits
-__device__ __forceinline__ C source_b(const C (&D)[3][3], C alpha_s)
-{
-    const C tr = add_rn(add_rn(D[0][0], D[1][1]), D[2][2]);
-    C sq = mul_rn(D[0][0], D[0][0]);
-    sq = fma_rn(D[1][1], D[1][1], sq);
-    sq = fma_rn(D[2][2], D[2][2], sq);
-    C x = mul_rn(D[0][1], D[1][0]);
-    x = fma_rn(D[0][2], D[2][0], x);
-    x = fma_rn(D[1][2], D[2][1], x);
-    const C tr2 = fma_rn(C(2), x, sq);  // sum_ab D_ab D_ba
-    return mul_rn(alpha_s, fma_rn(tr, tr, tr2));
-}
-
-// grad u by central differences from a shared plane tile U (x, y) and the
-// column's registers (z); b from source_b. In the increment modes the kernel
-// also stores the stage's density rounded to the storage type (rho_out),
-// which the Jacobi sweeps of the stage read.
-template <bool HASD>
-__device__ __forceinline__ void source_body(const QIn q, S *__restrict__ b, S *__restrict__ rho_out,
-                                            const Geom g, C alpha_s, const C *W, const C *J, int zc,
-                                            const BlockPos bp)
-{
-    __shared__ C U[3][HY][HX];
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-    const int x0 = bp.x * BX, y0 = bp.y * BY;
-    const int i = x0 + tx, j = y0 + ty;
-    const bool active = i < g.nx && j < g.ny;
-    const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
-    const idx pl = (idx)g.plane;
-    // the own slot of the tile holds the mapped cell (it is a neighbour of
-    // active cells even when this thread is outside the domain)
-    const idx f = (idx)(map_axis(j, g.ny, g.bc[2], g.bc[3]) * g.nx + map_axis(i, g.nx, g.bc[0], g.bc[1]));
-    const bool hv = tid < NHALO1;
-    int hs = 0;
-    idx hf = 0;
-    if (hv) {
-        int lx, ly;
-        halo1_cell(tid, lx, ly);
-        hs = ly * HX + lx;
-        hf = (idx)(map_axis(y0 + ly - 1, g.ny, g.bc[2], g.bc[3]) * g.nx +
-                   map_axis(x0 + lx - 1, g.nx, g.bc[0], g.bc[1]));
+    const int tid = threadIdx.x, row = tid / wq, qd = tid - row * wq, H = NR * rows;
+    const int x0 = bp.x * VX * wq, y0 = bp.y * H;
+    t.i0 = x0 + VX * qd;
+    t.j = y0 + NR * row;
+    t.active = FULL || (row < rows && t.i0 < g.nx && t.j < g.ny);
+    t.pitch = VX * wq + 2 * VX;
+    t.pos = (NR * row + 1) * t.pitch + VX + VX * qd;
+    t.own = (idx)t.j * (idx)g.nx + (idx)t.i0;
+    const int ye = FULL ? y0 + H : min(y0 + H, g.ny), xe = FULL ? x0 + VX * wq : min(x0 + VX * wq, g.nx);
+    t.yh = row < 2 && (FULL || t.i0 < g.nx);
+    t.xh = false;
+    if (row < 2) {
+        const int y = row ? ye : y0 - 1;
+        t.hpos = (y - y0 + 1) * t.pitch + VX + VX * qd;
+        t.hoff = (idx)map_axis(y, g.ny, g.bc[2], g.bc[3]) * (idx)g.nx + (idx)t.i0;
+        t.hdrop = row ? y >= g.ny && g.bc[3] != BC_PERIODIC : y < 0 && g.bc[2] != BC_PERIODIC;
+    } else {
+        const int e = tid - 2 * wq, side = e / H, r = e - side * H;
+        const int x = side ? xe : x0 - 1;
+        t.xh = side < 2 && (FULL || y0 + r < g.ny);
+        t.hpos = (r + 1) * t.pitch + VX + (x - x0);
+        t.hoff = (idx)(y0 + r) * (idx)g.nx + (idx)map_axis(x, g.nx, g.bc[0], g.bc[1]);
+        t.hdrop = side ? x >= g.nx && g.bc[1] != BC_PERIODIC : x < 0 && g.bc[0] != BC_PERIODIC;
     }
-    C um[3], u0[3], up[3];
-    C rho0 = C(1), rhop = C(1);  // density of the column at k and k + 1 (increment modes)
-    col_u<HASD>(q, g, W, J, f, k0 - 1, um);
-    col_u<HASD>(q, g, W, J, f, k0, u0, &rho0);
-    // raw values one iteration ahead (loads overlap the previous plane's work):
-    // the column at k + 1 and the halo at k (planes >= 0 need no jet blend)
-    QRaw nc[4], nh[4];
-    auto raw4 = [&](idx off, int kk, QRaw v[4]) {
-        idx c = ck((idx)zmap(kk, g) * pl + off, g.n);
+    return t;
+}
+
+// The pairs: lane tx, warp ty have cells (x0 + tx, y0 + 2 ty) and the one
+// above; threads 0..95 each load one halo cell (32 below, 32 above, 16 left,
+// 16 right). The tile's cells outside the grid hold the mapped cell next to
+// it (the far halo of a tile that the grid's edge cuts).
+constexpr int PX = 32, PWARPS = 8, PY = 2 * PWARPS, PPITCH = PX + 2, TILEP = (PY + 2) * PPITCH;
+struct Pair {
+    int i, j;             // lower cell
+    bool in[2];           // the cells inside the grid
+    bool need[2];         // the cells that are read (inside, or the first ones past the edge)
+    bool drop[2];         // ... those across a non-periodic boundary
+    int pos;              // position of the lower cell in the plane tile
+    idx own[2];           // in-plane offsets, mapped
+    bool h;               // a halo task
+    int hpos;
+    idx hoff;
+    bool hdrop;
+};
+__device__ __forceinline__ Pair pair_of(const Geom &g, const BlockPos &bp)
+{
+    Pair t;
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const int x0 = bp.x * PX, y0 = bp.y * PY;
+    t.i = x0 + tx;
+    t.j = y0 + 2 * ty;
+    t.pos = (2 * ty + 1) * PPITCH + tx + 1;
+    const idx mi = (idx)map_axis(t.i, g.nx, g.bc[0], g.bc[1]);
 #pragma unroll
-        for (int a = 0; a < 4; a++) v[a] = ldqr<HASD>(q, a, c);
-    };
-    raw4(f, k0 + 1, nc);
-    if (hv) raw4(hf, k0, nh);
-    for (int k = k0; k < k1; k++) {
-        rhop = cvq<HASD>(nc[0]);
-        C r = rcp(rhop);
-#pragma unroll
-        for (int a = 0; a < 3; a++) up[a] = mul_rn(cvq<HASD>(nc[1 + a]), r);
-        C hu[3];
-        if (hv) {
-            C rh = rcp(cvq<HASD>(nh[0]));
-#pragma unroll
-            for (int a = 0; a < 3; a++) hu[a] = mul_rn(cvq<HASD>(nh[1 + a]), rh);
-        }
-        if (k + 1 < k1) {
-            raw4(f, k + 2, nc);
-            if (hv) raw4(hf, k + 1, nh);
-        }
-        __syncthreads();  // readers of the previous plane are done
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            U[a][ty + 1][tx + 1] = u0[a];
-            if (hv) (&U[a][0][0])[cks(hs, HY * HX)] = hu[a];
-        }
-        __syncthreads();
-        if (active) {
-            C D[3][3];  // D[a][c]: undivided central difference of u_a along c
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                D[a][0] = U[a][ty + 1][tx + 2] - U[a][ty + 1][tx];
-                D[a][1] = U[a][ty + 2][tx + 1] - U[a][ty][tx + 1];
-                D[a][2] = up[a] - um[a];
-            }
-            stc(CKP(b + (idx)k * pl + (idx)(j * g.nx + i), b, g.n), source_b(D, alpha_s));
-            if constexpr (kInc) stc(CKP(rho_out + (idx)k * pl + (idx)(j * g.nx + i), rho_out, g.n), rho0);
-        }
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            um[a] = u0[a];
-            u0[a] = up[a];
-        }
-        rho0 = rhop;
+    for (int c = 0; c < 2; c++) {
+        const int j = t.j + c;
+        t.in[c] = t.i < g.nx && j < g.ny;
+        t.need[c] = t.i <= g.nx && j <= g.ny;
+        t.drop[c] = (t.i >= g.nx && g.bc[1] != BC_PERIODIC) || (j >= g.ny && g.bc[3] != BC_PERIODIC);
+        t.own[c] = (idx)map_axis(j, g.ny, g.bc[2], g.bc[3]) * (idx)g.nx + mi;
     }
-}
-template <bool HASD>
-__global__ void __launch_bounds__(BT) k_source(QIn q, S *__restrict__ b, S *__restrict__ rho_out, Geom g,
-                                                C alpha_s, const C *W, const C *J, int zc)
-{
-    source_body<HASD>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch());
-}
-
-
-// --------------------------------------------------------------- Jacobi
-// One sweep s_out = (b + beta sum_f c_f s_nb) / (1/rho + beta sum_f c_f),
-// c_f = (1/rho_i + 1/rho_nb)/2; a face on a non-periodic boundary carries no
-// term. 1/rho and sigma of plane k sit in a shared tile with a halo of 1;
-// the z-neighbours stay in registers.
-//
-// colour >= 0 makes it one half of a red-black Gauss-Seidel sweep, in place
-// (s_in == s_out): only the cells with (i + j + k) % 2 == colour change.
-// Their neighbours all have the other colour (periodic axes have even
-// length), which no thread writes during the launch, so every updated value
-// is the same whatever the order of execution; values read from cells of
-// the updated colour feed only results that are discarded.
-
-// One update of one cell: e[f] the face factor (beta / 2, 0 for a face on a
-// non-periodic boundary), rn[f] the reciprocal density and sn[f] Sigma of
-// the neighbour across face f, faces in the order -x, +x, -y, +y, -z, +z. A
-// fixed order of rounded operations, lane for lane that of the packed form
-// of k_jacobi_v4, so that every form of the sweep gives the same bits.
-__device__ __forceinline__ C jacobi_cell(C r0, const C (&e)[6], const C (&rn)[6], const C (&sn)[6], C bv)
-{
-    C c[6];
-#pragma unroll
-    for (int f = 0; f < 6; f++) c[f] = mul_rn(e[f], add_rn(r0, rn[f]));
-    C diag = r0;
-#pragma unroll
-    for (int f = 0; f < 6; f++) diag = add_rn(diag, c[f]);
-    C off = mul_rn(c[0], sn[0]);
-#pragma unroll
-    for (int f = 1; f < 6; f++) off = fma_rn(c[f], sn[f], off);
-    return quot(add_rn(bv, off), diag);
-}
-
-__device__ __forceinline__ void jacobi_body(const S *__restrict__ q, const S *__restrict__ b, const S *sin,
-                                            S *sout, const Geom g, C beta, int zc, int colour,
-                                            const BlockPos bp)
-{
-    __shared__ C R[HY][HX], SG[HY][HX];
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-    const int x0 = bp.x * BX, y0 = bp.y * BY;
-    const int i = x0 + tx, j = y0 + ty;
-    const bool active = i < g.nx && j < g.ny;
-    const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
-    const idx pl = (idx)g.plane;
-    const idx f = (idx)(map_axis(j, g.ny, g.bc[2], g.bc[3]) * g.nx + map_axis(i, g.nx, g.bc[0], g.bc[1]));
-    const bool hv = tid < NHALO1;
-    int hs = 0;
-    idx hf = 0;
-    if (hv) {
-        int lx, ly;
-        halo1_cell(tid, lx, ly);
-        hs = ly * HX + lx;
-        hf = (idx)(map_axis(y0 + ly - 1, g.ny, g.bc[2], g.bc[3]) * g.nx +
-                   map_axis(x0 + lx - 1, g.nx, g.bc[0], g.bc[1]));
+    int lx, ly;  // halo cell in the tile
+    if (tid < 2 * PX) {
+        lx = 1 + tx;
+        ly = ty ? PY + 1 : 0;
+    } else {
+        lx = tid - 2 * PX < PY ? 0 : PX + 1;
+        ly = 1 + (tid & (PY - 1));
     }
-    const C hb = C(0.5) * beta;
-    // a face term exists unless the face is a non-periodic domain boundary
-    const C exm = (i > 0 || g.bc[0] == BC_PERIODIC) ? hb : C(0);
-    const C exp_ = (i < g.nx - 1 || g.bc[1] == BC_PERIODIC) ? hb : C(0);
-    const C eym = (j > 0 || g.bc[2] == BC_PERIODIC) ? hb : C(0);
-    const C eyp = (j < g.ny - 1 || g.bc[3] == BC_PERIODIC) ? hb : C(0);
-    C rm, sm, r0, s0, rp, sp;
-    {
-        idx c = ck((idx)zmap(k0 - 1, g) * pl + f, g.n);
-        rm = rcp(ldc(q + c));
-        sm = ldc(sin + c);
-        c = ck((idx)k0 * pl + f, g.n);
-        r0 = rcp(ldc(q + c));
-        s0 = ldc(sin + c);
-    }
-    // raw values one iteration ahead: column at k + 1, halo and b at k
-    S ncr, ncs, nhr = S(1.0f), nhs = S(0.0f), nb;
-    auto pre = [&](int kk) {
-        idx c = ck((idx)zmap(kk + 1, g) * pl + f, g.n);
-        ncr = ldr(q + c);
-        ncs = ldr(sin + c);
-        if (hv) {
-            idx h = ck((idx)kk * pl + hf, g.n);
-            nhr = ldr(q + h);
-            nhs = ldr(sin + h);
-        }
-        nb = ldr(CKP(b + (idx)kk * pl + f, b, g.n));
-    };
-    pre(k0);
-    for (int k = k0; k < k1; k++) {
-        rp = rcp(cv(ncr));
-        sp = cv(ncs);
-        C hr = rcp(cv(nhr)), hsg = cv(nhs), bv = cv(nb);
-        if (k + 1 < k1) pre(k + 1);
-        __syncthreads();
-        R[ty + 1][tx + 1] = r0;
-        SG[ty + 1][tx + 1] = s0;
-        if (hv) {
-            (&R[0][0])[cks(hs, HY * HX)] = hr;
-            (&SG[0][0])[cks(hs, HY * HX)] = hsg;
-        }
-        __syncthreads();
-        if (active) {
-            const C ezm = (k > 0 || g.bc[4] == BC_PERIODIC) ? hb : C(0);
-            const C ezp = (k < g.nz - 1 || g.bc[5] == BC_PERIODIC) ? hb : C(0);
-            // faces in the order -x, +x, -y, +y, -z, +z
-            const C e[6] = {exm, exp_, eym, eyp, ezm, ezp};
-            const C rn[6] = {R[ty + 1][tx], R[ty + 1][tx + 2], R[ty][tx + 1], R[ty + 2][tx + 1], rm, rp};
-            const C sn[6] = {SG[ty + 1][tx], SG[ty + 1][tx + 2], SG[ty][tx + 1], SG[ty + 2][tx + 1], sm, sp};
-            if (colour < 0 || ((i + j + k) & 1) == colour)
-                stc(CKP(sout + (idx)k * pl + (idx)(j * g.nx + i), sout, g.n), jacobi_cell(r0, e, rn, sn, bv));
-        }
-        rm = r0; sm = s0;
-        r0 = rp; s0 = sp;
-    }
-}
-__global__ void __launch_bounds__(BT) k_jacobi(const S *__restrict__ q, const S *__restrict__ b,
-                                                const S *sin, S *sout, Geom g, C beta, int zc,
-                                                int colour)
-{
-    jacobi_body(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch());
+    const int x = x0 + lx - 1, y = y0 + ly - 1;
+    t.h = tid < 2 * PX + 2 * PY && x <= g.nx && y <= g.ny;
+    t.hpos = ly * PPITCH + lx;
+    t.hoff = (idx)map_axis(y, g.ny, g.bc[2], g.bc[3]) * (idx)g.nx + (idx)map_axis(x, g.nx, g.bc[0], g.bc[1]);
+    t.hdrop = (x < 0 && g.bc[0] != BC_PERIODIC) || (x >= g.nx && g.bc[1] != BC_PERIODIC) ||
+              (y < 0 && g.bc[2] != BC_PERIODIC) || (y >= g.ny && g.bc[3] != BC_PERIODIC);
+    return t;
 }
 
-
-// Vector form of the sweep for rows whose length is a multiple of 4: each
-// thread owns 4 consecutive cells of a row (one 4-wide load/store per field),
-// takes x-neighbours from its own registers, y-neighbours as aligned 4-wide
-// shared loads. Same arithmetic per cell, in the same order, as k_jacobi.
-__device__ __forceinline__ void ld4(const double *p, double v[4])
-{
-    double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
-__device__ __forceinline__ void ld4(const float *p, float v[4])
-{
-    float4 a = __ldg(reinterpret_cast<const float4 *>(p));
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-}
-__device__ __forceinline__ void ld4(const __half *p, float v[4])
-{
-    uint2 a = __ldg(reinterpret_cast<const uint2 *>(p));
-    float2 lo = __half22float2(*reinterpret_cast<const __half2 *>(&a.x));
-    float2 hi = __half22float2(*reinterpret_cast<const __half2 *>(&a.y));
-    v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
-}
-__device__ __forceinline__ void ld4(const __nv_bfloat16 *p, float v[4])
-{
-    uint2 a = __ldg(reinterpret_cast<const uint2 *>(p));
-    float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&a.x));
-    float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&a.y));
-    v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
-}
+// ------------------------------------------- 4-wide loads, stores, shared rows
 __device__ __forceinline__ void st4(double *p, const double v[4])
 {
     reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
@@ -892,7 +711,8 @@ __device__ __forceinline__ void st4(__nv_bfloat16 *p, const float v[4])
     *reinterpret_cast<uint2 *>(p) = u;
 }
 
-// four consecutive stored values kept raw after one vector load
+// Four consecutive values as loaded: they stay raw until they are used, so
+// that nothing waits on the load before then
 template <typename T> struct Vec4;
 template <> struct Vec4<double> { double2 a, b; };
 template <> struct Vec4<float> { float4 a; };
@@ -936,25 +756,6 @@ __device__ __forceinline__ void cv4(const Vec4<__nv_bfloat16> &v, float o[4])
     float2 a = __bfloat1622float2(lo.h), b = __bfloat1622float2(hi.h);
     o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
 }
-__device__ __forceinline__ Vec4<double> pack4(double a, double b, double c, double d)
-{
-    return {make_double2(a, b), make_double2(c, d)};
-}
-__device__ __forceinline__ Vec4<float> pack4(float a, float b, float c, float d) { return {make_float4(a, b, c, d)}; }
-__device__ __forceinline__ Vec4<__half> pack4(__half a, __half b, __half c, __half d)
-{
-    return {make_uint2(__half_as_ushort(a) | ((unsigned)__half_as_ushort(b) << 16),
-                       __half_as_ushort(c) | ((unsigned)__half_as_ushort(d) << 16))};
-}
-__device__ __forceinline__ Vec4<__nv_bfloat16> pack4(__nv_bfloat16 a, __nv_bfloat16 b, __nv_bfloat16 c,
-                                                      __nv_bfloat16 d)
-{
-    return {make_uint2(__bfloat16_as_ushort(a) | ((unsigned)__bfloat16_as_ushort(b) << 16),
-                       __bfloat16_as_ushort(c) | ((unsigned)__bfloat16_as_ushort(d) << 16))};
-}
-
-constexpr int VX = 4, TXV = BX * VX;        // 128 cells per tile row
-
 // 4 consecutive values of a 16-byte aligned shared row (one 128-bit access
 // for FP32, two for FP64; scalar accesses at stride 4 would conflict 4-way)
 __device__ __forceinline__ void sh_st4(float *p, const float v[4])
@@ -976,116 +777,450 @@ __device__ __forceinline__ void sh_ld4(const double *p, double v[4])
     double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
     v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
-constexpr int HXV = TXV + 2 * VX;           // interior at column VX (16-byte aligned)
-constexpr int NYH = 2 * BX, NXH = 2 * BY;   // 4-wide y-halo tasks, scalar x-halo tasks
 
-// The update of four cells (x-consecutive, of one row) as two packed FP32x2
-// pairs, cells (0, 1) and (2, 3); lane for lane the sequence of jacobi_cell
-// (faces -x, +x, -y, +y, -z, +z). r0, s0: the cells; rl, sl / rr, sr: the
-// x-neighbours left of cell 0 and right of cell 3; ry0 / ry1 (sy0 / sy1):
-// the rows below / above; rm, sm / rp, sp: the planes below / above; bv:
-// the source; hb = beta / 2 and the face factors of the four cells' outer
-// faces (the inner x-faces are always hb).
-__device__ __forceinline__ void jacobi4_packed(const float (&r0)[4], const float (&s0)[4], float rl, float sl,
-                                               float rr, float sr, const float (&ry0)[4], const float (&ry1)[4],
-                                               const float (&sy0)[4], const float (&sy1)[4], const float (&rm)[4],
-                                               const float (&sm)[4], const float (&rp)[4], const float (&sp)[4],
-                                               const float (&bv)[4], float hb, float exm, float exp_, float eym,
-                                               float eyp, float ezm, float ezp, float (&o)[4])
+// Asynchronous copies global -> shared of a quad and of a single value (at 16
+// bits the aligned pair that holds it), and reading them back
+__device__ __forceinline__ unsigned sh_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait()
 {
-    const float2 r01 = make_float2(r0[0], r0[1]), r23 = make_float2(r0[2], r0[3]), r12 = make_float2(r0[1], r0[2]);
-    const float2 s12 = make_float2(s0[1], s0[2]);
-    const float2 rxm[2] = {make_float2(rl, r0[0]), r12}, rxp[2] = {r12, make_float2(r0[3], rr)};
-    const float2 sxm[2] = {make_float2(sl, s0[0]), s12}, sxp[2] = {s12, make_float2(s0[3], sr)};
-    const float2 exmp[2] = {make_float2(exm, hb), make_float2(hb, hb)};
-    const float2 expp[2] = {make_float2(hb, hb), make_float2(hb, exp_)};
-    const float2 rc[2] = {r01, r23};
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int c = 2 * h;
-        float2 c0 = pmul(exmp[h], padd(rc[h], rxm[h]));
-        float2 c1 = pmul(expp[h], padd(rc[h], rxp[h]));
-        float2 c2 = pmul(make_float2(eym, eym), padd(rc[h], make_float2(ry0[c], ry0[c + 1])));
-        float2 c3 = pmul(make_float2(eyp, eyp), padd(rc[h], make_float2(ry1[c], ry1[c + 1])));
-        float2 c4 = pmul(make_float2(ezm, ezm), padd(rc[h], make_float2(rm[c], rm[c + 1])));
-        float2 c5 = pmul(make_float2(ezp, ezp), padd(rc[h], make_float2(rp[c], rp[c + 1])));
-        float2 diag = padd(padd(padd(padd(padd(padd(rc[h], c0), c1), c2), c3), c4), c5);
-        float2 off = pmul(c0, sxm[h]);
-        off = pfma(c1, sxp[h], off);
-        off = pfma(c2, make_float2(sy0[c], sy0[c + 1]), off);
-        off = pfma(c3, make_float2(sy1[c], sy1[c + 1]), off);
-        off = pfma(c4, make_float2(sm[c], sm[c + 1]), off);
-        off = pfma(c5, make_float2(sp[c], sp[c + 1]), off);
-        float2 num = padd(make_float2(bv[c], bv[c + 1]), off);
-        float2 res = pmul(num, make_float2(rcp(diag.x), rcp(diag.y)));
-        o[c] = res.x;
-        o[c + 1] = res.y;
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void cp_quad(unsigned dst, const S *src)
+{
+    if constexpr (sizeof(S) == 2) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
+    } else {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+        if constexpr (sizeof(S) == 8)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16), "l"(src + 2) : "memory");
     }
 }
-__device__ __forceinline__ void jacobi4_packed(const double (&)[4], const double (&)[4], double, double, double,
-                                               double, const double (&)[4], const double (&)[4],
-                                               const double (&)[4], const double (&)[4], const double (&)[4],
-                                               const double (&)[4], const double (&)[4], const double (&)[4],
-                                               const double (&)[4], double, double, double, double, double,
-                                               double, double, double (&)[4])
+__device__ __forceinline__ void cp_one(unsigned dst, const S *src)
 {
-}  // FP64 takes the scalar cells; this overload only lets the FP32 call compile in the FP64 build
-
-// 4 raw values of field a at cells (x .. x+3) of row-plane offset rowoff:
-// one 4-wide load when the cells lie inside the row, mapped single loads otherwise
-template <class T>
-__device__ __forceinline__ Vec4<T> ld4_mapped(const T *__restrict__ a, const Geom &g, idx rowoff, int x)
-{
-    if (x + VX <= g.nx) return ld4r(CKP4(a + rowoff + x, a, g.n));
-    T v[VX];
-#pragma unroll
-    for (int c = 0; c < VX; c++)
-        v[c] = __ldg(CKP(a + rowoff + (idx)map_axis(x + c, g.nx, g.bc[0], g.bc[1]), a, g.n));
-    return pack4(v[0], v[1], v[2], v[3]);
+    if constexpr (sizeof(S) == 2)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"((size_t)src & ~(size_t)3) : "memory");
+    else if constexpr (sizeof(S) == 4)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
 }
 
-// 4 raw state values (cells x .. x+3) and their stage values, as StateIO
+// --------------------------------------------------------------- Jacobi
+// One sweep s_out = (b + beta sum_f c_f s_nb) / (1/rho + beta sum_f c_f),
+// c_f = (1/rho_i + 1/rho_nb)/2; a face on a non-periodic boundary carries no
+// term. 1/rho and sigma of plane k sit in a shared tile with a halo of 1;
+// the z-neighbours stay in registers.
+//
+// The faces are summed without the common factor hb = beta / 2,
+//   C_f = 1/rho_i + 1/rho_nb, D = 1/rho_i + hb sum C_f, N = b + hb sum C_f s_nb,
+// so no factor per face is held or multiplied, and the z-face below a cell is
+// the face above the cell of the last plane, kept from there. Across a
+// dropped face the neighbour's 1/rho is taken as -1/rho_i and its Sigma as 0:
+// C_f is then exactly 0.
+//
+// colour >= 0 makes it one half of a red-black Gauss-Seidel sweep, in place
+// (s_in == s_out): only the cells with (i + j + k) % 2 == colour change.
+// Their neighbours all have the other colour (periodic axes have even
+// length), which no thread writes during the launch, so every updated value
+// is the same whatever the order of execution; values read from cells of
+// the updated colour feed only results that are discarded.
+
+// The update of two cells: rc their 1/rho, bv their source; r*, s* the
+// neighbours' 1/rho and Sigma in x and y; zm, zp the z-faces below and above,
+// sm, sp Sigma there. Packed FP32x2 operations (FP64: two scalar ones).
+__device__ __forceinline__ float2 pquot(float2 a, float2 b) { return pmul(a, make_float2(rcp(b.x), rcp(b.y))); }
+__device__ __forceinline__ double2 pquot(double2 a, double2 b)
+{
+    return make_double2(__ddiv_rn(a.x, b.x), __ddiv_rn(a.y, b.y));
+}
+__device__ __forceinline__ C2 jacobi2(C2 rc, C2 rxm, C2 rxp, C2 rym, C2 ryp, C2 zm, C2 zp, C2 sxm, C2 sxp, C2 sym,
+                                      C2 syp, C2 sm, C2 sp, C2 bv, C hb)
+{
+    const C2 c0 = padd(rc, rxm), c1 = padd(rc, rxp), c2 = padd(rc, rym), c3 = padd(rc, ryp);
+    const C2 sum = padd(padd(padd(c0, c1), padd(c2, c3)), padd(zm, zp));
+    C2 off = pmul(c0, sxm);
+    off = pfma(c1, sxp, off);
+    off = pfma(c2, sym, off);
+    off = pfma(c3, syp, off);
+    off = pfma(zm, sm, off);
+    off = pfma(zp, sp, off);
+    return pquot(pfma(bcast(hb), off, bv), pfma(bcast(hb), sum, rc));
+}
+
+// Raw values are copied to shared memory JRING - 1 planes ahead, each by the
+// thread that uses it (so no barrier guards them): a plane's time is then not
+// the latency of its loads. Register prefetch does not get there: loads of
+// several planes in flight share a warp's six scoreboards, and a wait for
+// the oldest waits for the youngest too. What bounds the 16-bit sweep next is
+// instructions and shared-memory bandwidth: Sigma is exchanged in its storage
+// type, the x-neighbours within a warp's row by shuffles, and on large grids
+// a thread has two quads, one above the other (NR = 2): addresses, loop and
+// barrier serve both, and they exchange in registers.
+constexpr int JRING = sizeof(S) == 8 ? 2 : 4;
+template <int NR> struct JShape {
+    static constexpr int TILE = NR * QUAD_TILE;                      // cells of a plane tile with its halo
+    static constexpr int HT = 96;                                    // threads that may have a halo task
+    static constexpr int PLANE = VX * (3 * NR * BT + 2 * HT);        // values of one plane of the ring
+    static constexpr int SMEM = JRING * PLANE * (int)sizeof(S) + 2 * TILE * (int)(sizeof(C) + sizeof(S));
+};
+template <bool FULL, bool RB, int NR>
+__device__ __forceinline__ void jacobi_quads(const S *__restrict__ q, const S *__restrict__ b, const S *sin, S *sout,
+                                             const Geom &g, C beta, int zc, int colour, const BlockPos &bp, int wq,
+                                             int rows, unsigned char *smem)
+{
+    static_assert(FULL || NR == 1, "two rows per thread: full tiles");
+    constexpr int JPLANE = JShape<NR>::PLANE, JTILE = JShape<NR>::TILE, HT = JShape<NR>::HT;
+    S *ring = reinterpret_cast<S *>(smem);
+    C *R2 = reinterpret_cast<C *>(ring + JRING * JPLANE);
+    S *S2 = reinterpret_cast<S *>(R2 + 2 * JTILE);
+    const Quad t = quad_of<FULL, NR>(g, bp, wq, rows);
+    const int tid = threadIdx.x;
+    const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
+    const idx pl = (idx)g.plane;
+    const C hb = C(0.5) * beta;
+    idx own[NR];
+#pragma unroll
+    for (int r = 0; r < NR; r++) own[r] = t.own + (idx)r * (idx)g.nx;
+    S *const mine = ring + VX * tid, *const minh = ring + VX * (3 * NR * BT + (tid < HT ? tid : 0));
+    constexpr int F = VX * BT, FH = VX * HT;
+    // start the copies of own density and Sigma of plane kk + 1, source and halo of plane kk
+    auto load = [&](int kk) {
+        const int at = ((kk - k0) & (JRING - 1)) * JPLANE;
+        const unsigned d = sh_addr(mine + at), dh = sh_addr(minh + at);
+        const idx pk = (idx)kk * pl, h = pk + t.hoff;
+        if (FULL || t.active) {
+            const idx pz = (idx)zmap(kk + 1, g) * pl;
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                cp_quad(d + (3 * r) * F * sizeof(S), CKP4(q + pz + own[r], q, g.n));
+                cp_quad(d + (3 * r + 1) * F * sizeof(S), CKP4(sin + pz + own[r], sin, g.n));
+                cp_quad(d + (3 * r + 2) * F * sizeof(S), CKP4(b + pk + own[r], b, g.n));
+            }
+        }
+        if (t.yh) {
+            cp_quad(dh, CKP4(q + h, q, g.n));
+            cp_quad(dh + FH * sizeof(S), CKP4(sin + h, sin, g.n));
+        } else if (t.xh) {
+            cp_one(dh, CKP(q + h, q, g.n));
+            cp_one(dh + FH * sizeof(S), CKP(sin + h, sin, g.n));
+        }
+    };
+    auto conv = [&](const V4 &v, C (&r)[VX]) {
+        cv4(v, r);
+#pragma unroll
+        for (int c = 0; c < VX; c++) r[c] = rcp(r[c]);
+    };
+    C sm[NR][VX], r0[NR][VX], s0[NR][VX];
+    V4 s0r[NR];  // s0 as stored
+    C2 zm[NR][2];
+#pragma unroll
+    for (int m = 0; m < JRING - 1; m++) {
+        if (k0 + m < k1) load(k0 + m);
+        cp_async_commit();
+    }
+    if (FULL || t.active) {
+        const idx zb = (idx)zmap(k0 - 1, g) * pl, z0 = (idx)k0 * pl;
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+            const V4 ar = ld4r(CKP4(q + zb + own[r], q, g.n));
+            const V4 as = ld4r(CKP4(sin + zb + own[r], sin, g.n));
+            const V4 or_ = ld4r(CKP4(q + z0 + own[r], q, g.n));
+            s0r[r] = ld4r(CKP4(sin + z0 + own[r], sin, g.n));
+            C rm[VX];
+            conv(ar, rm);
+            cv4(as, sm[r]);
+            conv(or_, r0[r]);
+            cv4(s0r[r], s0[r]);
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+                zm[r][h] = padd(pset(r0[r][2 * h], r0[r][2 * h + 1]), pset(rm[2 * h], rm[2 * h + 1]));
+            if (k0 == 0 && g.bc[4] != BC_PERIODIC) {
+#pragma unroll
+                for (int c = 0; c < VX; c++) sm[r][c] = C(0);
+                zm[r][0] = zm[r][1] = bcast(C(0));
+            }
+        }
+    }
+    const int hodd = sizeof(S) == 2 ? (int)(t.hoff & 1) : 0;  // the halo cell in its pair (nx is even)
+    for (int k = k0; k < k1; k++) {
+        // two plane tiles, alternating: the buffer a plane writes was last
+        // read two planes ago, before the barrier of the previous plane
+        C *R = R2 + ((k - k0) & 1) * JTILE;
+        S *SG = S2 + ((k - k0) & 1) * JTILE;
+        const int at = ((k - k0) & (JRING - 1)) * JPLANE;
+        C rp[NR][VX], sp[NR][VX], bv[NR][VX];
+        V4 spr[NR];
+        if (FULL || t.active) {
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                sh_st4(R + t.pos + r * t.pitch, r0[r]);
+                *reinterpret_cast<V4 *>(SG + t.pos + r * t.pitch) = s0r[r];
+            }
+        }
+        cp_async_wait<JRING - 2>();
+        if (t.yh) {
+            C w[VX];
+            conv(*reinterpret_cast<const V4 *>(minh + at), w);
+            if (t.hdrop) {
+#pragma unroll
+                for (int c = 0; c < VX; c++) w[c] = -w[c];
+            }
+            sh_st4(R + cks4(t.hpos, JTILE), w);
+            V4 hs = *reinterpret_cast<const V4 *>(minh + at + FH);
+            if (t.hdrop) hs = V4{};
+            *reinterpret_cast<V4 *>(SG + cks4(t.hpos, JTILE)) = hs;
+        } else if (t.xh) {
+            const C w = rcp(C(cv(minh[at + hodd])));
+            R[cks(t.hpos, JTILE)] = t.hdrop ? -w : w;
+            SG[cks(t.hpos, JTILE)] = t.hdrop ? S(0.0f) : minh[at + FH + hodd];
+        }
+        if (FULL || t.active) {
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                conv(*reinterpret_cast<const V4 *>(mine + at + (3 * r) * F), rp[r]);
+                spr[r] = *reinterpret_cast<const V4 *>(mine + at + (3 * r + 1) * F);
+                cv4(spr[r], sp[r]);
+                cv4(*reinterpret_cast<const V4 *>(mine + at + (3 * r + 2) * F), bv[r]);
+            }
+        }
+        if (k + JRING - 1 < k1) load(k + JRING - 1);
+        cp_async_commit();
+        __syncthreads();
+        if (FULL || t.active) {
+            if (k == g.nz - 1 && g.bc[5] != BC_PERIODIC) {  // no face above the last plane
+#pragma unroll
+                for (int r = 0; r < NR; r++)
+#pragma unroll
+                    for (int c = 0; c < VX; c++) {
+                        rp[r][c] = -r0[r][c];
+                        sp[r][c] = C(0);
+                    }
+            }
+            C rb[VX], ra[VX], sb[VX], sa[VX];  // rows below and above
+            sh_ld4(R + t.pos - t.pitch, rb);
+            sh_ld4(R + t.pos + NR * t.pitch, ra);
+            cv4(*reinterpret_cast<const V4 *>(SG + t.pos - t.pitch), sb);
+            cv4(*reinterpret_cast<const V4 *>(SG + t.pos + NR * t.pitch), sa);
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                const C (&ry0)[VX] = r ? r0[0] : rb, (&sy0)[VX] = r ? s0[0] : sb;
+                const C (&ry1)[VX] = r + 1 < NR ? r0[NR - 1] : ra, (&sy1)[VX] = r + 1 < NR ? s0[NR - 1] : sa;
+                const int pos = t.pos + r * t.pitch;
+                C rl, rr, sl, sr;  // x-neighbours of the quad
+                if (FULL) {        // a warp is a row: only its ends read the tile
+                    const int lane = tid & 31;
+                    rl = __shfl_up_sync(0xffffffffu, r0[r][3], 1);
+                    sl = __shfl_up_sync(0xffffffffu, s0[r][3], 1);
+                    rr = __shfl_down_sync(0xffffffffu, r0[r][0], 1);
+                    sr = __shfl_down_sync(0xffffffffu, s0[r][0], 1);
+                    if (lane == 0 || lane == 31) {
+                        const int e = lane ? pos + VX : pos - 1;
+                        const C re = R[e], se = C(cv(SG[e]));
+                        if (lane) {
+                            rr = re;
+                            sr = se;
+                        } else {
+                            rl = re;
+                            sl = se;
+                        }
+                    }
+                } else {
+                    rl = R[pos - 1];
+                    rr = R[pos + VX];
+                    sl = C(cv(SG[pos - 1]));
+                    sr = C(cv(SG[pos + VX]));
+                }
+                const C rx[VX + 2] = {rl, r0[r][0], r0[r][1], r0[r][2], r0[r][3], rr};
+                const C sx[VX + 2] = {sl, s0[r][0], s0[r][1], s0[r][2], s0[r][3], sr};
+                C o[VX];
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int c = 2 * h;
+                    const C2 rc = pset(r0[r][c], r0[r][c + 1]), zp = padd(rc, pset(rp[r][c], rp[r][c + 1]));
+                    const C2 v = jacobi2(rc, pset(rx[c], rx[c + 1]), pset(rx[c + 2], rx[c + 3]),
+                                         pset(ry0[c], ry0[c + 1]), pset(ry1[c], ry1[c + 1]), zm[r][h], zp,
+                                         pset(sx[c], sx[c + 1]), pset(sx[c + 2], sx[c + 3]),
+                                         pset(sy0[c], sy0[c + 1]), pset(sy1[c], sy1[c + 1]),
+                                         pset(sm[r][c], sm[r][c + 1]), pset(sp[r][c], sp[r][c + 1]),
+                                         pset(bv[r][c], bv[r][c + 1]), hb);
+                    o[c] = v.x;
+                    o[c + 1] = v.y;
+                    zm[r][h] = zp;
+                }
+                if (RB || (!FULL && colour >= 0)) {
+#pragma unroll
+                    for (int c = 0; c < VX; c++)
+                        if (((t.i0 + c + t.j + r + k) & 1) != colour) o[c] = s0[r][c];
+                }
+                st4(CKP4(sout + (idx)k * pl + own[r], sout, g.n), o);
+            }
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+#pragma unroll
+                for (int c = 0; c < VX; c++) {
+                    sm[r][c] = s0[r][c];
+                    r0[r][c] = rp[r][c];
+                    s0[r][c] = sp[r][c];
+                }
+                s0r[r] = spr[r];
+            }
+        }
+    }
+}
+
+// the pairs: one halo cell per thread of the first three warps, own values
+// one plane ahead
+__device__ __forceinline__ void jacobi_pairs(const S *__restrict__ q, const S *__restrict__ b, const S *sin, S *sout,
+                                             const Geom &g, C beta, int zc, int colour, const BlockPos &bp, C *R2,
+                                             C *S2)
+{
+    const Pair t = pair_of(g, bp);
+    const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
+    const idx pl = (idx)g.plane;
+    const C hb = C(0.5) * beta;
+    S nr[2] = {S(1.0f), S(1.0f)}, ns[2] = {S(0.0f), S(0.0f)}, nb[2] = {S(0.0f), S(0.0f)};
+    S xr = S(1.0f), xs = S(0.0f);
+    auto own = [&](int kk) {  // own cells of plane kk
+        const idx pz = (idx)zmap(kk, g) * pl;
+#pragma unroll
+        for (int c = 0; c < 2; c++)
+            if (t.need[c]) {
+                nr[c] = ldr(CKP(q + pz + t.own[c], q, g.n));
+                ns[c] = ldr(CKP(sin + pz + t.own[c], sin, g.n));
+            }
+    };
+    auto rest = [&](int kk) {  // source and halo of plane kk
+        const idx pk = (idx)kk * pl;
+#pragma unroll
+        for (int c = 0; c < 2; c++)
+            if (t.in[c]) nb[c] = ldr(CKP(b + pk + t.own[c], b, g.n));
+        if (t.h) {
+            xr = ldr(CKP(q + pk + t.hoff, q, g.n));
+            xs = ldr(CKP(sin + pk + t.hoff, sin, g.n));
+        }
+    };
+    // a cell past a non-periodic edge stands for the dropped face's neighbour
+    auto conv = [&](C2 &r, C2 &s) {
+        const C a = rcp(C(cv(nr[0]))), e = rcp(C(cv(nr[1])));
+        r = pset(t.drop[0] ? -a : a, t.drop[1] ? -e : e);
+        s = pset(t.drop[0] ? C(0) : C(cv(ns[0])), t.drop[1] ? C(0) : C(cv(ns[1])));
+    };
+    C2 rm, sm, r0, s0, zm;
+    own(k0 - 1);
+    conv(rm, sm);
+    own(k0);
+    conv(r0, s0);
+    own(k0 + 1);
+    rest(k0);
+    zm = padd(r0, rm);
+    if (k0 == 0 && g.bc[4] != BC_PERIODIC) zm = sm = bcast(C(0));
+    for (int k = k0; k < k1; k++) {
+        C *R = R2 + ((k - k0) & 1) * TILEP, *SG = S2 + ((k - k0) & 1) * TILEP;
+        C2 rp, sp;
+        R[t.pos] = r0.x;
+        R[t.pos + PPITCH] = r0.y;
+        SG[t.pos] = s0.x;
+        SG[t.pos + PPITCH] = s0.y;
+        if (t.h) {
+            const C w = rcp(C(cv(xr)));
+            R[cks(t.hpos, TILEP)] = t.hdrop ? -w : w;
+            SG[cks(t.hpos, TILEP)] = t.hdrop ? C(0) : C(cv(xs));
+        }
+        conv(rp, sp);
+        const C2 bv = pset(C(cv(nb[0])), C(cv(nb[1])));
+        if (k + 1 < k1) {
+            own(k + 2);
+            rest(k + 1);
+        }
+        __syncthreads();
+        if (k == g.nz - 1 && g.bc[5] != BC_PERIODIC) {  // no face above the last plane
+            rp = pset(-r0.x, -r0.y);
+            sp = bcast(C(0));
+        }
+        const C2 zp = padd(r0, rp);
+        const C *Rc = R + t.pos, *Sc = SG + t.pos;
+        const C2 v = jacobi2(r0, pset(Rc[-1], Rc[PPITCH - 1]), pset(Rc[1], Rc[PPITCH + 1]),
+                             pset(Rc[-PPITCH], r0.x), pset(r0.y, Rc[2 * PPITCH]), zm, zp,
+                             pset(Sc[-1], Sc[PPITCH - 1]), pset(Sc[1], Sc[PPITCH + 1]),
+                             pset(Sc[-PPITCH], s0.x), pset(s0.y, Sc[2 * PPITCH]), sm, sp, bv, hb);
+        const int odd = (t.i + t.j + k) & 1;
+        S *o = sout + (idx)k * pl;
+        if (t.in[0] && (colour < 0 || odd == colour)) stc(CKP(o + t.own[0], sout, g.n), v.x);
+        if (t.in[1] && (colour < 0 || odd != colour)) stc(CKP(o + t.own[1], sout, g.n), v.y);
+        zm = zp;
+        sm = s0;
+        r0 = rp;
+        s0 = sp;
+    }
+}
+// resident blocks per SM that the registers are held to
+template <int NR> constexpr int kJacobiBlocks = sizeof(S) == 8 ? 1 : sizeof(S) == 2 && NR == 1 ? 3 : 2;
+constexpr int JACOBI_FIT_BLOCKS = sizeof(C) == 8 ? 1 : 2;
+constexpr int JACOBI_PAIR_BLOCKS = sizeof(C) == 8 ? 2 : 4;
+template <bool RB, int NR>
+__global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full(const S *__restrict__ q, const S *__restrict__ b,
+                                                                  const S *sin, S *sout, Geom g, C beta, int zc,
+                                                                  int colour)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    jacobi_quads<true, RB, NR>(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), FQ, FR, smem_raw);
+}
+__global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit(const S *__restrict__ q, const S *__restrict__ b,
+                                                                     const S *sin, S *sout, Geom g, C beta, int zc,
+                                                                     int colour, int wq, int rows)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    jacobi_quads<false, false, 1>(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), wq, rows, smem_raw);
+}
+__global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS) k_jacobi_pairs(const S *__restrict__ q,
+                                                                        const S *__restrict__ b, const S *sin,
+                                                                        S *sout, Geom g, C beta, int zc, int colour)
+{
+    __shared__ C R[2 * TILEP];
+    __shared__ C SG[2 * TILEP];
+    jacobi_pairs(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), R, SG);
+}
+
+// --------------------------------------------------------------- source
+// b = alpha [tr(G^2) + tr(G)^2] (Eq. igrelliptic) from the undivided central
+// differences D = 2 dx G of u, with alpha_s = alpha / (2 dx)^2:
+//   b = alpha_s [sum_ab D_ab D_ba + (sum_a D_aa)^2],
+// in one fixed order of rounded operations
+__device__ __forceinline__ C source_b(const C (&D)[3][3], C alpha_s)
+{
+    const C tr = add_rn(add_rn(D[0][0], D[1][1]), D[2][2]);
+    C sq = mul_rn(D[0][0], D[0][0]);
+    sq = fma_rn(D[1][1], D[1][1], sq);
+    sq = fma_rn(D[2][2], D[2][2], sq);
+    C x = mul_rn(D[0][1], D[1][0]);
+    x = fma_rn(D[0][2], D[2][0], x);
+    x = fma_rn(D[1][2], D[2][1], x);
+    const C tr2 = fma_rn(C(2), x, sq);  // sum_ab D_ab D_ba
+    return mul_rn(alpha_s, fma_rn(tr, tr, tr2));
+}
+
+// Four raw state values and their stage values, as StateIO
 struct QRaw4Inc {
     Vec4<QB> b;
     V4 d;
 };
-template <bool INC> struct StateIO4;
-template <> struct StateIO4<false> {  // (used where the state has the storage type)
-    using Raw = V4;
-    template <bool HASD>
-    static __device__ __forceinline__ V4 ld(const QIn &q, int u, const Geom &g, idx rowoff, int x)
-    {
-        return ld4_mapped(reinterpret_cast<const S *>(q.b[u]), g, rowoff, x);
-    }
-    template <bool HASD> static __device__ __forceinline__ void val(const V4 &r, C o[4]) { cv4(r, o); }
-    // cells off .. off+3 inside one row: one 4-wide load
-    template <bool HASD>
-    static __device__ __forceinline__ V4 ldd(const QIn &q, int u, const Geom &g, idx off)
-    {
-        const S *f = reinterpret_cast<const S *>(q.b[u]);
-        return ld4r(CKP4(f + off, f, g.n));
-    }
-};
-template <> struct StateIO4<true> {
-    using Raw = QRaw4Inc;
-    template <bool HASD>
-    static __device__ __forceinline__ QRaw4Inc ld(const QIn &q, int u, const Geom &g, idx rowoff, int x)
-    {
-        QRaw4Inc r;
-        r.b = ld4_mapped(q.b[0] + u * q.fs, g, rowoff, x);
-        if constexpr (HASD) r.d = ld4_mapped(q.d[0] + u * q.fs, g, rowoff, x);
-        return r;
-    }
-    template <bool HASD>
-    static __device__ __forceinline__ QRaw4Inc ldd(const QIn &q, int u, const Geom &g, idx off)
-    {
-        QRaw4Inc r;
+using QRaw4 = std::conditional<kInc, QRaw4Inc, V4>::type;
+template <bool HASD, class R = QRaw4> __device__ __forceinline__ R ldq4(const QIn &q, int u, const Geom &g, idx off)
+{
+    if constexpr (std::is_same<R, QRaw4Inc>::value) {
+        R r;
         r.b = ld4r(CKP4(q.b[0] + u * q.fs + off, q.b[0], 5 * g.n));
         if constexpr (HASD) r.d = ld4r(CKP4(q.d[0] + u * q.fs + off, q.d[0], 5 * g.n));
         return r;
+    } else {
+        const S *f = reinterpret_cast<const S *>(q.b[u]);
+        return ld4r(CKP4(f + off, f, g.n));
     }
-    template <bool HASD> static __device__ __forceinline__ void val(const QRaw4Inc &r, C o[4])
-    {
+}
+template <bool HASD, class R> __device__ __forceinline__ void cvq4(const R &r, C o[4])
+{
+    if constexpr (std::is_same<R, QRaw4Inc>::value) {
         cv4(r.b, o);
         if constexpr (HASD) {
             C d[4];
@@ -1093,360 +1228,27 @@ template <> struct StateIO4<true> {
 #pragma unroll
             for (int c = 0; c < 4; c++) o[c] = C(__fadd_rn(float(o[c]), float(d[c])));
         }
+    } else {
+        cv4(r, o);
     }
-};
-using QRaw4 = StateIO4<kInc>::Raw;
-template <bool HASD>
-__device__ __forceinline__ QRaw4 ldq4(const QIn &q, int u, const Geom &g, idx rowoff, int x)
-{
-    return StateIO4<kInc>::ld<HASD>(q, u, g, rowoff, x);
-}
-template <bool HASD> __device__ __forceinline__ void cvq4(const QRaw4 &r, C o[4])
-{
-    StateIO4<kInc>::val<HASD>(r, o);
 }
 
-// The four-cell sweep of any block (tiles that cross the grid's edge in x
-// or y: lanes past the row's end, rows past the last, mapped loads).
-__device__ __forceinline__ void jacobi_v4_edge(const S *__restrict__ q, const S *__restrict__ b, const S *sin,
-                                               S *sout, const Geom &g, C beta, int zc, int colour,
-                                               const BlockPos &bp, C (*R)[HXV], C (*SG)[HXV])
+// grad u by central differences: u of plane k in a shared tile (x and y
+// neighbours), the planes below and above in registers. In the increment
+// modes the kernel also stores the stage's density rounded to the storage
+// type (rho_out), which the sweeps of the stage read. 16-bit storage
+// alternates two plane tiles (one barrier per plane); the others keep one.
+constexpr int SOURCE_BUFS = sizeof(S) == 2 ? 2 : 1;
+template <bool HASD, bool FULL>
+__device__ __forceinline__ void source_quads(const QIn q, S *__restrict__ b, S *__restrict__ rho_out, const Geom &g,
+                                            C alpha_s, const C *W, const C *J, int zc, const BlockPos &bp, int wq,
+                                            int rows, C *U2)
 {
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-    const int x0 = bp.x * TXV, y0 = bp.y * BY;
-    const int i0 = x0 + VX * tx, j = y0 + ty;
-    const bool active = i0 < g.nx && j < g.ny;
+    const Quad t = quad_of<FULL, 1>(g, bp, wq, rows);
     const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
     const idx pl = (idx)g.plane;
-    const idx rowj = (idx)(map_axis(j, g.ny, g.bc[2], g.bc[3]) * g.nx);
-    // halo tasks: 4-wide cells of the rows above/below the tile, then single
-    // cells left/right of each row
-    int htask = tid < NYH ? 0 : (tid < NYH + NXH ? 1 : 2);
-    int hsy = 0, hsx = 0, hx = 0;
-    idx hrow = 0;
-    if (htask == 0) {
-        int side = tid / BX, t = tid % BX;
-        hsy = side ? HY - 1 : 0;
-        hsx = VX + VX * t;
-        hx = x0 + VX * t;
-        hrow = (idx)(map_axis(y0 + (side ? BY : -1), g.ny, g.bc[2], g.bc[3]) * g.nx);
-    } else if (htask == 1) {
-        int e = tid - NYH, side = e / BY, r = e % BY;
-        hsy = 1 + r;
-        hsx = side ? VX + TXV : VX - 1;
-        hx = map_axis(side ? x0 + TXV : x0 - 1, g.nx, g.bc[0], g.bc[1]);
-        hrow = (idx)(map_axis(y0 + r, g.ny, g.bc[2], g.bc[3]) * g.nx);
-    }
-    const C hb = C(0.5) * beta;
-    const C exm = (i0 > 0 || g.bc[0] == BC_PERIODIC) ? hb : C(0);
-    const C exp_ = (i0 + VX - 1 < g.nx - 1 || g.bc[1] == BC_PERIODIC) ? hb : C(0);
-    const C eym = (j > 0 || g.bc[2] == BC_PERIODIC) ? hb : C(0);
-    const C eyp = (j < g.ny - 1 || g.bc[3] == BC_PERIODIC) ? hb : C(0);
-
-    C rm[VX], sm[VX], r0[VX], s0[VX], rp[VX], sp[VX];
-    {
-        C t[VX];
-        cv4(ld4_mapped(q, g, (idx)zmap(k0 - 1, g) * pl + rowj, i0), t);
-        cv4(ld4_mapped(sin, g, (idx)zmap(k0 - 1, g) * pl + rowj, i0), sm);
-#pragma unroll
-        for (int c = 0; c < VX; c++) rm[c] = rcp(t[c]);
-        cv4(ld4_mapped(q, g, (idx)k0 * pl + rowj, i0), t);
-        cv4(ld4_mapped(sin, g, (idx)k0 * pl + rowj, i0), s0);
-#pragma unroll
-        for (int c = 0; c < VX; c++) r0[c] = rcp(t[c]);
-    }
-    // raw values one iteration ahead: own cells at k + 1, halo and b at k
-    V4 ncr, ncs, nb, nhr, nhs;
-    S nxr = S(1.0f), nxs = S(0.0f);
-    auto pre = [&](int kk) {
-        idx pz = (idx)zmap(kk + 1, g) * pl + rowj;
-        ncr = ld4_mapped(q, g, pz, i0);
-        ncs = ld4_mapped(sin, g, pz, i0);
-        if (active) nb = ld4r(CKP4(b + (idx)kk * pl + rowj + (idx)i0, b, g.n));
-        if (htask == 0) {
-            nhr = ld4_mapped(q, g, (idx)kk * pl + hrow, hx);
-            nhs = ld4_mapped(sin, g, (idx)kk * pl + hrow, hx);
-        } else if (htask == 1) {
-            nxr = ldr(CKP(q + (idx)kk * pl + hrow + hx, q, g.n));
-            nxs = ldr(CKP(sin + (idx)kk * pl + hrow + hx, sin, g.n));
-        }
-    };
-    pre(k0);
-    for (int k = k0; k < k1; k++) {
-        C bv[VX], hr[VX], hsg[VX], t[VX];
-        cv4(ncr, t);
-        cv4(ncs, sp);
-#pragma unroll
-        for (int c = 0; c < VX; c++) rp[c] = rcp(t[c]);
-        if (active) cv4(nb, bv);
-        if (htask == 0) {
-            cv4(nhr, t);
-            cv4(nhs, hsg);
-#pragma unroll
-            for (int c = 0; c < VX; c++) hr[c] = rcp(t[c]);
-        } else if (htask == 1) {
-            hr[0] = rcp(cv(nxr));
-            hsg[0] = cv(nxs);
-        }
-        if (k + 1 < k1) pre(k + 1);
-        __syncthreads();
-        sh_st4(&R[ty + 1][VX + VX * tx], r0);
-        sh_st4(&SG[ty + 1][VX + VX * tx], s0);
-        if (htask == 0) {
-            sh_st4(&R[cks(hsy, HY)][cks4(hsx, HXV)], hr);
-            sh_st4(&SG[cks(hsy, HY)][cks4(hsx, HXV)], hsg);
-        } else if (htask == 1) {
-            R[cks(hsy, HY)][cks(hsx, HXV)] = hr[0];
-            SG[cks(hsy, HY)][cks(hsx, HXV)] = hsg[0];
-        }
-        __syncthreads();
-        if (active) {
-            const C ezm = (k > 0 || g.bc[4] == BC_PERIODIC) ? hb : C(0);
-            const C ezp = (k < g.nz - 1 || g.bc[5] == BC_PERIODIC) ? hb : C(0);
-            const int col = VX + VX * tx;
-            C ry0[VX], ry1[VX], sy0[VX], sy1[VX], o[VX];
-            sh_ld4(&R[ty][col], ry0);
-            sh_ld4(&R[ty + 2][col], ry1);
-            sh_ld4(&SG[ty][col], sy0);
-            sh_ld4(&SG[ty + 2][col], sy1);
-            if constexpr (sizeof(C) == 4) {
-                jacobi4_packed(r0, s0, R[ty + 1][col - 1], SG[ty + 1][col - 1], R[ty + 1][col + VX],
-                               SG[ty + 1][col + VX], ry0, ry1, sy0, sy1, rm, sm, rp, sp, bv, hb, exm, exp_, eym,
-                               eyp, ezm, ezp, o);
-#pragma unroll
-                for (int c = 0; c < VX; c++)
-                    if (colour >= 0 && ((i0 + c + j + k) & 1) != colour) o[c] = s0[c];
-            } else {
-#pragma unroll
-                for (int c = 0; c < VX; c++) {
-                    C rxm = c > 0 ? r0[c - 1] : R[ty + 1][col - 1];
-                    C sxm = c > 0 ? s0[c - 1] : SG[ty + 1][col - 1];
-                    C rxp = c < VX - 1 ? r0[c + 1] : R[ty + 1][col + VX];
-                    C sxp = c < VX - 1 ? s0[c + 1] : SG[ty + 1][col + VX];
-                    // faces in the order -x, +x, -y, +y, -z, +z
-                    const C e[6] = {c > 0 ? hb : exm, c < VX - 1 ? hb : exp_, eym, eyp, ezm, ezp};
-                    const C rn[6] = {rxm, rxp, ry0[c], ry1[c], rm[c], rp[c]};
-                    const C sn[6] = {sxm, sxp, sy0[c], sy1[c], sm[c], sp[c]};
-                    o[c] = jacobi_cell(r0[c], e, rn, sn, bv[c]);
-                    // red-black half-sweep: cells of the other colour keep (and
-                    // write back) the value read at the start of the launch
-                    if (colour >= 0 && ((i0 + c + j + k) & 1) != colour) o[c] = s0[c];
-                }
-            }
-            st4(CKP4(sout + (idx)k * pl + (idx)(j * g.nx + i0), sout, g.n), o);
-        }
-#pragma unroll
-        for (int c = 0; c < VX; c++) {
-            rm[c] = r0[c]; sm[c] = s0[c];
-            r0[c] = rp[c]; s0[c] = sp[c];
-        }
-    }
-}
-// The four-cell sweep of a block whose tile lies inside the grid in x and y
-// (FP32 arithmetic): every lane owns four cells of a row, its loads are
-// whole 4-wide rows, and the halo offsets are mapped once. Warps 0 and 1
-// load the rows below and above the tile, lanes 0..15 of warp 2 the cells
-// left and right of its rows. The plane tile is double buffered, so a plane
-// needs one barrier. The update is jacobi4_packed, as in jacobi_v4_edge, so
-// both give the same bits. RB: a red-black half-sweep of the given colour
-// (cells of the other colour keep and write back Sigma).
-template <bool RB>
-__device__ __forceinline__ void jacobi_v4_full(const S *__restrict__ q, const S *__restrict__ b, const S *sin,
-                                               S *sout, const Geom &g, C beta, int zc, int colour,
-                                               const BlockPos &bp, C (*R2)[HY][HXV], C (*SG2)[HY][HXV])
-{
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int x0 = bp.x * TXV, y0 = bp.y * BY;
-    const int i0 = x0 + VX * tx, j = y0 + ty;
-    const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
-    const idx pl = (idx)g.plane;
-    const idx own = (idx)j * (idx)g.nx + (idx)i0;
-    // halo: warp 0 the row below the tile, warp 1 the row above (4-wide),
-    // warp 2 lanes 0..7 the cells left of rows 0..7, lanes 8..15 right
-    const bool yh = ty < 2, xh = ty == 2 && tx < 2 * BY;
-    int hsy = 0, hsx = 0;
-    idx hoff = 0;
-    if (yh) {
-        hsy = ty ? HY - 1 : 0;
-        hsx = VX + VX * tx;
-        hoff = (idx)map_axis(y0 + (ty ? BY : -1), g.ny, g.bc[2], g.bc[3]) * (idx)g.nx + (idx)i0;
-    } else if (xh) {
-        const int side = tx / BY, r = tx % BY;
-        hsy = 1 + r;
-        hsx = side ? VX + TXV : VX - 1;
-        hoff = (idx)(y0 + r) * (idx)g.nx + (idx)map_axis(side ? x0 + TXV : x0 - 1, g.nx, g.bc[0], g.bc[1]);
-    }
-    const C hb = C(0.5) * beta;
-    const C exm = (i0 > 0 || g.bc[0] == BC_PERIODIC) ? hb : C(0);
-    const C exp_ = (i0 + VX - 1 < g.nx - 1 || g.bc[1] == BC_PERIODIC) ? hb : C(0);
-    const C eym = (j > 0 || g.bc[2] == BC_PERIODIC) ? hb : C(0);
-    const C eyp = (j < g.ny - 1 || g.bc[3] == BC_PERIODIC) ? hb : C(0);
-
-    C rm[VX], sm[VX], r0[VX], s0[VX], rp[VX], sp[VX];
-    {
-        C t[VX];
-        const idx zm = (idx)zmap(k0 - 1, g) * pl + own, z0 = (idx)k0 * pl + own;
-        cv4(ld4r(CKP4(q + zm, q, g.n)), t);
-        cv4(ld4r(CKP4(sin + zm, sin, g.n)), sm);
-#pragma unroll
-        for (int c = 0; c < VX; c++) rm[c] = rcp(t[c]);
-        cv4(ld4r(CKP4(q + z0, q, g.n)), t);
-        cv4(ld4r(CKP4(sin + z0, sin, g.n)), s0);
-#pragma unroll
-        for (int c = 0; c < VX; c++) r0[c] = rcp(t[c]);
-    }
-    // raw values one iteration ahead: own cells at k + 1, halo and b at k
-    V4 ncr, ncs, nb, nhr, nhs;
-    S nxr = S(1.0f), nxs = S(0.0f);
-    auto pre = [&](int kk) {
-        const idx pz = (idx)zmap(kk + 1, g) * pl + own, pk = (idx)kk * pl;
-        ncr = ld4r(CKP4(q + pz, q, g.n));
-        ncs = ld4r(CKP4(sin + pz, sin, g.n));
-        nb = ld4r(CKP4(b + pk + own, b, g.n));
-        if (yh) {
-            nhr = ld4r(CKP4(q + pk + hoff, q, g.n));
-            nhs = ld4r(CKP4(sin + pk + hoff, sin, g.n));
-        } else if (xh) {
-            nxr = ldr(CKP(q + pk + hoff, q, g.n));
-            nxs = ldr(CKP(sin + pk + hoff, sin, g.n));
-        }
-    };
-    pre(k0);
-    const int col = VX + VX * tx;
-    for (int k = k0; k < k1; k++) {
-        C bv[VX], t[VX];
-        // two tile buffers, planes alternating: the buffer written here was
-        // last read two planes ago, before the barrier of the previous plane
-        C (*R)[HXV] = R2[(k - k0) & 1], (*SG)[HXV] = SG2[(k - k0) & 1];
-        sh_st4(&R[ty + 1][col], r0);
-        sh_st4(&SG[ty + 1][col], s0);
-        if (yh) {
-            C hr[VX], hsg[VX];
-            cv4(nhr, t);
-            cv4(nhs, hsg);
-#pragma unroll
-            for (int c = 0; c < VX; c++) hr[c] = rcp(t[c]);
-            sh_st4(&R[cks(hsy, HY)][cks4(hsx, HXV)], hr);
-            sh_st4(&SG[cks(hsy, HY)][cks4(hsx, HXV)], hsg);
-        } else if (xh) {
-            R[cks(hsy, HY)][cks(hsx, HXV)] = rcp(cv(nxr));
-            SG[cks(hsy, HY)][cks(hsx, HXV)] = cv(nxs);
-        }
-        cv4(ncr, t);
-        cv4(ncs, sp);
-#pragma unroll
-        for (int c = 0; c < VX; c++) rp[c] = rcp(t[c]);
-        cv4(nb, bv);
-        if (k + 1 < k1) pre(k + 1);
-        __syncthreads();
-        const C ezm = (k > 0 || g.bc[4] == BC_PERIODIC) ? hb : C(0);
-        const C ezp = (k < g.nz - 1 || g.bc[5] == BC_PERIODIC) ? hb : C(0);
-        C ry0[VX], ry1[VX], sy0[VX], sy1[VX], o[VX];
-        sh_ld4(&R[ty][col], ry0);
-        sh_ld4(&R[ty + 2][col], ry1);
-        sh_ld4(&SG[ty][col], sy0);
-        sh_ld4(&SG[ty + 2][col], sy1);
-        jacobi4_packed(r0, s0, R[ty + 1][col - 1], SG[ty + 1][col - 1], R[ty + 1][col + VX], SG[ty + 1][col + VX],
-                       ry0, ry1, sy0, sy1, rm, sm, rp, sp, bv, hb, exm, exp_, eym, eyp, ezm, ezp, o);
-        if constexpr (RB) {
-#pragma unroll
-            for (int c = 0; c < VX; c++)
-                if (((i0 + c + j + k) & 1) != colour) o[c] = s0[c];
-        }
-        st4(CKP4(sout + (idx)k * pl + own, sout, g.n), o);
-#pragma unroll
-        for (int c = 0; c < VX; c++) {
-            rm[c] = r0[c]; sm[c] = s0[c];
-            r0[c] = rp[c]; s0[c] = sp[c];
-        }
-    }
-}
-
-__device__ __forceinline__ void jacobi_v4_body(const S *__restrict__ q, const S *__restrict__ b, const S *sin,
-                                               S *sout, const Geom g, C beta, int zc, int colour,
-                                               const BlockPos bp)
-{
-    __shared__ __align__(16) C R[2][HY][HXV];
-    __shared__ __align__(16) C SG[2][HY][HXV];
-    if constexpr (sizeof(C) == 4) {
-        if (bp.x * TXV + TXV <= g.nx && bp.y * BY + BY <= g.ny) {  // block-uniform
-            if (colour < 0)
-                jacobi_v4_full<false>(q, b, sin, sout, g, beta, zc, colour, bp, R, SG);
-            else
-                jacobi_v4_full<true>(q, b, sin, sout, g, beta, zc, colour, bp, R, SG);
-            return;
-        }
-    }
-    jacobi_v4_edge(q, b, sin, sout, g, beta, zc, colour, bp, R[0], SG[0]);
-}
-constexpr int JACOBI_V4_BLOCKS = sizeof(S) == 2 ? 3 : sizeof(S) == 4 ? 2 : 1;  // resident per SM
-__global__ void __launch_bounds__(BT, JACOBI_V4_BLOCKS) k_jacobi_v4(const S *__restrict__ q, const S *__restrict__ b,
-                                                                  const S *sin, S *sout, Geom g, C beta, int zc,
-                                                                  int colour)
-{
-    jacobi_v4_body(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch());
-}
-// Grids whose every 4-cell tile lies inside (rows a multiple of 128 cells,
-// a multiple of 8 rows; FP32 arithmetic) launch the full-tile body alone:
-// without the edge body in the same kernel it keeps its values in registers
-// (the combined kernel spills).
-template <bool RB>
-__global__ void __launch_bounds__(BT, JACOBI_V4_BLOCKS) k_jacobi_v4_full(const S *__restrict__ q,
-                                                                       const S *__restrict__ b, const S *sin,
-                                                                       S *sout, Geom g, C beta, int zc, int colour)
-{
-    if constexpr (sizeof(C) == 4) {
-        __shared__ __align__(16) C R[2][HY][HXV];
-        __shared__ __align__(16) C SG[2][HY][HXV];
-        jacobi_v4_full<RB>(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), R, SG);
-    }
-}
-
-
-// Vector form of the source for rows whose length is a multiple of 4, laid
-// out like k_jacobi_v4: each thread owns 4 consecutive cells of a row (one
-// 4-wide load per field), u of plane k sits in a shared tile with a halo of 1
-// (4-wide aligned rows), x-neighbours come from the thread's own registers
-// and z-neighbours from its register queue. The central differences are
-// taken undivided and 1/(2 dx)^2 is folded into alpha:
-//   b = (alpha / (4 dx^2)) [sum_ab D_ab D_ba + (sum_a D_aa)^2],
-//   D_ab = u_a(i + e_b) - u_a(i - e_b),
-// which is Eq. igrelliptic's left side with G = D / (2 dx). k_source takes the
-// same differences and source_b, so both forms give the same bits.
-template <bool HASD>
-__device__ __forceinline__ void source_v4_body(const QIn q, S *__restrict__ b, S *__restrict__ rho_out,
-                                               const Geom g, C alpha_s, const C *W, const C *J, int zc,
-                                               const BlockPos bp)
-{
-    __shared__ __align__(16) C U[3][HY][HXV];
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-    const int x0 = bp.x * TXV, y0 = bp.y * BY;
-    const int i0 = x0 + VX * tx, j = y0 + ty;
-    const bool active = i0 < g.nx && j < g.ny;
-    const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
-    const idx pl = (idx)g.plane;
-    const idx rowj = (idx)(map_axis(j, g.ny, g.bc[2], g.bc[3]) * g.nx);
-    // halo tasks: 4-wide cells of the rows above/below the tile, then single
-    // cells left/right of each row
-    int htask = tid < NYH ? 0 : (tid < NYH + NXH ? 1 : 2);
-    int hsy = 0, hsx = 0, hx = 0;
-    idx hrow = 0;
-    if (htask == 0) {
-        int side = tid / BX, t = tid % BX;
-        hsy = side ? HY - 1 : 0;
-        hsx = VX + VX * t;
-        hx = x0 + VX * t;
-        hrow = (idx)(map_axis(y0 + (side ? BY : -1), g.ny, g.bc[2], g.bc[3]) * g.nx);
-    } else if (htask == 1) {
-        int e = tid - NYH, side = e / BY, r = e % BY;
-        hsy = 1 + r;
-        hsx = side ? VX + TXV : VX - 1;
-        hx = map_axis(side ? x0 + TXV : x0 - 1, g.nx, g.bc[0], g.bc[1]);
-        hrow = (idx)(map_axis(y0 + r, g.ny, g.bc[2], g.bc[3]) * g.nx);
-    }
-
-    // u = m / rho of 4 cells from raw values (products rounded before they
-    // are differenced: equal neighbours give an exact 0)
+    // u = m / rho from raw values (products rounded before they are
+    // differenced: equal neighbours give an exact 0)
     auto u4 = [&](const QRaw4 (&r)[4], C u[3][VX], C rho[VX]) {
         C m[VX], rr[VX];
         cvq4<HASD>(r[0], rho);
@@ -1459,36 +1261,38 @@ __device__ __forceinline__ void source_v4_body(const QIn q, S *__restrict__ b, S
             for (int c = 0; c < VX; c++) u[a][c] = mul_rn(m[c], rr[c]);
         }
     };
-    // u of the own 4 cells of plane kk (the jet blend below an inflow face);
+    // u of the own cells of plane kk (the jet blend below an inflow face);
     // rho gets their (unblended) densities
     auto own_u = [&](int kk, C u[3][VX], C rho[VX]) {
-        idx zb = (idx)zmap(kk, g) * pl + rowj;
+        const idx zb = (idx)zmap(kk, g) * pl + t.own;
         C v[4][VX];
 #pragma unroll
-        for (int f = 0; f < 4; f++) cvq4<HASD>(ldq4<HASD>(q, f, g, zb, i0), v[f]);
+        for (int f = 0; f < 4; f++) cvq4<HASD>(ldq4<HASD>(q, f, g, zb), v[f]);
 #pragma unroll
         for (int c = 0; c < VX; c++) rho[c] = v[0][c];
         if (kk < 0 && g.bc[4] == BC_INFLOW) {
 #pragma unroll
             for (int c = 0; c < VX; c++) {
-                idx fc = ck(rowj + (idx)map_axis(i0 + c, g.nx, g.bc[0], g.bc[1]), g.plane);
-                C w = C(1) - W[fc];
+                const idx fc = ck(t.own + (idx)c, g.plane);
+                const C w = C(1) - W[fc];
 #pragma unroll
                 for (int f = 0; f < 4; f++) v[f][c] = fma_rn(w, v[f][c], J[(idx)f * pl + fc]);
             }
         }
 #pragma unroll
         for (int c = 0; c < VX; c++) {
-            C r = rcp(v[0][c]);
+            const C r = rcp(v[0][c]);
 #pragma unroll
             for (int a = 0; a < 3; a++) u[a][c] = mul_rn(v[1 + a][c], r);
         }
     };
     C um[3][VX], u0[3][VX], up[3][VX];
     C rho0[VX], rhop[VX];  // densities of the own cells at k and k + 1
-    own_u(k0 - 1, um, rhop);
-    own_u(k0, u0, rho0);
-    // raw values one iteration ahead: own cells at k + 1, halo at k (planes >= 0).
+    if (FULL || t.active) {
+        own_u(k0 - 1, um, rhop);
+        own_u(k0, u0, rho0);
+    }
+    // raw values one plane ahead: own cells at k + 1, halo at k (planes >= 0).
     // The increment modes' stages 2 and 3 (base and increments, 6 registers
     // per field and 4 cells) load the halo when it is used instead, which
     // keeps the registers under two blocks per SM with fewer spills.
@@ -1496,236 +1300,180 @@ __device__ __forceinline__ void source_v4_body(const QIn q, S *__restrict__ b, S
     QRaw4 nc[4], nh[4];
     QRaw nxh[4];
     auto halo = [&](int kk) {
-        if (htask == 0) {
+        if (t.yh) {
 #pragma unroll
-            for (int f = 0; f < 4; f++) nh[f] = ldq4<HASD>(q, f, g, (idx)kk * pl + hrow, hx);
-        } else if (htask == 1) {
+            for (int f = 0; f < 4; f++) nh[f] = ldq4<HASD>(q, f, g, (idx)kk * pl + t.hoff);
+        } else if (t.xh) {
 #pragma unroll
-            for (int f = 0; f < 4; f++) nxh[f] = ldqr<HASD>(q, f, ck((idx)kk * pl + hrow + hx, g.n));
+            for (int f = 0; f < 4; f++) nxh[f] = ldqr<HASD>(q, f, ck((idx)kk * pl + t.hoff, g.n));
         }
     };
     auto pre = [&](int kk) {
-        idx pz = (idx)zmap(kk + 1, g) * pl + rowj;
+        if (FULL || t.active) {
+            const idx pz = (idx)zmap(kk + 1, g) * pl + t.own;
 #pragma unroll
-        for (int f = 0; f < 4; f++) nc[f] = ldq4<HASD>(q, f, g, pz, i0);
+            for (int f = 0; f < 4; f++) nc[f] = ldq4<HASD>(q, f, g, pz);
+        }
         if (kHaloAhead) halo(kk);
     };
     pre(k0);
     for (int k = k0; k < k1; k++) {
         if (!kHaloAhead) halo(k);
-        u4(nc, up, rhop);
-        C hu[3][VX];
-        if (htask == 0) {
-            C hrho[VX];
+        // two buffers: the one written here was last read two planes ago,
+        // before the barrier of the previous plane
+        C *U = U2 + (SOURCE_BUFS == 2 ? ((k - k0) & 1) * 3 * TILEV : 0);
+        if (SOURCE_BUFS == 1) __syncthreads();  // readers of the previous plane are done
+        if (FULL || t.active) {
+#pragma unroll
+            for (int a = 0; a < 3; a++) sh_st4(U + a * TILEV + t.pos, u0[a]);
+        }
+        if (t.yh) {
+            C hu[3][VX], hrho[VX];
             u4(nh, hu, hrho);
-        } else if (htask == 1) {
-            C r = rcp(cvq<HASD>(nxh[0]));
 #pragma unroll
-            for (int a = 0; a < 3; a++) hu[a][0] = mul_rn(cvq<HASD>(nxh[1 + a]), r);
+            for (int a = 0; a < 3; a++) sh_st4(U + a * TILEV + cks4(t.hpos, TILEV), hu[a]);
+        } else if (t.xh) {
+            const C r = rcp(cvq<HASD>(nxh[0]));
+#pragma unroll
+            for (int a = 0; a < 3; a++) U[a * TILEV + cks(t.hpos, TILEV)] = mul_rn(cvq<HASD>(nxh[1 + a]), r);
         }
+        if (FULL || t.active) u4(nc, up, rhop);
         if (k + 1 < k1) pre(k + 1);
-        __syncthreads();  // readers of the previous plane are done
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            sh_st4(&U[a][ty + 1][VX + VX * tx], u0[a]);
-            if (htask == 0) sh_st4(&U[a][cks(hsy, HY)][cks4(hsx, HXV)], hu[a]);
-            else if (htask == 1) U[a][cks(hsy, HY)][cks(hsx, HXV)] = hu[a][0];
-        }
         __syncthreads();
-        if (active) {
-            const int col = VX + VX * tx;
-            C ym[3][VX], yp[3][VX], o[VX];
+        if (FULL || t.active) {
+            C ym[3][VX], yp[3][VX], o[VX], xl[3], xr[3];
 #pragma unroll
             for (int a = 0; a < 3; a++) {
-                sh_ld4(&U[a][ty][col], ym[a]);
-                sh_ld4(&U[a][ty + 2][col], yp[a]);
-            }
-            C xl[3], xr[3];
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                xl[a] = U[a][ty + 1][col - 1];
-                xr[a] = U[a][ty + 1][col + VX];
+                const C *T = U + a * TILEV + t.pos;
+                sh_ld4(T - t.pitch, ym[a]);
+                sh_ld4(T + t.pitch, yp[a]);
+                xl[a] = T[-1];
+                xr[a] = T[VX];
             }
 #pragma unroll
             for (int c = 0; c < VX; c++) {
                 C D[3][3];  // D[a][d]: undivided central difference of u_a along d
 #pragma unroll
                 for (int a = 0; a < 3; a++) {
-                    C xm = c > 0 ? u0[a][c - 1] : xl[a];
-                    C xp = c < VX - 1 ? u0[a][c + 1] : xr[a];
+                    const C xm = c > 0 ? u0[a][c - 1] : xl[a];
+                    const C xp = c < VX - 1 ? u0[a][c + 1] : xr[a];
                     D[a][0] = xp - xm;
                     D[a][1] = yp[a][c] - ym[a][c];
                     D[a][2] = up[a][c] - um[a][c];
                 }
                 o[c] = source_b(D, alpha_s);
             }
-            st4(CKP4(b + (idx)k * pl + (idx)(j * g.nx + i0), b, g.n), o);
-            if constexpr (kInc) st4(CKP4(rho_out + (idx)k * pl + (idx)(j * g.nx + i0), rho_out, g.n), rho0);
+            const idx at = (idx)k * pl + t.own;
+            st4(CKP4(b + at, b, g.n), o);
+            if constexpr (kInc) st4(CKP4(rho_out + at, rho_out, g.n), rho0);
+#pragma unroll
+            for (int a = 0; a < 3; a++)
+#pragma unroll
+                for (int c = 0; c < VX; c++) {
+                    um[a][c] = u0[a][c];
+                    u0[a][c] = up[a][c];
+                }
+#pragma unroll
+            for (int c = 0; c < VX; c++) rho0[c] = rhop[c];
         }
-#pragma unroll
-        for (int a = 0; a < 3; a++)
-#pragma unroll
-            for (int c = 0; c < VX; c++) {
-                um[a][c] = u0[a][c];
-                u0[a][c] = up[a][c];
-            }
-#pragma unroll
-        for (int c = 0; c < VX; c++) rho0[c] = rhop[c];
     }
-}
-// 4 raw state values (cells off .. off+3 of field u, inside one row)
-template <bool HASD>
-__device__ __forceinline__ QRaw4 ldq4d(const QIn &q, int u, const Geom &g, idx off)
-{
-    return StateIO4<kInc>::ldd<HASD>(q, u, g, off);
 }
 
-// The 4-cell source of a grid whose every tile lies inside (rows a multiple
-// of 128 cells, a multiple of 8 rows): the body of source_v4_body without
-// lanes past the row's end, with whole 4-wide loads and halo offsets mapped
-// once (warps 0 and 1: the rows below and above; lanes 0..15 of warp 2: the
-// cells left and right of the rows), and the plane tile double buffered.
-// The same operations per cell, so the same bits.
+// the pairs: u of a cell and the one above it, one halo cell per thread of
+// the first three warps, raw values one plane ahead
 template <bool HASD>
-__device__ __forceinline__ void source_v4_full(const QIn q, S *__restrict__ b, S *__restrict__ rho_out,
-                                               const Geom g, C alpha_s, const C *W, const C *J, int zc,
-                                               const BlockPos bp)
+__device__ __forceinline__ void source_pairs(const QIn q, S *__restrict__ b, S *__restrict__ rho_out, const Geom &g,
+                                             C alpha_s, const C *W, const C *J, int zc, const BlockPos &bp, C *U2)
 {
-    __shared__ __align__(16) C U2[2][3][HY][HXV];  // plane tiles of u, two planes alternating
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int x0 = bp.x * TXV, y0 = bp.y * BY;
-    const int i0 = x0 + VX * tx, j = y0 + ty;
+    const Pair t = pair_of(g, bp);
     const int k0 = bp.z * zc, k1 = min(g.nz, k0 + zc);
     const idx pl = (idx)g.plane;
-    const idx own = (idx)j * (idx)g.nx + (idx)i0;
-    const bool yh = ty < 2, xh = ty == 2 && tx < 2 * BY;
-    int hsy = 0, hsx = 0;
-    idx hoff = 0;
-    if (yh) {
-        hsy = ty ? HY - 1 : 0;
-        hsx = VX + VX * tx;
-        hoff = (idx)map_axis(y0 + (ty ? BY : -1), g.ny, g.bc[2], g.bc[3]) * (idx)g.nx + (idx)i0;
-    } else if (xh) {
-        const int side = tx / BY, r = tx % BY;
-        hsy = 1 + r;
-        hsx = side ? VX + TXV : VX - 1;
-        hoff = (idx)(y0 + r) * (idx)g.nx + (idx)map_axis(side ? x0 + TXV : x0 - 1, g.nx, g.bc[0], g.bc[1]);
-    }
-    auto u4 = [&](const QRaw4 (&r)[4], C u[3][VX], C rho[VX]) {
-        C m[VX], rr[VX];
-        cvq4<HASD>(r[0], rho);
+    QRaw nc[2][4], nh[4];
+    auto load = [&](int kk) {  // own cells of plane kk
+        const idx pz = (idx)zmap(kk, g) * pl;
 #pragma unroll
-        for (int c = 0; c < VX; c++) rr[c] = rcp(rho[c]);
+        for (int c = 0; c < 2; c++)
+            if (t.need[c]) {
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            cvq4<HASD>(r[1 + a], m);
-#pragma unroll
-            for (int c = 0; c < VX; c++) u[a][c] = mul_rn(m[c], rr[c]);
-        }
-    };
-    auto own_u = [&](int kk, C u[3][VX], C rho[VX]) {
-        const idx zb = (idx)zmap(kk, g) * pl + own;
-        C v[4][VX];
-#pragma unroll
-        for (int f = 0; f < 4; f++) cvq4<HASD>(ldq4d<HASD>(q, f, g, zb), v[f]);
-#pragma unroll
-        for (int c = 0; c < VX; c++) rho[c] = v[0][c];
-        if (kk < 0 && g.bc[4] == BC_INFLOW) {
-#pragma unroll
-            for (int c = 0; c < VX; c++) {
-                const idx fc = ck(own + (idx)c, g.plane);
-                C w = C(1) - W[fc];
-#pragma unroll
-                for (int f = 0; f < 4; f++) v[f][c] = fma_rn(w, v[f][c], J[(idx)f * pl + fc]);
+                for (int f = 0; f < 4; f++) nc[c][f] = ldqr<HASD>(q, f, ck(pz + t.own[c], g.n));
             }
-        }
-#pragma unroll
-        for (int c = 0; c < VX; c++) {
-            C r = rcp(v[0][c]);
-#pragma unroll
-            for (int a = 0; a < 3; a++) u[a][c] = mul_rn(v[1 + a][c], r);
-        }
     };
-    C um[3][VX], u0[3][VX], up[3][VX];
-    C rho0[VX], rhop[VX];
-    own_u(k0 - 1, um, rhop);
-    own_u(k0, u0, rho0);
-    constexpr bool kHaloAhead = !(kInc && HASD);
-    QRaw4 nc[4], nh[4];
-    QRaw nxh[4];
     auto halo = [&](int kk) {
-        if (yh) {
+        if (t.h) {
 #pragma unroll
-            for (int f = 0; f < 4; f++) nh[f] = ldq4d<HASD>(q, f, g, (idx)kk * pl + hoff);
-        } else if (xh) {
-#pragma unroll
-            for (int f = 0; f < 4; f++) nxh[f] = ldqr<HASD>(q, f, ck((idx)kk * pl + hoff, g.n));
+            for (int f = 0; f < 4; f++) nh[f] = ldqr<HASD>(q, f, ck((idx)kk * pl + t.hoff, g.n));
         }
     };
-    auto pre = [&](int kk) {
-        const idx pz = (idx)zmap(kk + 1, g) * pl + own;
+    // u = m / rho (products rounded before they are differenced: equal
+    // neighbours give an exact 0), with the jet blend below an inflow face
+    auto conv = [&](int kk, C (&u)[2][3], C (&rho)[2]) {
 #pragma unroll
-        for (int f = 0; f < 4; f++) nc[f] = ldq4d<HASD>(q, f, g, pz);
-        if (kHaloAhead) halo(kk);
+        for (int c = 0; c < 2; c++) {
+            if (!t.need[c]) continue;
+            C v[4];
+#pragma unroll
+            for (int f = 0; f < 4; f++) v[f] = cvq<HASD>(nc[c][f]);
+            rho[c] = v[0];
+            if (kk < 0 && g.bc[4] == BC_INFLOW) {
+                const idx f0 = ck(t.own[c], g.plane);
+                const C w = C(1) - W[f0];
+#pragma unroll
+                for (int f = 0; f < 4; f++) v[f] = fma_rn(w, v[f], J[(idx)f * pl + f0]);
+            }
+            const C r = rcp(v[0]);
+#pragma unroll
+            for (int a = 0; a < 3; a++) u[c][a] = mul_rn(v[1 + a], r);
+        }
     };
-    pre(k0);
-    const int col = VX + VX * tx;
+    C um[2][3] = {}, u0[2][3] = {}, up[2][3] = {}, rho0[2] = {}, rhop[2] = {};
+    load(k0 - 1);
+    conv(k0 - 1, um, rhop);
+    load(k0);
+    conv(k0, u0, rho0);
+    load(k0 + 1);
+    halo(k0);
     for (int k = k0; k < k1; k++) {
-        if (!kHaloAhead) halo(k);
-        // the buffer written here was last read two planes ago, before the
-        // barrier of the previous plane: one barrier per plane
-        C (*U)[HY][HXV] = U2[(k - k0) & 1];
+        C *U = U2 + ((k - k0) & 1) * 3 * TILEP;
 #pragma unroll
-        for (int a = 0; a < 3; a++) sh_st4(&U[a][ty + 1][col], u0[a]);
-        if (yh) {
-            C hu[3][VX], hrho[VX];
-            u4(nh, hu, hrho);
-#pragma unroll
-            for (int a = 0; a < 3; a++) sh_st4(&U[a][cks(hsy, HY)][cks4(hsx, HXV)], hu[a]);
-        } else if (xh) {
-            C r = rcp(cvq<HASD>(nxh[0]));
-#pragma unroll
-            for (int a = 0; a < 3; a++) U[a][cks(hsy, HY)][cks(hsx, HXV)] = mul_rn(cvq<HASD>(nxh[1 + a]), r);
+        for (int a = 0; a < 3; a++) {
+            U[a * TILEP + t.pos] = u0[0][a];
+            U[a * TILEP + t.pos + PPITCH] = u0[1][a];
         }
-        u4(nc, up, rhop);
-        if (k + 1 < k1) pre(k + 1);
+        if (t.h) {
+            const C r = rcp(cvq<HASD>(nh[0]));
+#pragma unroll
+            for (int a = 0; a < 3; a++) U[a * TILEP + cks(t.hpos, TILEP)] = mul_rn(cvq<HASD>(nh[1 + a]), r);
+        }
+        conv(k + 1, up, rhop);
+        if (k + 1 < k1) {
+            load(k + 2);
+            halo(k + 1);
+        }
         __syncthreads();
-        C ym[3][VX], yp[3][VX], o[VX];
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            sh_ld4(&U[a][ty][col], ym[a]);
-            sh_ld4(&U[a][ty + 2][col], yp[a]);
-        }
-        C xl[3], xr[3];
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            xl[a] = U[a][ty + 1][col - 1];
-            xr[a] = U[a][ty + 1][col + VX];
-        }
-#pragma unroll
-        for (int c = 0; c < VX; c++) {
-            C D[3][3];
+        for (int c = 0; c < 2; c++) {
+            if (!t.in[c]) continue;
+            C D[3][3];  // D[a][d]: undivided central difference of u_a along d
 #pragma unroll
             for (int a = 0; a < 3; a++) {
-                C xm = c > 0 ? u0[a][c - 1] : xl[a];
-                C xp = c < VX - 1 ? u0[a][c + 1] : xr[a];
-                D[a][0] = xp - xm;
-                D[a][1] = yp[a][c] - ym[a][c];
-                D[a][2] = up[a][c] - um[a][c];
+                const C *T = U + a * TILEP + t.pos + c * PPITCH;
+                D[a][0] = T[1] - T[-1];
+                D[a][1] = (c ? T[PPITCH] : u0[1][a]) - (c ? u0[0][a] : T[-PPITCH]);
+                D[a][2] = up[c][a] - um[c][a];
             }
-            o[c] = source_b(D, alpha_s);
+            const idx at = (idx)k * pl + t.own[c];
+            stc(CKP(b + at, b, g.n), source_b(D, alpha_s));
+            if constexpr (kInc) stc(CKP(rho_out + at, rho_out, g.n), rho0[c]);
         }
-        st4(CKP4(b + (idx)k * pl + own, b, g.n), o);
-        if constexpr (kInc) st4(CKP4(rho_out + (idx)k * pl + own, rho_out, g.n), rho0);
 #pragma unroll
-        for (int a = 0; a < 3; a++)
+        for (int c = 0; c < 2; c++) {
 #pragma unroll
-            for (int c = 0; c < VX; c++) {
-                um[a][c] = u0[a][c];
-                u0[a][c] = up[a][c];
+            for (int a = 0; a < 3; a++) {
+                um[c][a] = u0[c][a];
+                u0[c][a] = up[c][a];
             }
-#pragma unroll
-        for (int c = 0; c < VX; c++) rho0[c] = rhop[c];
+            rho0[c] = rhop[c];
+        }
     }
 }
 
@@ -1734,19 +1482,21 @@ __device__ __forceinline__ void source_v4_full(const QIn q, S *__restrict__ b, S
 // 156 registers), runs it 1.6x slower. The increment modes' form, which
 // holds raw FP32 values and 16-bit increments one plane ahead, spills a few
 // registers under this bound and still runs faster. FP64 keeps one block.
-constexpr int SOURCE_V4_BLOCKS = sizeof(C) == 8 ? 1 : 2;
-template <bool HASD>
-__global__ void __launch_bounds__(BT, SOURCE_V4_BLOCKS) k_source_v4(QIn q, S *__restrict__ b, S *__restrict__ rho_out, Geom g,
-                                                   C alpha_s, const C *W, const C *J, int zc)
+constexpr int SOURCE_BLOCKS = sizeof(C) == 8 ? 1 : 2;
+template <bool HASD, bool FULL>
+__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source(QIn q, S *__restrict__ b, S *__restrict__ rho_out, Geom g,
+                                                              C alpha_s, const C *W, const C *J, int zc, int wq,
+                                                              int rows)
 {
-    source_v4_body<HASD>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch());
+    __shared__ __align__(16) C U2[SOURCE_BUFS * 3 * TILEV];
+    source_quads<HASD, FULL>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch(), wq, rows, U2);
 }
 template <bool HASD>
-__global__ void __launch_bounds__(BT, SOURCE_V4_BLOCKS) k_source_v4_full(QIn q, S *__restrict__ b,
-                                                                        S *__restrict__ rho_out, Geom g,
-                                                                        C alpha_s, const C *W, const C *J, int zc)
+__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_pairs(QIn q, S *__restrict__ b, S *__restrict__ rho_out,
+                                                                    Geom g, C alpha_s, const C *W, const C *J, int zc)
 {
-    source_v4_full<HASD>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch());
+    __shared__ C U2[2 * 3 * TILEP];
+    source_pairs<HASD>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch(), U2);
 }
 
 
@@ -1863,7 +1613,6 @@ __device__ __forceinline__ void cp_async_elem(C *dst, const S *src)
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // shared bytes: the ring of plane tiles (pairs), two sets of x- and y-face fluxes
@@ -2851,14 +2600,14 @@ struct SourceInst {
     Geom g;
     C alpha_s;
     const C *W, *J;
-    int zc, gx, gy, blk0;
+    int zc, wq, rows, gx, gy, blk0;
 };
 struct JacobiInst {
     const S *q, *b, *sin;
     S *sout;
     Geom g;
     C beta;
-    int zc, gx, gy, blk0;
+    int zc, wq, rows, gx, gy, blk0;
 };
 struct FluxInst {
     QIn qin;
@@ -2892,51 +2641,47 @@ template <class I> __device__ __forceinline__ int group_find(const Group<I> &a, 
     return lo;
 }
 
-template <bool HASD>
-__global__ void __launch_bounds__(BT) k_source_group(const __grid_constant__ Group<SourceInst> a)
+template <bool HASD, bool FULL>
+__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_group(const __grid_constant__ Group<SourceInst> a)
 {
+    __shared__ __align__(16) C U2[SOURCE_BUFS * 3 * TILEV];
     const SourceInst &d = a.d[group_find(a, blockIdx.x)];
-    source_body<HASD>(d.q, d.b, d.rho_out, d.g, d.alpha_s, d.W, d.J, d.zc,
-                      BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy));
+    source_quads<HASD, FULL>(d.q, d.b, d.rho_out, d.g, d.alpha_s, d.W, d.J, d.zc,
+                             BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy), d.wq, d.rows, U2);
 }
 template <bool HASD>
-__global__ void __launch_bounds__(BT, SOURCE_V4_BLOCKS) k_source_v4_group(const __grid_constant__ Group<SourceInst> a)
+__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_pairs_group(const __grid_constant__ Group<SourceInst> a)
 {
+    __shared__ C U2[2 * 3 * TILEP];
     const SourceInst &d = a.d[group_find(a, blockIdx.x)];
-    source_v4_body<HASD>(d.q, d.b, d.rho_out, d.g, d.alpha_s, d.W, d.J, d.zc,
-                         BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy));
+    source_pairs<HASD>(d.q, d.b, d.rho_out, d.g, d.alpha_s, d.W, d.J, d.zc,
+                       BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy), U2);
 }
-__global__ void __launch_bounds__(BT) k_jacobi_group(const __grid_constant__ Group<JacobiInst> a, int colour)
+template <bool RB, int NR>
+__global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full_group(const __grid_constant__ Group<JacobiInst> a,
+                                                                        int colour)
 {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const JacobiInst &d = a.d[group_find(a, blockIdx.x)];
-    jacobi_body(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
-                BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy));
+    jacobi_quads<true, RB, NR>(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
+                           BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy), FQ, FR, smem_raw);
 }
-__global__ void __launch_bounds__(BT, JACOBI_V4_BLOCKS) k_jacobi_v4_group(const __grid_constant__ Group<JacobiInst> a,
-                                                                         int colour)
+__global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit_group(const __grid_constant__ Group<JacobiInst> a,
+                                                                           int colour)
 {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const JacobiInst &d = a.d[group_find(a, blockIdx.x)];
-    jacobi_v4_body(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
-                   BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy));
+    jacobi_quads<false, false, 1>(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
+                               BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy), d.wq, d.rows, smem_raw);
 }
-template <bool HASD>
-__global__ void __launch_bounds__(BT, SOURCE_V4_BLOCKS) k_source_v4_full_group(const __grid_constant__ Group<SourceInst> a)
+__global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS)
+    k_jacobi_pairs_group(const __grid_constant__ Group<JacobiInst> a, int colour)
 {
-    const SourceInst &d = a.d[group_find(a, blockIdx.x)];
-    source_v4_full<HASD>(d.q, d.b, d.rho_out, d.g, d.alpha_s, d.W, d.J, d.zc,
-                         BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy));
-}
-template <bool RB>
-__global__ void __launch_bounds__(BT, JACOBI_V4_BLOCKS) k_jacobi_v4_full_group(const __grid_constant__ Group<JacobiInst> a,
-                                                                              int colour)
-{
-    if constexpr (sizeof(C) == 4) {
-        __shared__ __align__(16) C R[2][HY][HXV];
-        __shared__ __align__(16) C SG[2][HY][HXV];
-        const JacobiInst &d = a.d[group_find(a, blockIdx.x)];
-        jacobi_v4_full<RB>(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
-                           BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy), R, SG);
-    }
+    __shared__ C R[2 * TILEP];
+    __shared__ C SG[2 * TILEP];
+    const JacobiInst &d = a.d[group_find(a, blockIdx.x)];
+    jacobi_pairs(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
+                 BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy), R, SG);
 }
 template <int mode, int ORD, bool VISC>
 __global__ void __maxnreg__(FLUX_MAXREG) k_flux_group(const __grid_constant__ Group<FluxInst> a)
@@ -2974,6 +2719,52 @@ QIn state_in(const void *q, const void *qd, long long n)
     return f;
 }
 
+template <class K> cudaError_t allow_smem(K kern, int bytes)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+// Kernel form of a source or sweep launch: 2 full quad tiles, 1 fitted quad
+// tiles, 0 pairs; a sweep's form 3: full tiles with two rows per thread
+// (16-bit storage; from 16M cells: FP16, 512 x 512 x 128: 74 us against 80
+// with one; 256 x 256 x 192: 32 against 29.5). Its grid and block.
+int quad_form(const Geom &g, const Tiles &t)
+{
+    if (t.elem || g.nx % VX != 0) return 0;
+    return quad_fit(g).full ? 2 : 1;
+}
+int sweep_form(const Geom &g, const Tiles &t)
+{
+    const int form = quad_form(g, t);
+    return form == 2 && sizeof(S) == 2 && g.ny % (2 * FR) == 0 && g.n >= (1 << 24) ? 3 : form;
+}
+// the source takes the compiled-in tile in the 16-bit forms only (FP32, 256^3:
+// 90.8 us against 72.2 with the tile's shape at run time)
+bool source_full(int form) { return form == 2 && sizeof(S) == 2; }
+dim3 quad_grid(const Geom &g, int form, int zc)
+{
+    if (!form) return grid_of(g, PX, PY, zc);
+    const QuadFit f = quad_fit(g);
+    return dim3(f.gx, form == 3 ? f.gy / 2 : f.gy, (g.nz + zc - 1) / zc);
+}
+int quad_threads(const Geom &g, int form) { return form ? quad_fit(g).threads : 32 * PWARPS; }
+// blocks per plane and blocks per SM (Ops::source_shape, Ops::jacobi_shape)
+void source_shape(const Geom &g, long long *cols, int *resident)
+{
+    const int form = quad_form(g, Tiles{});
+    const dim3 gr = quad_grid(g, form, g.nz);
+    *cols = (long long)gr.x * gr.y;
+    *resident = (sizeof(C) == 8 ? 256 : 512) / quad_threads(g, form);
+}
+void jacobi_shape(const Geom &g, long long *cols, int *resident)
+{
+    const int form = sweep_form(g, Tiles{});
+    const dim3 gr = quad_grid(g, form, g.nz);
+    *cols = (long long)gr.x * gr.y;
+    const int blocks = form == 3 ? kJacobiBlocks<2> : form == 2 ? kJacobiBlocks<1> : form ? JACOBI_FIT_BLOCKS : JACOBI_PAIR_BLOCKS;
+    *resident = blocks * BT / quad_threads(g, form);
+}
+
 cudaError_t launch_source(const Geom &g, const Phys &p, const Tiles &t, const Inflow &in,
                           const void *q, const void *qd, void *b, void *rho_out, cudaStream_t st)
 {
@@ -2982,42 +2773,47 @@ cudaError_t launch_source(const Geom &g, const Phys &p, const Tiles &t, const In
     const QIn qi = state_in(q, qd, g.n);
     const C as = C(p.alpha * 0.25 / (p.dx * p.dx));
     const C *W = (const C *)in.W, *J = (const C *)in.J;
-    if (t.vec_source && g.nx % VX == 0) {
-        auto kern = qd ? k_source_v4<kInc> : k_source_v4<false>;
-        // 16-bit storage: grids whose tiles all lie inside take the full-tile
-        // kernel (FP16 increments, full-size plume: 12.0 -> 10.7 ms); with
-        // FP32 storage it measured slower (8.6 -> 10.5 ms) and is not used
-        if (sizeof(S) == 2 && g.nx % TXV == 0 && g.ny % BY == 0)
-            kern = qd ? k_source_v4_full<kInc> : k_source_v4_full<false>;
-        kern<<<grid_of(g, TXV, BY, t.zc_source), dim3(BX, BY), 0, st>>>(qi, (S *)b, (S *)rho_out, g, as, W, J,
-                                                                       t.zc_source);
-        return cudaGetLastError();
+    const QuadFit f = quad_fit(g);
+    const int form = quad_form(g, t), threads = quad_threads(g, form);
+    const dim3 gr = quad_grid(g, form, t.zc_source);
+    if (form) {
+        auto kern = source_full(form) ? (qd ? k_source<kInc, true> : k_source<false, true>)
+                              : (qd ? k_source<kInc, false> : k_source<false, false>);
+        kern<<<gr, threads, 0, st>>>(qi, (S *)b, (S *)rho_out, g, as, W, J, t.zc_source, f.wq, f.rows);
+    } else {
+        auto kern = qd ? k_source_pairs<kInc> : k_source_pairs<false>;
+        kern<<<gr, threads, 0, st>>>(qi, (S *)b, (S *)rho_out, g, as, W, J, t.zc_source);
     }
-    auto kern = qd ? k_source<kInc> : k_source<false>;
-    kern<<<grid_of(g, BX, BY, t.zc_source), dim3(BX, BY), 0, st>>>(qi, (S *)b, (S *)rho_out, g, as, W, J,
-                                                                   t.zc_source);
     return cudaGetLastError();
 }
 
+constexpr int kRows = sizeof(S) == 2 ? 2 : 1;  // rows per thread of form 3
+template <int NR> auto full_sweep(int colour) { return colour < 0 ? k_jacobi_full<false, NR> : k_jacobi_full<true, NR>; }
+template <int NR> auto full_sweep_group(int colour)
+{
+    return colour < 0 ? k_jacobi_full_group<false, NR> : k_jacobi_full_group<true, NR>;
+}
 cudaError_t launch_jacobi(const Geom &g, const Phys &p, const Tiles &t, const void *q,
                           const void *b, const void *s_in, void *s_out, int colour, cudaStream_t st)
 {
-    if (t.vec_jacobi && g.nx % VX == 0) {
-        if (sizeof(C) == 4 && g.nx % TXV == 0 && g.ny % BY == 0) {
-            auto kern = colour < 0 ? k_jacobi_v4_full<false> : k_jacobi_v4_full<true>;
-            kern<<<grid_of(g, TXV, BY, t.zc_jacobi), dim3(BX, BY), 0, st>>>(
-                (const S *)q, (const S *)b, (const S *)s_in, (S *)s_out, g, C(p.alpha / (p.dx * p.dx)),
-                t.zc_jacobi, colour);
-            return cudaGetLastError();
-        }
-        k_jacobi_v4<<<grid_of(g, TXV, BY, t.zc_jacobi), dim3(BX, BY), 0, st>>>(
-            (const S *)q, (const S *)b, (const S *)s_in, (S *)s_out, g, C(p.alpha / (p.dx * p.dx)),
-            t.zc_jacobi, colour);
-        return cudaGetLastError();
+    const QuadFit f = quad_fit(g);
+    const int form = sweep_form(g, t), threads = quad_threads(g, form);
+    const dim3 gr = quad_grid(g, form, t.zc_jacobi);
+    const C beta = C(p.alpha / (p.dx * p.dx));
+    const S *qs = (const S *)q, *bs = (const S *)b, *si = (const S *)s_in;
+    if (form >= 2) {
+        auto kern = form == 3 ? full_sweep<kRows>(colour) : full_sweep<1>(colour);
+        const int smem = form == 3 ? JShape<kRows>::SMEM : JShape<1>::SMEM;
+        cudaError_t e = allow_smem(kern, smem);
+        if (e != cudaSuccess) return e;
+        kern<<<gr, threads, smem, st>>>(qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour);
+    } else if (form) {
+        cudaError_t e = allow_smem(k_jacobi_fit, JShape<1>::SMEM);
+        if (e != cudaSuccess) return e;
+        k_jacobi_fit<<<gr, threads, JShape<1>::SMEM, st>>>(qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour, f.wq, f.rows);
+    } else {
+        k_jacobi_pairs<<<gr, threads, 0, st>>>(qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour);
     }
-    k_jacobi<<<grid_of(g, BX, BY, t.zc_jacobi), dim3(BX, BY), 0, st>>>(
-        (const S *)q, (const S *)b, (const S *)s_in, (S *)s_out, g, C(p.alpha / (p.dx * p.dx)),
-        t.zc_jacobi, colour);
     return cudaGetLastError();
 }
 
@@ -3115,20 +2911,15 @@ cudaError_t launch_source_group(const SourceCall *calls, int n, cudaStream_t st)
 {
     for (int i = 0; i < n; i++)
         if ((kInc != (calls[i].rho_out != nullptr)) || (!kInc && calls[i].qd)) return cudaErrorInvalidValue;
-    // 0: one cell per thread, 1: four cells, 2: four cells, every tile inside
-    // the grid (16-bit storage; as launch_source)
-    auto vec = [](const SourceCall &c) {
-        if (!c.t.vec_source || c.g.nx % VX != 0) return 0;
-        return sizeof(S) == 2 && c.g.nx % TXV == 0 && c.g.ny % BY == 0 ? 2 : 1;
-    };
-    auto key = [&](const SourceCall &c) { return 2 * vec(c) + (c.qd ? 1 : 0); };
+    auto key = [](const SourceCall &c) { return 2 * quad_form(c.g, c.t) + (c.qd ? 1 : 0); };
     return by_runs(calls, n, key, [&](const SourceCall *cs, int m) {
         Group<SourceInst> a;
         a.count = m;
-        int blk = 0;
-        const int v = vec(cs[0]);
+        int blk = 0, threads = 0;
+        const int form = key(cs[0]) >> 1;
         for (int i = 0; i < m; i++) {
             const SourceCall &c = cs[i];
+            const QuadFit f = quad_fit(c.g);
             SourceInst &d = a.d[i];
             d.q = state_in(c.q, c.qd, c.g.n);
             d.b = (S *)c.b;
@@ -3138,35 +2929,34 @@ cudaError_t launch_source_group(const SourceCall *calls, int n, cudaStream_t st)
             d.W = (const C *)c.in.W;
             d.J = (const C *)c.in.J;
             d.zc = c.t.zc_source;
-            const dim3 gr = grid_of(c.g, v ? TXV : BX, BY, d.zc);
+            d.wq = f.wq;
+            d.rows = f.rows;
+            const dim3 gr = quad_grid(c.g, form, d.zc);
             d.gx = (int)gr.x;
             d.gy = (int)gr.y;
             d.blk0 = blk;
             blk += (int)(gr.x * gr.y * gr.z);
+            threads = std::max(threads, quad_threads(c.g, form));
         }
-        auto kern = v == 2 ? (cs[0].qd ? k_source_v4_full_group<kInc> : k_source_v4_full_group<false>)
-                    : v ? (cs[0].qd ? k_source_v4_group<kInc> : k_source_v4_group<false>)
-                        : (cs[0].qd ? k_source_group<kInc> : k_source_group<false>);
-        kern<<<blk, dim3(BX, BY), 0, st>>>(a);
+        auto kern = source_full(form) ? (cs[0].qd ? k_source_group<kInc, true> : k_source_group<false, true>)
+                    : form ? (cs[0].qd ? k_source_group<kInc, false> : k_source_group<false, false>)
+                           : (cs[0].qd ? k_source_pairs_group<kInc> : k_source_pairs_group<false>);
+        kern<<<blk, threads, 0, st>>>(a);
         return cudaGetLastError();
     });
 }
 
 cudaError_t launch_jacobi_group(const JacobiCall *calls, int n, int colour, cudaStream_t st)
 {
-    // 0: one cell per thread, 1: four cells, 2: four cells, every tile inside
-    // the grid (FP32 arithmetic; as launch_jacobi)
-    auto vec = [](const JacobiCall &c) {
-        if (!c.t.vec_jacobi || c.g.nx % VX != 0) return 0;
-        return sizeof(C) == 4 && c.g.nx % TXV == 0 && c.g.ny % BY == 0 ? 2 : 1;
-    };
-    return by_runs(calls, n, vec, [&](const JacobiCall *cs, int m) {
+    auto key = [](const JacobiCall &c) { return sweep_form(c.g, c.t); };
+    return by_runs(calls, n, key, [&](const JacobiCall *cs, int m) {
         Group<JacobiInst> a;
         a.count = m;
-        int blk = 0;
-        const int v = vec(cs[0]);
+        int blk = 0, threads = 0;
+        const int form = key(cs[0]);
         for (int i = 0; i < m; i++) {
             const JacobiCall &c = cs[i];
+            const QuadFit f = quad_fit(c.g);
             JacobiInst &d = a.d[i];
             d.q = (const S *)c.q;
             d.b = (const S *)c.b;
@@ -3175,20 +2965,21 @@ cudaError_t launch_jacobi_group(const JacobiCall *calls, int n, int colour, cuda
             d.g = c.g;
             d.beta = C(c.p.alpha / (c.p.dx * c.p.dx));
             d.zc = c.t.zc_jacobi;
-            const dim3 gr = grid_of(c.g, v ? TXV : BX, BY, d.zc);
+            d.wq = f.wq;
+            d.rows = f.rows;
+            const dim3 gr = quad_grid(c.g, form, d.zc);
             d.gx = (int)gr.x;
             d.gy = (int)gr.y;
             d.blk0 = blk;
             blk += (int)(gr.x * gr.y * gr.z);
+            threads = std::max(threads, quad_threads(c.g, form));
         }
-        if (v == 2) {
-            auto kern = colour < 0 ? k_jacobi_v4_full_group<false> : k_jacobi_v4_full_group<true>;
-            kern<<<blk, dim3(BX, BY), 0, st>>>(a, colour);
-        } else if (v) {
-            k_jacobi_v4_group<<<blk, dim3(BX, BY), 0, st>>>(a, colour);
-        } else {
-            k_jacobi_group<<<blk, dim3(BX, BY), 0, st>>>(a, colour);
-        }
+        auto kern = form == 3 ? full_sweep_group<kRows>(colour)
+                    : form == 2 ? full_sweep_group<1>(colour) : form ? k_jacobi_fit_group : k_jacobi_pairs_group;
+        const int smem = form == 3 ? JShape<kRows>::SMEM : form ? JShape<1>::SMEM : 0;
+        cudaError_t e = allow_smem(kern, smem);
+        if (e != cudaSuccess) return e;
+        kern<<<blk, threads, smem, st>>>(a, colour);
         return cudaGetLastError();
     });
 }
@@ -3388,7 +3179,7 @@ extern const Ops IGR_OPS = {
     (int)sizeof(S), (int)sizeof(C), (int)sizeof(QB), launch_source, launch_jacobi, launch_flux, flux_blocks,
     launch_speed, launch_rk_combine, launch_adj_rk, launch_adj_rhs, launch_adj_jacobi, launch_adj_rho,
     launch_adj_source, launch_adj_jets, launch_diag, bounds_hits, bounds_selftest,
-    launch_source_group, launch_jacobi_group, launch_flux_group,
+    launch_source_group, launch_jacobi_group, launch_flux_group, source_shape, jacobi_shape,
 };
 
 }  // namespace igr

@@ -116,9 +116,9 @@ igr_status igr_solve_sigma_noalloc(const igr_config *cfg, const void *q, void *s
     p.order = cfg->order == 3 ? 3 : 5;
     p.mu = cfg->mu;
     p.zeta = cfg->zeta;
-    Tiles t = default_tiles(g);
+    Tiles t = default_tiles(g, o);
     if (!is_aligned(q, vec4_align(sb)) || !is_aligned(sigma_inout, vec4_align(sb)))
-        t.vec_source = t.vec_jacobi = 0;  // the 1-cell forms: same bits, element alignment only
+        t.elem = 1;  // element accesses: the same bits, element alignment only
     Inflow none;
     none.W = nullptr;
     none.J = nullptr;
