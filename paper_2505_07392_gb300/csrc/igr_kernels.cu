@@ -245,7 +245,7 @@ __device__ __forceinline__ double sqrt_c(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_c(float x)
 {
     float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 
@@ -280,6 +280,20 @@ __device__ __forceinline__ double2 pmul(double2 a, double2 b)
 __device__ __forceinline__ double2 pfma(double2 a, double2 b, double2 c)
 {
     return make_double2(__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y));
+}
+// a - b
+__device__ __forceinline__ float2 psub(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 ra, rb, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n sub.rn.f32x2 rd, ra, rb;\n"
+        " mov.b64 {%0, %1}, rd;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ double2 psub(double2 a, double2 b)
+{
+    return make_double2(__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y));
 }
 __device__ __forceinline__ C2 pset(C x, C y)
 {
@@ -346,26 +360,37 @@ template <class T> __device__ __forceinline__ void flag_face(T &f, C a, C b, C c
 }
 __device__ __forceinline__ bool flag_bad(bool f) { return f; }
 template <class T> __device__ __forceinline__ bool flag_bad(T f) { return !(f > T(0)); }
+// The five components of a flux: (rho, m_x), (m_y, m_z), E
+struct Flux {
+    C2 a, b;
+    C e;
+};
+// gas constants of the flux: gamma - 1 and sqrt(gamma (gamma - 1))
+struct Gas {
+    C gm1, sg;
+};
 template <int D>
-__device__ __forceinline__ void lf_flux2(const C *L, const C *R, C gamma, C gm1, C *G, FaceFlag &bad)
+__device__ __forceinline__ void lf_flux2(const C2 (&L)[3], const C2 (&R)[3], const Gas gas, Flux &G, FaceFlag &bad)
 {
-    C rL = rcp(L[0]), rR = rcp(R[0]);
-    C uL = L[1 + D] * rL, uR = R[1 + D] * rR;
-    C pL = gm1 * (L[4] - C(0.5) * ((L[1] * L[1] + L[2] * L[2] + L[3] * L[3]) * rL));
-    C pR = gm1 * (R[4] - C(0.5) * ((R[1] * R[1] + R[2] * R[2] + R[3] * R[3]) * rR));
-    flag_face(bad, L[0], R[0], pL, pR);
-    C aL = fabs(uL) + sqrt_c(gamma * pL * rL);
-    C aR = fabs(uR) + sqrt_c(gamma * pR * rR);
-    C lam = fmax(aL, aR);  // a NaN speed comes with a flagged face
-    C PL = pL + L[5], PR = pR + R[5];
-    G[0] = (L[1 + D] + R[1 + D]) - lam * (R[0] - L[0]);
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        C f = L[1 + a] * uL + R[1 + a] * uR;
-        if (a == D) f += PL + PR;
-        G[1 + a] = f - lam * (R[1 + a] - L[1 + a]);
-    }
-    G[4] = ((L[4] + PL) * uL + (R[4] + PR) * uR) - lam * (R[4] - L[4]);
+    const C mL = D == 0 ? L[0].y : D == 1 ? L[1].x : L[1].y, mR = D == 0 ? R[0].y : D == 1 ? R[1].x : R[1].y;
+    const C rL = rcp(L[0].x), rR = rcp(R[0].x);
+    const C uL = mL * rL, uR = mR * rR;
+    // e = p / (gamma - 1), c = sqrt(gamma p / rho) = sg sqrt(e / rho)
+    const C eL = L[2].x - C(0.5) * ((L[0].y * L[0].y + L[1].x * L[1].x + L[1].y * L[1].y) * rL);
+    const C eR = R[2].x - C(0.5) * ((R[0].y * R[0].y + R[1].x * R[1].x + R[1].y * R[1].y) * rR);
+    flag_face(bad, L[0].x, R[0].x, eL, eR);
+    const C aL = fabs(uL) + gas.sg * sqrt_c(eL * rL);
+    const C aR = fabs(uR) + gas.sg * sqrt_c(eR * rR);
+    const C lam = fmax(aL, aR);  // a NaN speed comes with a flagged face
+    const C PL = gas.gm1 * eL + L[2].y, PR = gas.gm1 * eR + R[2].y;
+    const C2 nl = bcast(-lam);
+    C fx = L[0].y * uL + R[0].y * uR, fy = L[1].x * uL + R[1].x * uR, fz = L[1].y * uL + R[1].y * uR;
+    if (D == 0) fx += PL + PR;
+    if (D == 1) fy += PL + PR;
+    if (D == 2) fz += PL + PR;
+    G.a = pfma(nl, psub(R[0], L[0]), pset(mL + mR, fx));
+    G.b = pfma(nl, psub(R[1], L[1]), pset(fy, fz));
+    G.e = ((L[2].x + PL) * uL + (R[2].x + PR) * uR) - lam * (R[2].x - L[2].x);
 }
 
 // wave speed max_d |u_d| + c at a cell
@@ -1599,7 +1624,24 @@ __device__ __forceinline__ void st_cell(C2 *T, int e, C2 a, C2 b, C2 c)
     st_quad(T, e, a, b);
     T[QUADS + e] = c;
 }
-constexpr int NFX = 5 * TY * (TX + 1), NFY = 5 * (TY + 1) * TX;  // one parity of the face buffers
+// Face buffers of one parity: x-faces at w (TX + 1) + i, y-faces at w TX + i,
+// each its two pairs side by side, then the E fluxes of all faces
+constexpr int NFX = (TY * (TX + 1) + 3) / 4 * 4, NFY = (TY + 1) * TX, NFACE = 5 * (NFX + NFY);
+__device__ __forceinline__ void ld_face(const C *B, int nf, int e, Flux &f)
+{
+    ld_quad(reinterpret_cast<const C2 *>(B), e, f.a, f.b);
+    f.e = B[4 * nf + e];
+}
+__device__ __forceinline__ void st_face(C *B, int nf, int e, const Flux &f)
+{
+    st_quad(reinterpret_cast<C2 *>(B), e, f.a, f.b);
+    B[4 * nf + e] = f.e;
+}
+// planes per turn of the march's loop: two in FP32 storage, where half the
+// register rotations go (512 x 512 x 256, stages 1 to 3: 1.84 -> 1.78 ms per
+// launch); the 16-bit forms, whose raw values are in flight in registers, and
+// FP64 measured the same or slower (FP16 0.937 -> 0.965 ms, 512 x 512 x 128)
+constexpr int kUnroll = sizeof(S) == 4 ? 2 : 1;
 constexpr int RING = 7;             // plane tiles resident: k-2..k+3 and k+4 in flight
 
 // Storage equal to the arithmetic type: plane tiles are copied global ->
@@ -1618,7 +1660,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // shared bytes: the ring of plane tiles (pairs), two sets of x- and y-face fluxes
 __host__ __device__ constexpr size_t flux_smem_bytes()
 {
-    return RING * TILE2 * sizeof(C2) + 2 * (5 * TY * (TX + 1) + 5 * (TY + 1) * TX) * sizeof(C);
+    return RING * TILE2 * sizeof(C2) + 2 * NFACE * sizeof(C);
 }
 
 // tile cell e (0 <= e < NPLANE) -> position (lx, ly) in the PW x PH tile
@@ -1631,29 +1673,23 @@ __device__ __forceinline__ void plane_cell(int e, int &lx, int &ly)
 }
 
 template <int D, int ORD>
-__device__ __forceinline__ void face_from_stencil(const C2 (&s)[6][3], C gamma, C gm1, C *F,
-                                                  FaceFlag &bad)
+__device__ __forceinline__ void face_from_stencil(const C2 (&s)[6][3], const Gas gas, Flux &F, FaceFlag &bad)
 {
-    C L[6], R[6];
+    C2 L[3], R[3];
 #pragma unroll
     for (int p = 0; p < 3; p++) {
-        C2 l = ORD == 3 ? rec3_left2(s[1][p], s[2][p], s[3][p])
+        L[p] = ORD == 3 ? rec3_left2(s[1][p], s[2][p], s[3][p])
                         : rec_left2(s[0][p], s[1][p], s[2][p], s[3][p], s[4][p]);
-        C2 r = ORD == 3 ? rec3_right2(s[2][p], s[3][p], s[4][p])
+        R[p] = ORD == 3 ? rec3_right2(s[2][p], s[3][p], s[4][p])
                         : rec_right2(s[1][p], s[2][p], s[3][p], s[4][p], s[5][p]);
-        L[2 * p] = l.x;
-        L[2 * p + 1] = l.y;
-        R[2 * p] = r.x;
-        R[2 * p + 1] = r.y;
     }
-    lf_flux2<D>(L, R, gamma, gm1, F, bad);
+    lf_flux2<D>(L, R, gas, F, bad);
 }
 
 // face along D (0, 1) from six consecutive cells of one plane tile starting
 // at element `at`, `step` elements apart
 template <int D, int ORD>
-__device__ __forceinline__ void tile_face(const C2 *T, int at, int step, C gamma, C gm1, C *F,
-                                          FaceFlag &bad)
+__device__ __forceinline__ void tile_face(const C2 *T, int at, int step, const Gas gas, Flux &F, FaceFlag &bad)
 {
     C2 s[6][3];
 #pragma unroll
@@ -1664,14 +1700,14 @@ __device__ __forceinline__ void tile_face(const C2 *T, int at, int step, C gamma
             ld_cell(T, cks(at + m * step, PH * PW), s[m][0], s[m][1], s[m][2]);
         }
     }
-    face_from_stencil<D, ORD>(s, gamma, gm1, F, bad);
+    face_from_stencil<D, ORD>(s, gas, F, bad);
 }
 
 // tile_face with the stencil's point 3 (the cell the face lies below / left of
 // the row warp's own cell) given: the row warp holds it from its z-stencil
 template <int D, int ORD>
-__device__ __forceinline__ void tile_face_c(const C2 *T, int at, int step, const C2 (&c3)[3], C gamma, C gm1,
-                                            C *F, FaceFlag &bad)
+__device__ __forceinline__ void tile_face_c(const C2 *T, int at, int step, const C2 (&c3)[3], const Gas gas, Flux &F,
+                                            FaceFlag &bad)
 {
     C2 s[6][3];
 #pragma unroll
@@ -1686,7 +1722,7 @@ __device__ __forceinline__ void tile_face_c(const C2 *T, int at, int step, const
             ld_cell(T, cks(at + m * step, PH * PW), s[m][0], s[m][1], s[m][2]);
         }
     }
-    face_from_stencil<D, ORD>(s, gamma, gm1, F, bad);
+    face_from_stencil<D, ORD>(s, gas, F, bad);
 }
 
 // ------------------------------------------------------- viscous stresses
@@ -1715,7 +1751,7 @@ __device__ __forceinline__ void visc_face(const C2 *TA, int a, const C2 *TB, int
                                           int a1m, const C2 *T1Ap, int a1p, const C2 *T1Bm, int b1m,
                                           const C2 *T1Bp, int b1p, const C2 *T2Am, int a2m,
                                           const C2 *T2Ap, int a2p, const C2 *T2Bm, int b2m,
-                                          const C2 *T2Bp, int b2p, C mu, C lam, C inv_dx, C *G)
+                                          const C2 *T2Bp, int b2p, C mu, C lam, C inv_dx, Flux &G)
 {
     constexpr int t1 = D == 0 ? 1 : 0, t2 = D == 2 ? 1 : 2;
     C uA[3], uB[3], p[3], m[3], q[3], r[3], Gr[3][3];
@@ -1736,10 +1772,10 @@ __device__ __forceinline__ void visc_face(const C2 *TA, int a, const C2 *TB, int
     for (int c = 0; c < 3; c++) {
         C tau = mu * (Gr[c][D] + Gr[D][c]);
         if (c == D) tau += lam * div;
-        G[1 + c] -= C(2) * tau;
+        (c == 0 ? G.a.y : c == 1 ? G.b.x : G.b.y) -= C(2) * tau;
         work += C(0.5) * (uA[c] + uB[c]) * tau;
     }
-    G[4] -= C(2) * work;
+    G.e -= C(2) * work;
 }
 
 // registers per thread such that NWARP / 4 warps fit one sub-partition's 16K
@@ -1760,6 +1796,17 @@ constexpr int FLUX_MAXREG = sizeof(C) == 8 ? 224 : 128;
 // mapping and, below an inflow face, the jet blend). Every plane is read from
 // global memory once per block; nothing relies on the L1 cache.
 //
+// What bounds it is the latency of 16 warps' shared loads, MUFU operations
+// and dependent arithmetic (issue slots 57% busy, shared-memory bandwidth
+// 42%, no pipe above 45%): the face flux is packed by variable pairs and the
+// face buffers hold quads (FP16 increments, stage 2: 695 -> 604 instructions
+// per cell), and the prologue's planes are loaded three at a time. Per launch,
+// stages 1 to 3: FP16 increments 1024 x 1024 x 256 7.26 -> 7.02 ms, FP32
+// 512 x 512 x 256 1.96 -> 1.78 ms, 32^3 18.6 -> 16.8 us. Measured and not
+// better: a split barrier with three face buffers (FP32 1.83 ms, FP16
+// increments 7.9: the waits' polling costs issue slots), two rows per warp in
+// eight warps of 255 registers (7.12 and 1.75 ms, FP16 6% slower).
+//
 // In the increment modes the input q_s is read as RN32(q^n + d_s) (d_s from
 // stage 2 on), stages 1 and 2 store the 16-bit increment
 // d_{s+1} = RN16(w [(q_s - q^n) + dt L]) into `out`, and stage 3 stores the
@@ -1767,7 +1814,7 @@ constexpr int FLUX_MAXREG = sizeof(C) == 8 ? 224 : 128;
 template <int mode, int ORD, bool VISC>
 __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ sig, const QBIn qn,
                                           const Fout<5> out, const QBOut outb, const Frhs rhs,
-                                          const Fout<5> base_out, const Geom g, C gamma, C half_inv_dx,
+                                          const Fout<5> base_out, const Geom g, C gamma, C sg, C half_inv_dx,
                                           const Scalars *sc, double *blockmax, int *err, const C *W,
                                           const C *J, int zc, int cz0, C mu, C lamv, const BlockPos bp)
 {
@@ -1799,8 +1846,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
     auto fin = [&](int u) -> const S * { return u < 5 ? reinterpret_cast<const S *>(qin.b[u]) : sig; };
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2 *P = reinterpret_cast<C2 *>(smem_raw);        // [RING][3][PH][PW]
-    C *FXb = reinterpret_cast<C *>(P + RING * TILE2); // [2][5][TY][TX+1]
-    C *FYb = FXb + 2 * NFX;                           // [2][5][TY+1][TX]
+    C *FB = reinterpret_cast<C *>(P + RING * TILE2);  // [2][NFACE]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int x0 = bp.x * TX, y0 = bp.y * TY;
     const int cz = cz0 + bp.z;  // z-chunk (a launch may cover chunks cz0.. only)
@@ -1811,7 +1857,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
     const idx pl = (idx)g.plane;
     const idx own = (idx)(j * g.nx + i);
     const int tcell = (w + 3) * PW + lane + 3;  // this row-warp lane's cell in a tile
-    const C gm1 = gamma - C(1);
+    const Gas gas = {gamma - C(1), sg};
     FaceFlag bad = FaceFlag(kFaceMin ? 1 : 0);  // face states with rho <= 0 or p <= 0 (warning)
     bool nonfinite = false; // a non-finite output (error)
     // ring slot offsets (in pairs) of planes k-2..k+4 in iteration k, rotated
@@ -1838,28 +1884,44 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
         }
     }
 
-    // planes k0 - 3..k0 + 2, loaded and stored directly (index mapping in z,
-    // jet blend below an inflow face)
+    // planes k0 - 3..k0 + 2, loaded (several planes' loads in flight: each
+    // would cost a latency of its own) and stored directly, with the index
+    // mapping in z and the jet blend below an inflow face
+    constexpr int PLN = sizeof(C) == 8 ? 2 : 3;
 #pragma unroll 1
-    for (int kk = k0 - 3; kk < k0 + 3; kk++) {
-        C2 *T = P + (kk - k0 + 3) * TILE2;
-        const idx zb = (idx)zmap(kk, g) * pl;
-        const bool blend = kk < 0 && g.bc[4] == BC_INFLOW;
+    for (int kp = k0 - 3; kp < k0 + 3; kp += PLN) {
+        QRaw v0[PLN][LPT][5];
+        S v5[PLN][LPT];
 #pragma unroll
-        for (int r = 0; r < LPT; r++)
-            if ((kR0 && r == 0) || soff[r] >= 0) {
-                C v[6];
-                const idx c = ck(zb + goff[r], g.n);
+        for (int m = 0; m < PLN; m++) {
+            const idx zb = (idx)zmap(kp + m, g) * pl;
 #pragma unroll
-                for (int u = 0; u < 5; u++) v[u] = cvq<HASD>(ldq_raw(u, c));
-                v[5] = ldc(sig + c);
-                if (blend) {
-                    C wf = C(1) - W[ck(goff[r], g.plane)];
+            for (int r = 0; r < LPT; r++)
+                if ((kR0 && r == 0) || soff[r] >= 0) {
+                    const idx c = ck(zb + goff[r], g.n);
 #pragma unroll
-                    for (int u = 0; u < 5; u++) v[u] = wf * v[u] + J[(idx)u * pl + ck(goff[r], g.plane)];
+                    for (int u = 0; u < 5; u++) v0[m][r][u] = ldq_raw(u, c);
+                    v5[m][r] = ldr(sig + c);
                 }
-                st_cell(T, cks(soff[r], PH * PW), pset(v[0], v[1]), pset(v[2], v[3]), pset(v[4], v[5]));
-            }
+        }
+#pragma unroll
+        for (int m = 0; m < PLN; m++) {
+            C2 *T = P + (kp + m - k0 + 3) * TILE2;
+            const bool blend = kp + m < 0 && g.bc[4] == BC_INFLOW;
+#pragma unroll
+            for (int r = 0; r < LPT; r++)
+                if ((kR0 && r == 0) || soff[r] >= 0) {
+                    C v[5];
+#pragma unroll
+                    for (int u = 0; u < 5; u++) v[u] = cvq<HASD>(v0[m][r][u]);
+                    if (blend) {
+                        C wf = C(1) - W[ck(goff[r], g.plane)];
+#pragma unroll
+                        for (int u = 0; u < 5; u++) v[u] = wf * v[u] + J[(idx)u * pl + ck(goff[r], g.plane)];
+                    }
+                    st_cell(T, cks(soff[r], PH * PW), pset(v[0], v[1]), pset(v[2], v[3]), pset(v[4], C(cv(v5[m][r]))));
+                }
+        }
     }
 
     // plane kk >= k0 + 3 of the pipeline: FP32/FP64 storage copies with
@@ -1921,7 +1983,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
     }
     C smax = C(0);  // running wave-speed maximum (FP32 here: FP64 is slow on this GPU)
 
-    C Fzm[5], Fzp[5];
+    Flux Fzm, Fzp;
     // planes k and k + 1 at a row-warp lane's cell before iteration k: the
     // z-stencils of consecutive planes share them, so each iteration loads
     // four of its six points (shared loads are the flux kernel's most
@@ -1931,7 +1993,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
     // row) of the last plane: the divergence of that plane takes them from
     // registers and only the faces of its neighbours from the face buffers
     constexpr bool kOwnFaces = sizeof(C) == 4;
-    C Fxo[5], Fyo[5];
+    Flux Fxo, Fyo;
     C2 zq[2][3];
     if (!VISC && rowwarp) {
         ld_cell(P + ro[2], cks(tcell, PH * PW), zq[0][0], zq[0][1], zq[0][2]);  // plane k0 - 1
@@ -1946,22 +2008,25 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
     // plane k combines in the next iteration, so none is loaded twice.
     C2 cc[3];
     auto finish = [&](int kk) {
-        const C *FX = FXb + (kk & 1) * NFX;
-        const C *FY = FYb + (kk & 1) * NFY;
+        const C *FX = FB + (kk & 1) * NFACE, *FY = FX + 5 * NFX;
         idx c = ck((idx)kk * pl + own, g.n);
-        C Lv[5];
-#pragma unroll
-        for (int u = 0; u < 5; u++) {
-            // the faces above and right of the cell from the buffers, the two
-            // below and left of it computed by this lane (Fxo, Fyo; FP64
-            // arithmetic reads them back, its extra registers would spill)
-            const C fxl = kOwnFaces ? Fxo[u] : FX[cks((u * TY + w) * (TX + 1) + lane, NFX)];
-            const C fyl = kOwnFaces ? Fyo[u] : FY[cks((u * (TY + 1) + w) * TX + lane, NFY)];
-            C dfx = FX[cks((u * TY + w) * (TX + 1) + lane + 1, NFX)] - fxl;
-            C dfy = FY[cks((u * (TY + 1) + w + 1) * TX + lane, NFY)] - fyl;
-            C dfz = Fzp[u] - Fzm[u];
-            Lv[u] = -((dfx + dfy) + dfz) * half_inv_dx;
+        // the faces above and right of the cell from the buffers, the two
+        // below and left of it computed by this lane (Fxo, Fyo; FP64
+        // arithmetic reads them back, its extra registers would spill)
+        Flux xr, yr, xl, yl;
+        ld_face(FX, NFX, cks(w * (TX + 1) + lane + 1, NFX), xr);
+        ld_face(FY, NFY, cks((w + 1) * TX + lane, NFY), yr);
+        if (kOwnFaces) {
+            xl = Fxo;
+            yl = Fyo;
+        } else {
+            ld_face(FX, NFX, cks(w * (TX + 1) + lane, NFX), xl);
+            ld_face(FY, NFY, cks(w * TX + lane, NFY), yl);
         }
+        const C2 nh = bcast(-half_inv_dx);
+        const C2 La = pmul(padd(padd(psub(xr.a, xl.a), psub(yr.a, yl.a)), psub(Fzp.a, Fzm.a)), nh);
+        const C2 Lb = pmul(padd(padd(psub(xr.b, xl.b), psub(yr.b, yl.b)), psub(Fzp.b, Fzm.b)), nh);
+        const C Lv[5] = {La.x, La.y, Lb.x, Lb.y, -(((xr.e - xl.e) + (yr.e - yl.e)) + (Fzp.e - Fzm.e)) * half_inv_dx};
         if (mode == FLUX_RHS) {
 #pragma unroll
             for (int u = 0; u < 5; u++) rhs.p[u][c] = Lv[u];
@@ -1980,7 +2045,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
             if constexpr (kInc) {
 #pragma unroll
                 for (int u = 0; u < 5; u++) {
-                    const C inc = w32 * ((qsv[u] - qb[u]) + dt32 * Lv[u]);
+                    const C inc = mode == FLUX_STAGE1 ? dt32 * Lv[u] : w32 * ((qsv[u] - qb[u]) + dt32 * Lv[u]);
                     if (mode == FLUX_STAGE3)
                         o[u] = stc(outb0 + u * fs + c, qb[u] + inc);  // q^n+1 in FP32
                     else
@@ -1991,19 +2056,19 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
             }
             nonfinite |= !isfinite((o[0] + o[1]) + (o[2] + o[3]) + o[4]);
             if (mode == FLUX_STAGE3) {
-                C sp = cell_speed(o[0], o[1], o[2], o[3], o[4], gamma, gm1);
+                C sp = cell_speed(o[0], o[1], o[2], o[3], o[4], gamma, gas.gm1);
                 smax = (sp > smax || sp != sp) ? sp : smax;
             }
         }
     };
 
+#pragma unroll kUnroll
     for (int k = k0 - 1; k < k1; k++) {
         const bool more = k + 4 <= k1 + 2;  // plane k + 4 feeds the z-faces
         if (more) fetch(k + 4, P + ro[6]);
         const C2 *T = P + ro[2];  // plane k
-        C *FX = FXb + (k & 1) * NFX;
-        C *FY = FYb + (k & 1) * NFY;
-        C F[5];
+        C *FX = FB + (k & 1) * NFACE, *FY = FX + 5 * NFX;
+        Flux F;
         const C2 *Tm = P + ro[1], *Tp = P + ro[3];  // planes k - 1, k + 1 (viscous terms)
         const C inv_dx = C(2) * half_inv_dx;
         // viscous x-face between tile cells a and a + 1 (same row)
@@ -2025,8 +2090,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
                     for (int u = 0; u < 5; u++) qnv[u] = __ldg(kInc ? qn0 + u * fs + c : qn.p[u] + c);
                 }
             }
-#pragma unroll
-            for (int u = 0; u < 5; u++) Fzm[u] = Fzp[u];
+            Fzm = Fzp;
             C2 sz[6][3];  // z-stencil: planes k - 2..k + 3 at this cell
 #pragma unroll
             for (int m = 0; m < 6; m++) {
@@ -2044,7 +2108,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
                     zq[1][p] = sz[4][p];
                 }
             }
-            face_from_stencil<2, ORD>(sz, gamma, gm1, Fzp, bad);  // z-face k + 1/2
+            face_from_stencil<2, ORD>(sz, gas, Fzp, bad);  // z-face k + 1/2
             cc[0] = sz[2][0];  // plane k at this cell
             cc[1] = sz[2][1];
             cc[2] = sz[2][2];
@@ -2056,34 +2120,26 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
             }
             if (k >= k0) {
                 // x-face at the low side of cell `lane` of row w (tile cells lane-3..lane+2)
-                tile_face_c<0, ORD>(T, (w + 3) * PW + lane, 1, cc, gamma, gm1, F, bad);
+                tile_face_c<0, ORD>(T, (w + 3) * PW + lane, 1, cc, gas, F, bad);
                 if constexpr (VISC) visc_x((w + 3) * PW + lane + 2);
-#pragma unroll
-                for (int u = 0; u < 5; u++) {
-                    FX[cks((u * TY + w) * (TX + 1) + lane, NFX)] = F[u];
-                    if constexpr (kOwnFaces) Fxo[u] = F[u];
-                }
+                st_face(FX, NFX, cks(w * (TX + 1) + lane, NFX), F);
+                if constexpr (kOwnFaces) Fxo = F;
                 // y-face below row w in column lane (tile rows w-3..w+2)
-                tile_face_c<1, ORD>(T, w * PW + lane + 3, PW, cc, gamma, gm1, F, bad);
+                tile_face_c<1, ORD>(T, w * PW + lane + 3, PW, cc, gas, F, bad);
                 if constexpr (VISC) visc_y((w + 2) * PW + lane + 3);
-#pragma unroll
-                for (int u = 0; u < 5; u++) {
-                    FY[cks((u * (TY + 1) + w) * TX + lane, NFY)] = F[u];
-                    if constexpr (kOwnFaces) Fyo[u] = F[u];
-                }
+                st_face(FY, NFY, cks(w * TX + lane, NFY), F);
+                if constexpr (kOwnFaces) Fyo = F;
             }
         } else if (k >= k0) {
             // y-face above the last row, column lane
-            tile_face<1, ORD>(T, TY * PW + lane + 3, PW, gamma, gm1, F, bad);
+            tile_face<1, ORD>(T, TY * PW + lane + 3, PW, gas, F, bad);
             if constexpr (VISC) visc_y((TY + 2) * PW + lane + 3);
-#pragma unroll
-            for (int u = 0; u < 5; u++) FY[cks((u * (TY + 1) + TY) * TX + lane, NFY)] = F[u];
+            st_face(FY, NFY, cks(TY * TX + lane, NFY), F);
             if (lane < TY) {
                 // x-face at the high end of row `lane`
-                tile_face<0, ORD>(T, (lane + 3) * PW + TX, 1, gamma, gm1, F, bad);
+                tile_face<0, ORD>(T, (lane + 3) * PW + TX, 1, gas, F, bad);
                 if constexpr (VISC) visc_x((lane + 3) * PW + TX + 2);
-#pragma unroll
-                for (int u = 0; u < 5; u++) FX[cks((u * TY + lane) * (TX + 1) + TX, NFX)] = F[u];
+                st_face(FX, NFX, cks(lane * (TX + 1) + TX, NFX), F);
             }
         }
         if (more) land(P + ro[6]);
@@ -2107,10 +2163,10 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
 template <int mode, int ORD, bool VISC>
 __global__ void __maxnreg__(FLUX_MAXREG)
     k_flux(QIn qin, const S *__restrict__ sig, QBIn qn, Fout<5> out, QBOut outb, Frhs rhs, Fout<5> base_out,
-           Geom g, C gamma, C half_inv_dx, const Scalars *sc, double *blockmax, int *err, const C *W,
+           Geom g, C gamma, C sg, C half_inv_dx, const Scalars *sc, double *blockmax, int *err, const C *W,
            const C *J, int zc, int cz0, C mu, C lamv)
 {
-    flux_body<mode, ORD, VISC>(qin, sig, qn, out, outb, rhs, base_out, g, gamma, half_inv_dx, sc, blockmax, err,
+    flux_body<mode, ORD, VISC>(qin, sig, qn, out, outb, rhs, base_out, g, gamma, sg, half_inv_dx, sc, blockmax, err,
                                W, J, zc, cz0, mu, lamv, BlockPos::of_launch());
 }
 
@@ -2616,7 +2672,7 @@ struct FluxInst {
     Fout<5> out;
     QBOut outb;
     Geom g;
-    C gamma, half_inv_dx, mu, lamv;
+    C gamma, sg, half_inv_dx, mu, lamv;
     const Scalars *sc;
     double *blockmax;
     int *err;
@@ -2690,7 +2746,7 @@ __global__ void __maxnreg__(FLUX_MAXREG) k_flux_group(const __grid_constant__ Gr
     const Frhs none_rhs = {};
     const Fout<5> none_base = {};
     flux_body<mode, ORD, VISC>(d.qin, d.sig, d.qn, d.out, d.outb, none_rhs, none_base, d.g, d.gamma,
-                               d.half_inv_dx, d.sc, d.blockmax, d.err, d.W, d.J, d.zc, 0, d.mu, d.lamv,
+                               d.sg, d.half_inv_dx, d.sc, d.blockmax, d.err, d.W, d.J, d.zc, 0, d.mu, d.lamv,
                                BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy));
 }
 
@@ -2853,7 +2909,8 @@ cudaError_t launch_flux(const Geom &g, const Phys &p, const Tiles &t, const Infl
         dim3 gr = grid_of(g, TX, TY, t.zc_flux);
         const int cz0 = t.z_begin / t.zc_flux;
         if (t.z_end > 0) gr.z = (t.z_end - t.z_begin + t.zc_flux - 1) / t.zc_flux;
-        kern<<<gr, NT, smem, st>>>(fi, (const S *)sig, fn, fo, fob, fr, fb, g, C(p.gamma), C(0.5 / p.dx), sc,
+        kern<<<gr, NT, smem, st>>>(fi, (const S *)sig, fn, fo, fob, fr, fb, g, C(p.gamma),
+                                   C(sqrt(p.gamma * (p.gamma - 1.0))), C(0.5 / p.dx), sc,
                                    blockmax, err, (const C *)in.W, (const C *)in.J, t.zc_flux, cz0, C(p.mu),
                                    C(p.zeta - 2.0 * p.mu / 3.0));
         e = cudaGetLastError();
@@ -3012,6 +3069,7 @@ cudaError_t launch_flux_group(const FluxCall *calls, int n, int mode, cudaStream
             }
             d.g = c.g;
             d.gamma = C(c.p.gamma);
+            d.sg = C(sqrt(c.p.gamma * (c.p.gamma - 1.0)));
             d.half_inv_dx = C(0.5 / c.p.dx);
             d.mu = C(c.p.mu);
             d.lamv = C(c.p.zeta - 2.0 * c.p.mu / 3.0);
