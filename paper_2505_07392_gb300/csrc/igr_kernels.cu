@@ -365,9 +365,9 @@ struct Flux {
     C2 a, b;
     C e;
 };
-// gas constants of the flux: gamma - 1 and sqrt(gamma (gamma - 1))
+// gas constants of the flux: gamma and gamma - 1
 struct Gas {
-    C gm1, sg;
+    C gamma, gm1;
 };
 template <int D>
 __device__ __forceinline__ void lf_flux2(const C2 (&L)[3], const C2 (&R)[3], const Gas gas, Flux &G, FaceFlag &bad)
@@ -375,14 +375,13 @@ __device__ __forceinline__ void lf_flux2(const C2 (&L)[3], const C2 (&R)[3], con
     const C mL = D == 0 ? L[0].y : D == 1 ? L[1].x : L[1].y, mR = D == 0 ? R[0].y : D == 1 ? R[1].x : R[1].y;
     const C rL = rcp(L[0].x), rR = rcp(R[0].x);
     const C uL = mL * rL, uR = mR * rR;
-    // e = p / (gamma - 1), c = sqrt(gamma p / rho) = sg sqrt(e / rho)
-    const C eL = L[2].x - C(0.5) * ((L[0].y * L[0].y + L[1].x * L[1].x + L[1].y * L[1].y) * rL);
-    const C eR = R[2].x - C(0.5) * ((R[0].y * R[0].y + R[1].x * R[1].x + R[1].y * R[1].y) * rR);
-    flag_face(bad, L[0].x, R[0].x, eL, eR);
-    const C aL = fabs(uL) + gas.sg * sqrt_c(eL * rL);
-    const C aR = fabs(uR) + gas.sg * sqrt_c(eR * rR);
+    const C pL = gas.gm1 * (L[2].x - C(0.5) * ((L[0].y * L[0].y + L[1].x * L[1].x + L[1].y * L[1].y) * rL));
+    const C pR = gas.gm1 * (R[2].x - C(0.5) * ((R[0].y * R[0].y + R[1].x * R[1].x + R[1].y * R[1].y) * rR));
+    flag_face(bad, L[0].x, R[0].x, pL, pR);
+    const C aL = fabs(uL) + sqrt_c(gas.gamma * pL * rL);
+    const C aR = fabs(uR) + sqrt_c(gas.gamma * pR * rR);
     const C lam = fmax(aL, aR);  // a NaN speed comes with a flagged face
-    const C PL = gas.gm1 * eL + L[2].y, PR = gas.gm1 * eR + R[2].y;
+    const C PL = pL + L[2].y, PR = pR + R[2].y;
     const C2 nl = bcast(-lam);
     C fx = L[0].y * uL + R[0].y * uR, fy = L[1].x * uL + R[1].x * uR, fz = L[1].y * uL + R[1].y * uR;
     if (D == 0) fx += PL + PR;
@@ -837,12 +836,10 @@ __device__ __forceinline__ void cp_one(unsigned dst, const S *src)
 // term. 1/rho and sigma of plane k sit in a shared tile with a halo of 1;
 // the z-neighbours stay in registers.
 //
-// The faces are summed without the common factor hb = beta / 2,
-//   C_f = 1/rho_i + 1/rho_nb, D = 1/rho_i + hb sum C_f, N = b + hb sum C_f s_nb,
-// so no factor per face is held or multiplied, and the z-face below a cell is
-// the face above the cell of the last plane, kept from there. Across a
-// dropped face the neighbour's 1/rho is taken as -1/rho_i and its Sigma as 0:
-// C_f is then exactly 0.
+// The face factors c_f = hb (1/rho_i + 1/rho_nb), hb = beta / 2, take one
+// constant: across a dropped face the neighbour's 1/rho is taken as -1/rho_i
+// and its Sigma as 0, so that c_f is exactly 0. The z-face below a cell is the
+// face above the cell of the last plane, kept from there.
 //
 // colour >= 0 makes it one half of a red-black Gauss-Seidel sweep, in place
 // (s_in == s_out): only the cells with (i + j + k) % 2 == colour change.
@@ -852,8 +849,8 @@ __device__ __forceinline__ void cp_one(unsigned dst, const S *src)
 // the updated colour feed only results that are discarded.
 
 // The update of two cells: rc their 1/rho, bv their source; r*, s* the
-// neighbours' 1/rho and Sigma in x and y; zm, zp the z-faces below and above,
-// sm, sp Sigma there. Packed FP32x2 operations (FP64: two scalar ones).
+// neighbours' 1/rho and Sigma in x and y; zm, zp the factors of the z-faces
+// below and above, sm, sp Sigma there. Packed FP32x2 operations (FP64: two scalar ones).
 __device__ __forceinline__ float2 pquot(float2 a, float2 b) { return pmul(a, make_float2(rcp(b.x), rcp(b.y))); }
 __device__ __forceinline__ double2 pquot(double2 a, double2 b)
 {
@@ -862,15 +859,17 @@ __device__ __forceinline__ double2 pquot(double2 a, double2 b)
 __device__ __forceinline__ C2 jacobi2(C2 rc, C2 rxm, C2 rxp, C2 rym, C2 ryp, C2 zm, C2 zp, C2 sxm, C2 sxp, C2 sym,
                                       C2 syp, C2 sm, C2 sp, C2 bv, C hb)
 {
-    const C2 c0 = padd(rc, rxm), c1 = padd(rc, rxp), c2 = padd(rc, rym), c3 = padd(rc, ryp);
-    const C2 sum = padd(padd(padd(c0, c1), padd(c2, c3)), padd(zm, zp));
+    const C2 h = bcast(hb);
+    const C2 c0 = pmul(h, padd(rc, rxm)), c1 = pmul(h, padd(rc, rxp));
+    const C2 c2 = pmul(h, padd(rc, rym)), c3 = pmul(h, padd(rc, ryp));
+    const C2 diag = padd(padd(padd(padd(padd(padd(rc, c0), c1), c2), c3), zm), zp);
     C2 off = pmul(c0, sxm);
     off = pfma(c1, sxp, off);
     off = pfma(c2, sym, off);
     off = pfma(c3, syp, off);
     off = pfma(zm, sm, off);
     off = pfma(zp, sp, off);
-    return pquot(pfma(bcast(hb), off, bv), pfma(bcast(hb), sum, rc));
+    return pquot(padd(bv, off), diag);
 }
 
 // Raw values are copied to shared memory JRING - 1 planes ahead, each by the
@@ -959,7 +958,7 @@ __device__ __forceinline__ void jacobi_quads(const S *__restrict__ q, const S *_
             cv4(s0r[r], s0[r]);
 #pragma unroll
             for (int h = 0; h < 2; h++)
-                zm[r][h] = padd(pset(r0[r][2 * h], r0[r][2 * h + 1]), pset(rm[2 * h], rm[2 * h + 1]));
+                zm[r][h] = pmul(bcast(hb), padd(pset(r0[r][2 * h], r0[r][2 * h + 1]), pset(rm[2 * h], rm[2 * h + 1])));
             if (k0 == 0 && g.bc[4] != BC_PERIODIC) {
 #pragma unroll
                 for (int c = 0; c < VX; c++) sm[r][c] = C(0);
@@ -1062,7 +1061,8 @@ __device__ __forceinline__ void jacobi_quads(const S *__restrict__ q, const S *_
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
                     const int c = 2 * h;
-                    const C2 rc = pset(r0[r][c], r0[r][c + 1]), zp = padd(rc, pset(rp[r][c], rp[r][c + 1]));
+                    const C2 rc = pset(r0[r][c], r0[r][c + 1]);
+                    const C2 zp = pmul(bcast(hb), padd(rc, pset(rp[r][c], rp[r][c + 1])));
                     const C2 v = jacobi2(rc, pset(rx[c], rx[c + 1]), pset(rx[c + 2], rx[c + 3]),
                                          pset(ry0[c], ry0[c + 1]), pset(ry1[c], ry1[c + 1]), zm[r][h], zp,
                                          pset(sx[c], sx[c + 1]), pset(sx[c + 2], sx[c + 3]),
@@ -1138,7 +1138,7 @@ __device__ __forceinline__ void jacobi_pairs(const S *__restrict__ q, const S *_
     conv(r0, s0);
     own(k0 + 1);
     rest(k0);
-    zm = padd(r0, rm);
+    zm = pmul(bcast(hb), padd(r0, rm));
     if (k0 == 0 && g.bc[4] != BC_PERIODIC) zm = sm = bcast(C(0));
     for (int k = k0; k < k1; k++) {
         C *R = R2 + ((k - k0) & 1) * TILEP, *SG = S2 + ((k - k0) & 1) * TILEP;
@@ -1163,7 +1163,7 @@ __device__ __forceinline__ void jacobi_pairs(const S *__restrict__ q, const S *_
             rp = pset(-r0.x, -r0.y);
             sp = bcast(C(0));
         }
-        const C2 zp = padd(r0, rp);
+        const C2 zp = pmul(bcast(hb), padd(r0, rp));
         const C *Rc = R + t.pos, *Sc = SG + t.pos;
         const C2 v = jacobi2(r0, pset(Rc[-1], Rc[PPITCH - 1]), pset(Rc[1], Rc[PPITCH + 1]),
                              pset(Rc[-PPITCH], r0.x), pset(r0.y, Rc[2 * PPITCH]), zm, zp,
@@ -1814,7 +1814,7 @@ constexpr int FLUX_MAXREG = sizeof(C) == 8 ? 224 : 128;
 template <int mode, int ORD, bool VISC>
 __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ sig, const QBIn qn,
                                           const Fout<5> out, const QBOut outb, const Frhs rhs,
-                                          const Fout<5> base_out, const Geom g, C gamma, C sg, C half_inv_dx,
+                                          const Fout<5> base_out, const Geom g, C gamma, C half_inv_dx,
                                           const Scalars *sc, double *blockmax, int *err, const C *W,
                                           const C *J, int zc, int cz0, C mu, C lamv, const BlockPos bp)
 {
@@ -1857,7 +1857,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
     const idx pl = (idx)g.plane;
     const idx own = (idx)(j * g.nx + i);
     const int tcell = (w + 3) * PW + lane + 3;  // this row-warp lane's cell in a tile
-    const Gas gas = {gamma - C(1), sg};
+    const Gas gas = {gamma, gamma - C(1)};
     FaceFlag bad = FaceFlag(kFaceMin ? 1 : 0);  // face states with rho <= 0 or p <= 0 (warning)
     bool nonfinite = false; // a non-finite output (error)
     // ring slot offsets (in pairs) of planes k-2..k+4 in iteration k, rotated
@@ -2163,10 +2163,10 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
 template <int mode, int ORD, bool VISC>
 __global__ void __maxnreg__(FLUX_MAXREG)
     k_flux(QIn qin, const S *__restrict__ sig, QBIn qn, Fout<5> out, QBOut outb, Frhs rhs, Fout<5> base_out,
-           Geom g, C gamma, C sg, C half_inv_dx, const Scalars *sc, double *blockmax, int *err, const C *W,
+           Geom g, C gamma, C half_inv_dx, const Scalars *sc, double *blockmax, int *err, const C *W,
            const C *J, int zc, int cz0, C mu, C lamv)
 {
-    flux_body<mode, ORD, VISC>(qin, sig, qn, out, outb, rhs, base_out, g, gamma, sg, half_inv_dx, sc, blockmax, err,
+    flux_body<mode, ORD, VISC>(qin, sig, qn, out, outb, rhs, base_out, g, gamma, half_inv_dx, sc, blockmax, err,
                                W, J, zc, cz0, mu, lamv, BlockPos::of_launch());
 }
 
@@ -2672,7 +2672,7 @@ struct FluxInst {
     Fout<5> out;
     QBOut outb;
     Geom g;
-    C gamma, sg, half_inv_dx, mu, lamv;
+    C gamma, half_inv_dx, mu, lamv;
     const Scalars *sc;
     double *blockmax;
     int *err;
@@ -2746,7 +2746,7 @@ __global__ void __maxnreg__(FLUX_MAXREG) k_flux_group(const __grid_constant__ Gr
     const Frhs none_rhs = {};
     const Fout<5> none_base = {};
     flux_body<mode, ORD, VISC>(d.qin, d.sig, d.qn, d.out, d.outb, none_rhs, none_base, d.g, d.gamma,
-                               d.sg, d.half_inv_dx, d.sc, d.blockmax, d.err, d.W, d.J, d.zc, 0, d.mu, d.lamv,
+                               d.half_inv_dx, d.sc, d.blockmax, d.err, d.W, d.J, d.zc, 0, d.mu, d.lamv,
                                BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy));
 }
 
@@ -2909,8 +2909,7 @@ cudaError_t launch_flux(const Geom &g, const Phys &p, const Tiles &t, const Infl
         dim3 gr = grid_of(g, TX, TY, t.zc_flux);
         const int cz0 = t.z_begin / t.zc_flux;
         if (t.z_end > 0) gr.z = (t.z_end - t.z_begin + t.zc_flux - 1) / t.zc_flux;
-        kern<<<gr, NT, smem, st>>>(fi, (const S *)sig, fn, fo, fob, fr, fb, g, C(p.gamma),
-                                   C(sqrt(p.gamma * (p.gamma - 1.0))), C(0.5 / p.dx), sc,
+        kern<<<gr, NT, smem, st>>>(fi, (const S *)sig, fn, fo, fob, fr, fb, g, C(p.gamma), C(0.5 / p.dx), sc,
                                    blockmax, err, (const C *)in.W, (const C *)in.J, t.zc_flux, cz0, C(p.mu),
                                    C(p.zeta - 2.0 * p.mu / 3.0));
         e = cudaGetLastError();
@@ -3069,7 +3068,6 @@ cudaError_t launch_flux_group(const FluxCall *calls, int n, int mode, cudaStream
             }
             d.g = c.g;
             d.gamma = C(c.p.gamma);
-            d.sg = C(sqrt(c.p.gamma * (c.p.gamma - 1.0)));
             d.half_inv_dx = C(0.5 / c.p.dx);
             d.mu = C(c.p.mu);
             d.lamv = C(c.p.zeta - 2.0 * c.p.mu / 3.0);
