@@ -239,9 +239,11 @@ igr_status igr_rhs(igr_ctx *ctx, const void *q, const void *sigma, void *rhs, ig
  * values; outputs may not alias inputs); grad_jet_w: host array of njets
  * doubles or NULL (synchronises when given). The first call allocates a
  * workspace of about (29 + 3 sweeps) n stored values plus 30 n arithmetic
- * values through the context's allocator. The scatter steps use atomics, so
- * FP32 results vary in the last bits from run to run. The increment modes
- * return IGR_ERR_UNSUPPORTED. */
+ * values through the context's allocator. In FP64,
+ * and in the other modes without jets, every adjoint is gathered in a fixed
+ * order and results are deterministic; with jets in FP32 arithmetic the
+ * faces and the source scatter by atomics, so results vary in the last bits
+ * from run to run. The increment modes return IGR_ERR_UNSUPPORTED. */
 igr_status igr_adjoint_step(igr_ctx *ctx, const void *q_n, const void *sigma_n,
                             const void *lam_q_np1, const void *lam_sigma_np1, void *lam_q_n,
                             void *lam_sigma_n, double *grad_jet_w, double dt, igr_dtype dtype);

@@ -1592,7 +1592,7 @@ static igr_status ensure_adjoint(igr_ctx *c)
     for (void **p : one)
         if (s == IGR_OK) s = adj_alloc(c, p, n * cb);
     if (s == IGR_OK) s = adj_alloc(c, &c->adj.lamJ, 5 * (size_t)c->g.plane * cb);
-    if (s == IGR_OK) s = adj_alloc(c, (void **)&c->adj.gw, (size_t)(c->cfg.njets > 0 ? c->cfg.njets : 1) * sizeof(double));
+    if (s == IGR_OK) s = adj_alloc(c, (void **)&c->adj.gw, (size_t)(c->cfg.njets > 0 ? c->cfg.njets : 1) * (1 + ADJ_JET_BLOCKS) * sizeof(double));
     if (s == IGR_OK) s = adj_alloc(c, (void **)&c->adj.sc, sizeof(Scalars));
     if (s != IGR_OK) return s;
     CU(c, cudaMemsetAsync(c->adj.sc, 0, sizeof(Scalars), c->st));
@@ -1647,32 +1647,51 @@ igr_status igr_adjoint_step(igr_ctx *c, const void *q_n, const void *sigma_n, co
             CU(c, cudaMemcpyAsync(it(st + 1, 0), it(st, S), n * sb, cudaMemcpyDeviceToDevice, c->st));
         }
     }
-    // reverse
-    void *lout = A.lout, *lqs = A.lqs, *lsig = A.lsig, *nl = A.nl;
-    CU(c, cudaMemcpyAsync(lout, lam_q_np1, 5 * n * cb, cudaMemcpyDeviceToDevice, c->st));
+    // reverse, stage by stage: `in` the adjoint of the stage's output, `out` that of its
+    // input (lq0 gathers that of the step's input), by gathering or, in FP32 arithmetic
+    // with jets, scattering (igr_kernels.cu says why). Scratch: once the faces are done,
+    // the buffer `free5` (5 n) and Lb (5 n) hold 1 / rho, the diagonal and, with mu, the
+    // nine gradient adjoints of the gathered source.
+    const bool gather = cb == 8 || c->cfg.njets == 0;
+    const void *in = lam_q_np1;
+    void *out = A.lqs, *free5 = A.lout, *lsig = A.lsig, *nl = A.nl;
+    auto at = [&](void *p, int f) { return (void *)((unsigned char *)p + (size_t)f * n * cb); };
     CU(c, cudaMemcpyAsync(lsig, lam_sigma_np1, n * cb, cudaMemcpyDeviceToDevice, c->st));
-    CU(c, cudaMemsetAsync(A.lq0, 0, 5 * n * cb, c->st));
     CU(c, cudaMemsetAsync(A.lamJ, 0, 5 * (size_t)c->g.plane * cb, c->st));
-    CU(c, cudaMemsetAsync(A.rb, 0, n * cb, c->st));
+    if (!gather) CU(c, cudaMemsetAsync(A.lq0, 0, 5 * n * cb, c->st));
+    void *r = at(A.Lb, 0), *diag = at(A.Lb, 1);
     for (int st = 2; st >= 0; st--) {
-        CU(c, o->adj_rk(lout, A.lq0, lqs, A.Lb, 5 * (long long)n, wst[st], dt, c->st));
-        CU(c, o->adj_rhs(c->g, c->p, inflow_of(c), qs[st], it(st, S), A.Lb, lqs, lsig, A.lamJ, c->st));
-        CU(c, cudaMemsetAsync(A.lb, 0, n * cb, c->st));
+        if (gather) {
+            CU(c, o->adj_rhs(c->g, c->p, inflow_of(c), qs[st], it(st, S), in, out, A.lq0, lsig, A.lamJ, wst[st], dt,
+                             st == 2, c->st));
+        } else {
+            CU(c, o->adj_rk(in, A.lq0, out, A.Lb, 5 * (long long)n, wst[st], dt, c->st));
+            CU(c, o->adj_rhs_scatter(c->g, c->p, inflow_of(c), qs[st], it(st, S), A.Lb, out, lsig, A.lamJ, c->st));
+        }
+        if (st < 2) free5 = (void *)in;  // (stage 3's `in` is the caller's)
+        CU(c, o->adj_diag(c->g, c->p, qs[st], r, diag, c->st));
         for (int k = S - 1; k >= 0; k--) {
-            CU(c, o->adj_jacobi(c->g, c->p, qs[st], it(st, k), it(st, k + 1), lsig, nl, A.lb, A.rb, A.mu, c->st));
+            CU(c, o->adj_jacobi(c->g, c->p, r, diag, it(st, k), it(st, k + 1), lsig, nl, A.lb, A.rb, k == S - 1,
+                                c->st));
             std::swap(lsig, nl);
         }
-        CU(c, o->adj_rho(c->g, qs[st], A.rb, lqs, c->st));
-        CU(c, o->adj_source(c->g, c->p, inflow_of(c), qs[st], A.lb, lqs, A.lamJ, c->st));
-        if (st == 0)  // the first stage reads q_n itself: lq0 += lqs
-            CU(c, o->adj_rk(lqs, A.lq0, lqs, A.Lb, 5 * (long long)n, 0.0, 0.0, c->st));
-        else
-            std::swap(lout, lqs);
+        if (gather) {
+            void *grads[9] = {at(free5, 0), at(free5, 1), at(free5, 2), at(free5, 3), at(free5, 4),
+                              at(A.Lb, 2),  at(A.Lb, 3),  at(A.Lb, 4),  A.mu};
+            CU(c, o->adj_source(c->g, c->p, inflow_of(c), qs[st], r, A.lb, A.rb, grads, out, A.lamJ, c->st));
+        } else {
+            CU(c, o->adj_rho(c->g, qs[st], A.rb, out, c->st));
+            CU(c, o->adj_source_scatter(c->g, c->p, inflow_of(c), qs[st], A.lb, out, A.lamJ, c->st));
+        }
+        if (st > 0) {
+            in = out;
+            out = free5;
+        }
     }
-    CU(c, cudaMemcpyAsync(lam_q_n, A.lq0, 5 * n * cb, cudaMemcpyDeviceToDevice, c->st));
+    // the first stage reads q_n itself
+    CU(c, o->adj_add(A.lq0, out, lam_q_n, 5 * (long long)n, c->st));
     CU(c, cudaMemcpyAsync(lam_sigma_n, lsig, n * cb, cudaMemcpyDeviceToDevice, c->st));
     if (grad_jet_w && c->cfg.njets > 0) {
-        CU(c, cudaMemsetAsync(A.gw, 0, c->cfg.njets * sizeof(double), c->st));
         CU(c, o->adj_jets(c->g, c->p, c->jets_dev, c->cfg.njets, A.lamJ, A.gw, c->st));
         std::vector<double> h(c->cfg.njets);
         CU(c, cudaMemcpyAsync(h.data(), A.gw, h.size() * sizeof(double), cudaMemcpyDeviceToHost, c->st));

@@ -153,26 +153,43 @@ struct Ops {
                               long long n, double dt, double w, cudaStream_t st);
 
     // ---- adjoint (all adjoint buffers in the arithmetic type) ----
+    // reverse of the stage combination (weight w) and of L(qs; sig), from the adjoint
+    // lout of the stage's output: lqs (5 n) = the adjoint of qs, lq0 += (1 - w) lout
+    // (first: =), lsig += the adjoint of sig, lamJ += that of the inflow tables (5 x plane)
+    cudaError_t (*adj_rhs)(const Geom &, const Phys &, const Inflow &, const void *qs, const void *sig,
+                           const void *lout, void *lqs, void *lq0, void *lsig, void *lamJ, double w, double dt,
+                           int first, cudaStream_t st);
+    // r = 1 / rho and the diagonal of the sweeps (FP64: its inverse)
+    cudaError_t (*adj_diag)(const Geom &, const Phys &, const void *q, void *r, void *diag, cudaStream_t st);
+    // one reversed Jacobi sweep s_k -> F: lsig (adjoint of F) -> nl (adjoint of s_k);
+    // lb += mu, rb += d/d(1/rho) (first: =)
+    cudaError_t (*adj_jacobi)(const Geom &, const Phys &, const void *r, const void *diag, const void *sk,
+                              const void *F, const void *lsig, void *nl, void *lb, void *rb, int first,
+                              cudaStream_t st);
+    // reverse of the IGR source and of 1 / rho: lb, rb -> lqs (rho, m), lamJ; grads: nine
+    // scratch arrays of n values
+    cudaError_t (*adj_source)(const Geom &, const Phys &, const Inflow &, const void *q, const void *r,
+                              const void *lb, const void *rb, void *const grads[9], void *lqs, void *lamJ,
+                              cudaStream_t st);
+    // out = a + b (n values)
+    cudaError_t (*adj_add)(const void *a, const void *b, void *out, long long n, cudaStream_t st);
+    // gw[n] = sum over the inflow face of s_n (rho_n lamJ_mz + rho_n w_n lamJ_E); gw holds
+    // njets (1 + ADJ_JET_BLOCKS) values, the sums and the blocks' shares
+    cudaError_t (*adj_jets)(const Geom &, const Phys &, const double *jets, int njets,
+                            const void *lamJ, double *gw, cudaStream_t st);
+    // ---- the scatter forms of the faces' and the source's reverse (by atomics)
     // lq0 += (1 - w) lout; lqs = w lout; Lb = w dt lout   (5 n values)
     cudaError_t (*adj_rk)(const void *lout, void *lq0, void *lqs, void *Lb, long long n5, double w,
                           double dt, cudaStream_t st);
-    // reverse of L(qs; sig): Lb -> lqs (5 fields), lsig, lamJ (5 x plane), by atomics
-    cudaError_t (*adj_rhs)(const Geom &, const Phys &, const Inflow &, const void *qs,
-                           const void *sig, const void *Lb, void *lqs, void *lsig, void *lamJ,
-                           cudaStream_t st);
-    // one reversed Jacobi sweep s_k -> F: lsig (in: adjoint of F) -> nl (adjoint
-    // of s_k); lb += mu; rb += d/d(1/rho); mu is scratch
-    cudaError_t (*adj_jacobi)(const Geom &, const Phys &, const void *q, const void *sk,
-                              const void *F, const void *lsig, void *nl, void *lb, void *rb,
-                              void *mu, cudaStream_t st);
-    // lqs[rho] -= rb / rho^2; rb = 0
+    // reverse of L(qs; sig): Lb -> lqs (5 fields), lsig, lamJ (5 x plane)
+    cudaError_t (*adj_rhs_scatter)(const Geom &, const Phys &, const Inflow &, const void *qs,
+                                   const void *sig, const void *Lb, void *lqs, void *lsig, void *lamJ,
+                                   cudaStream_t st);
+    // lqs[rho] -= rb / rho^2
     cudaError_t (*adj_rho)(const Geom &, const void *q, void *rb, void *lqs, cudaStream_t st);
-    // reverse of the IGR source: lb -> lqs (rho, m), lamJ, by atomics
-    cudaError_t (*adj_source)(const Geom &, const Phys &, const Inflow &, const void *q,
-                              const void *lb, void *lqs, void *lamJ, cudaStream_t st);
-    // gw[n] += sum over the inflow face of s_n (rho_n lamJ_mz + rho_n w_n lamJ_E)
-    cudaError_t (*adj_jets)(const Geom &, const Phys &, const double *jets, int njets,
-                            const void *lamJ, double *gw, cudaStream_t st);
+    // reverse of the IGR source: lb -> lqs (rho, m), lamJ
+    cudaError_t (*adj_source_scatter)(const Geom &, const Phys &, const Inflow &, const void *q,
+                                      const void *lb, void *lqs, void *lamJ, cudaStream_t st);
 
     // ---- diagnostics (FP64) ----
     // per-block partials (DIAG_PARTS doubles each) of the state's totals,
@@ -231,6 +248,9 @@ struct FluxCall {
     double *blockmax;
     int *err;
 };
+
+// blocks per jet of the adjoint's sum over the inflow face
+enum { ADJ_JET_BLOCKS = 32 };
 
 // instances per grouped launch: their descriptors travel as one kernel
 // parameter (at most 32 KB)

@@ -2325,12 +2325,24 @@ __global__ void __launch_bounds__(DIAG_NT) k_diag(const QB *__restrict__ q, cons
 }
 
 // ---------------------------------------------------------------- adjoint
-// Reverse of one stage (discrete adjoint with dt frozen). Simple kernels: one
-// thread per face or cell, grid-stride loops, and atomics where the forward
-// gathers (each reverse stencil scatters to the cells it read). Adjoint
-// values are in the arithmetic type C. Non-smooth points follow the forward's
-// branch: the LF speed max(aL, aR) sends its adjoint to the side the forward
-// took (aR on a tie), |u| takes sign(u) with sign(0) = 0.
+// Reverse of one stage (discrete adjoint with dt frozen). The faces and the
+// source send their adjoints to the cells that they read in one of two ways
+// (Ops::adj_rhs, Ops::adj_source and the scatter forms):
+//   gather   a cell sums what the faces and cells that read it send back, in a
+//            fixed order: deterministic, no atomics. Taken in FP64, and in
+//            FP32 arithmetic without jets.
+//   scatter  one thread per face or cell adds to the cells it read by atomics
+//            (36 per face and 36 per cell of the source). Kept in FP32
+//            arithmetic with jets, where it is 3.9 times slower (128^3, four
+//            jets: 10.0 ms against 2.6 for the step): a jet's gradient is a
+//            double summed from these FP32 values with cancellation, so
+//            another order of addition moves it by 1e-7, beyond what two runs
+//            of the scatter differ by (4e-8; near the inflow face its order
+//            hardly varies).
+// The reversed sweeps gather in both. Adjoint values are in the arithmetic
+// type C. Non-smooth points follow the forward's branch: the LF speed
+// max(aL, aR) sends its adjoint to the side the forward took (aR on a tie),
+// |u| takes sign(u) with sign(0) = 0.
 
 __device__ __forceinline__ void aadd(float *p, float v) { atomicAdd(p, v); }
 __device__ __forceinline__ void aadd(double *p, double v) { atomicAdd(p, v); }
@@ -2386,7 +2398,7 @@ __global__ void k_adj_rk(const C *lout, C *lq0, C *lqs, C *Lb, long long n5, C w
 // reverse of the physical flux along D at a face state v = (rho, m, E) and
 // Sigma s: Fb (adjoint of F) and ab (adjoint of |u_D| + c) into vb, sb
 template <int D>
-__device__ __forceinline__ void flux_rev(const C v[5], C s, const C Fb[5], C ab, C gamma, C vb[5], C &sb)
+__device__ __forceinline__ void flux_rev_at(const C v[5], C s, const C Fb[5], C ab, C gamma, C vb[5], C &sb)
 {
     C rho = v[0], E = v[4], r = C(1) / rho;
     C u[3] = {v[1] * r, v[2] * r, v[3] * r};
@@ -2440,7 +2452,7 @@ __device__ __forceinline__ C fwd_flux(const C v[5], C s, C gamma, C F[5])
 
 // one thread per face normal to D: face f sits between cells f-1 and f
 template <int D>
-__global__ void k_adj_rhs(const S *q, const S *sig, const C *Lb, C *lq, C *lsig, C *lamJ, Geom g, C gamma,
+__global__ void k_adj_rhs_scatter(const S *q, const S *sig, const C *Lb, C *lq, C *lsig, C *lamJ, Geom g, C gamma,
                           C inv_dx, const C *W, const C *J)
 {
     const int nf[3] = {g.nx + (D == 0), g.ny + (D == 1), g.nz + (D == 2)};
@@ -2496,8 +2508,8 @@ __global__ void k_adj_rhs(const S *q, const S *sig, const C *Lb, C *lq, C *lsig,
             lamb -= C(0.5) * (R[u] - L[u]) * Fb[u];
         }
         C sLb = C(0), sRb = C(0);
-        flux_rev<D>(L, L[5], FLb, aL > aR ? lamb : C(0), gamma, Lbv, sLb);
-        flux_rev<D>(R, R[5], FRb, aL > aR ? C(0) : lamb, gamma, Rbv, sRb);
+        flux_rev_at<D>(L, L[5], FLb, aL > aR ? lamb : C(0), gamma, Lbv, sLb);
+        flux_rev_at<D>(R, R[5], FRb, aL > aR ? C(0) : lamb, gamma, Rbv, sRb);
 #pragma unroll
         for (int m = 0; m < 6; m++) {
             int cc[3] = {c3[0], c3[1], c3[2]};
@@ -2513,77 +2525,17 @@ __global__ void k_adj_rhs(const S *q, const S *sig, const C *Lb, C *lq, C *lsig,
     }
 }
 
-// neighbour of cell (i,j,k) across face d (0:-x .. 5:+z); false on a
-// non-periodic domain boundary (no face term there)
-__device__ __forceinline__ bool nbr(const Geom &g, int i, int j, int k, int d, idx &out)
-{
-    int c[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz};
-    int ax = d >> 1;
-    c[ax] += (d & 1) ? 1 : -1;
-    if (c[ax] < 0 || c[ax] >= n[ax]) {
-        if (g.bc[d] != BC_PERIODIC) return false;
-        c[ax] = c[ax] < 0 ? c[ax] + n[ax] : c[ax] - n[ax];
-    }
-    out = ck(((idx)c[2] * (idx)g.ny + (idx)c[1]) * (idx)g.nx + (idx)c[0], g.n);
-    return true;
-}
-
-// mu = lambda / D_i, lb += mu
-__global__ void k_adj_jac_mu(const S *q, const C *lsig, C *mu, C *lb, Geom g, C beta)
-{
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < g.n;
-         t += (long long)gridDim.x * blockDim.x) {
-        int i = (int)(t % g.nx), j = (int)((t / g.nx) % g.ny), k = (int)(t / g.plane);
-        C ri = C(1) / ldc(q + t), diag = ri;
-        for (int d = 0; d < 6; d++) {
-            idx m;
-            if (nbr(g, i, j, k, d, m)) diag += beta * C(0.5) * (ri + C(1) / ldc(q + m));
-        }
-        C mv = lsig[t] / diag;
-        mu[t] = mv;
-        lb[t] += mv;
-    }
-}
-
-// gather form of the transposed sweep (the neighbour relation is symmetric):
-// nl_m = sum_i beta c_im mu_i; rb_m += mu_m (beta/2 sum s_nb - F_m (1 + beta nf/2))
-//                                  + sum_i mu_i beta/2 (s_m - F_i)
-__global__ void k_adj_jac_gather(const S *q, const S *sk, const S *F, const C *mu, C *nl, C *rb, Geom g,
-                                 C beta)
-{
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < g.n;
-         t += (long long)gridDim.x * blockDim.x) {
-        int i = (int)(t % g.nx), j = (int)((t / g.nx) % g.ny), k = (int)(t / g.plane);
-        C rm = C(1) / ldc(q + t), sm = ldc(sk + t), Fm = ldc(F + t), mum = mu[t];
-        C acc = C(0), ssum = C(0), rbm = C(0);
-        int nfc = 0;
-        for (int d = 0; d < 6; d++) {
-            idx n;
-            if (!nbr(g, i, j, k, d, n)) continue;
-            C rn = C(1) / ldc(q + n), mun = mu[n];
-            acc += beta * C(0.5) * (rm + rn) * mun;
-            ssum += ldc(sk + n);
-            nfc++;
-            rbm += mun * C(0.5) * beta * (sm - ldc(F + n));
-        }
-        rbm += mum * (C(0.5) * beta * ssum - Fm * (C(1) + C(0.5) * beta * C(nfc)));
-        nl[t] = acc;
-        rb[t] += rbm;
-    }
-}
-
 __global__ void k_adj_rho(const S *q, C *rb, C *lqs, long long n)
 {
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
          t += (long long)gridDim.x * blockDim.x) {
         C rho = ldc(q + t);
         lqs[t] -= rb[t] / (rho * rho);
-        rb[t] = C(0);
     }
 }
 
 // reverse of the source at one cell: lambda_b -> u at the 6 neighbours -> (rho, m) there
-__global__ void k_adj_source(const S *q, const C *lb, C *lq, C *lamJ, Geom g, C alpha, C inv2dx, const C *W,
+__global__ void k_adj_source_scatter(const S *q, const C *lb, C *lq, C *lamJ, Geom g, C alpha, C inv2dx, const C *W,
                              const C *J)
 {
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < g.n;
@@ -2622,28 +2574,560 @@ __global__ void k_adj_source(const S *q, const C *lb, C *lq, C *lamJ, Geom g, C 
     }
 }
 
-// gw[n] += sum over the inflow face of s_n (rho_n lamJ_mz + rho_n w_n lamJ_E); one block per jet
-__global__ void k_adj_jets(const double *jets, const C *lamJ, double *gw, int nx, int ny, double dx)
+// forward value of field u (0..4 conserved, 5 Sigma) at mapped in-plane
+// offset f and plane kk: index mapping in z plus the jet blend of the -z
+// inflow face
+__device__ __forceinline__ C val_col(const S *q, const S *sig, const Geom &g, const C *W, const C *J, idx f, int kk,
+                                     int u)
+{
+    const idx c = ck((idx)zmap(kk, g) * (idx)g.plane + f, g.n);
+    if (u == 5) return ldc(sig + c);
+    C v = ldc(q + ckl((size_t)u * (size_t)g.n + c, 5 * g.n));
+    if (kk < 0 && g.bc[4] == BC_INFLOW)
+        v = (C(1) - W[ck(f, g.plane)]) * v + J[ckl((size_t)u * (size_t)g.plane + f, 5 * g.plane)];
+    return v;
+}
+
+// a face state's primitives: 1 / rho, u, p and the sound speed
+struct Prim {
+    C r, u[3], p, c;
+};
+__device__ __forceinline__ Prim prim_of(const C (&v)[6], C gamma)
+{
+    Prim w;
+    w.r = C(1) / v[0];
+    C ke = C(0);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        w.u[a] = v[1 + a] * w.r;
+        ke += v[1 + a] * w.u[a];
+    }
+    w.p = (gamma - C(1)) * (v[4] - C(0.5) * ke);
+    w.c = sqrt(gamma * w.p * w.r);
+    return w;
+}
+
+// reverse of the physical flux along D at a face state v = (rho, m, E, Sigma)
+// with primitives w: Fb (adjoint of F) and the adjoints pb, rhob, uDb that
+// p, rho and u_D have besides (from the wave speed), added to vb
+template <int D>
+__device__ __forceinline__ void flux_rev(const C (&v)[6], const Prim &w, const C (&Fb)[5], C pb, C rhob, C uDb,
+                                         C gamma, C (&vb)[6])
+{
+    C ub[3] = {C(0), C(0), C(0)};
+    ub[D] = uDb + Fb[0] * v[0];
+    rhob += Fb[0] * w.u[D];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        vb[1 + a] += Fb[1 + a] * w.u[D];
+        ub[D] += Fb[1 + a] * v[1 + a];
+    }
+    const C Pb = Fb[1 + D] + Fb[4] * w.u[D];
+    ub[D] += Fb[4] * (v[4] + (w.p + v[5]));
+    pb += Pb;
+    vb[5] += Pb;
+    const C keb = -(gamma - C(1)) * pb;
+    vb[4] += Fb[4] * w.u[D] - keb;
+    C uu = C(0);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        ub[a] += keb * v[1 + a];
+        uu += w.u[a] * w.u[a];
+    }
+    rhob += keb * C(0.5) * uu;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const C mb = ub[a] * w.r;
+        vb[1 + a] += mb;
+        rhob -= mb * w.u[a];
+    }
+    vb[0] += rhob;
+}
+
+// Reverse of one face along D: from the six cells s it reads (cell, field)
+// and the adjoint Fb of its flux, the adjoints Lb, Rb of its two face values
+template <int D>
+__device__ __forceinline__ void face_rev(const C (&s)[6][6], const C (&Fb)[5], C gamma, C (&Lb)[6], C (&Rb)[6])
+{
+    C L[6], R[6];
+#pragma unroll
+    for (int u = 0; u < 6; u++) {
+        L[u] = rec_left(s[0][u], s[1][u], s[2][u], s[3][u], s[4][u]);
+        R[u] = rec_right(s[1][u], s[2][u], s[3][u], s[4][u], s[5][u]);
+    }
+    const Prim l = prim_of(L, gamma), r = prim_of(R, gamma);
+    const C aL = fabs(l.u[D]) + l.c, aR = fabs(r.u[D]) + r.c;
+    const bool left = aL > aR;
+    const C lam = left ? aL : aR;
+    C FLb[5], lamb = C(0);
+#pragma unroll
+    for (int u = 0; u < 5; u++) {
+        FLb[u] = C(0.5) * Fb[u];
+        Lb[u] = C(0.5) * lam * Fb[u];
+        Rb[u] = -Lb[u];
+        lamb -= C(0.5) * (R[u] - L[u]) * Fb[u];
+    }
+    Lb[5] = Rb[5] = C(0);
+    // the wave speed's adjoint goes to the side it came from
+    const C c = left ? l.c : r.c, ri = left ? l.r : r.r, uD = left ? l.u[D] : r.u[D];
+    const C pb = lamb * gamma * ri / (C(2) * c), rhob = -lamb * c * ri * C(0.5);
+    const C uDb = lamb * (uD > C(0) ? C(1) : (uD < C(0) ? C(-1) : C(0)));
+    flux_rev<D>(L, l, FLb, left ? pb : C(0), left ? rhob : C(0), left ? uDb : C(0), gamma, Lb);
+    flux_rev<D>(R, r, FLb, left ? C(0) : pb, left ? C(0) : rhob, left ? C(0) : uDb, gamma, Rb);
+}
+// weight of cell m (0..5) of a face's stencil in its left and right value
+__device__ __forceinline__ C w_left(int m)
+{
+    return m == 0 ? C(2.0 / 60) : m == 1 ? C(-13.0 / 60) : m == 2 ? C(47.0 / 60) : m == 3 ? C(27.0 / 60) : m == 4 ? C(-3.0 / 60) : C(0);
+}
+__device__ __forceinline__ C w_right(int m) { return w_left(5 - m); }
+
+// The stage combination's reverse and the x-faces': with lout the adjoint of
+// the stage's output, lqs (the adjoint of its input) starts as w lout, lq0
+// (of the step's input) gains (1 - w) lout, and L's adjoint is w dt lout
+// (wdt = w dt); then every cell gathers from the six x-faces that read it. A
+// warp takes 32 consecutive faces of a row (each loads its six cells; the
+// next lanes' loads hit the same lines) and gathers by shuffles for the 27
+// cells whose faces it has. Faces of a periodic row wrap; of another row
+// there are faces 0..nx, and the three cells past each end, which stand for
+// the end cell, are summed into it by the warp that has them all.
+constexpr int XCELLS = 27, XWARPS = 4;
+__global__ void __launch_bounds__(32 * XWARPS) k_adj_rhs_x(const S *q, const S *sig, const C *lout, C *lqs, C *lq0,
+                                                           C *lsig, Geom g, C gamma, C inv_dx, C w, C wdt, int first,
+                                                           int nseg)
+{
+    const unsigned wid = blockIdx.x * XWARPS + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, seg = (int)(wid % nseg);
+    const idx row = wid / nseg;
+    if (row >= (idx)g.ny * (idx)g.nz) return;
+    const idx base = row * (idx)g.nx;
+    const int n = g.nx;
+    const bool per = g.bc[0] == BC_PERIODIC;
+    int c0, c1, fs;  // cells of this warp, its first face
+    if (per) {
+        c0 = XCELLS * seg;
+        c1 = min(n, c0 + XCELLS);
+        fs = c0 - 2;
+    } else {
+        const bool last = seg == nseg - 1;
+        c0 = last ? min(XCELLS * seg - 3, n - 1) : XCELLS * seg - 3;
+        c1 = last ? n + 3 : min(c0 + XCELLS, n - 1);
+        fs = last ? n + 3 - XCELLS - 2 : c0 - 2;
+        if (last && nseg == 1) c0 = -3;
+    }
+    const int f = fs + lane;
+    C Lb[6], Rb[6];
+#pragma unroll
+    for (int u = 0; u < 6; u++) Lb[u] = Rb[u] = C(0);
+    if (per || (f >= 0 && f <= n)) {
+        C s[6][6], Fb[5];
+#pragma unroll
+        for (int m = 0; m < 6; m++) {
+            const idx c = ck(base + (idx)map_axis(f - 3 + m, n, g.bc[0], g.bc[1]), g.n);
+#pragma unroll
+            for (int u = 0; u < 5; u++) s[m][u] = ldc(q + ckl((size_t)u * (size_t)g.n + c, 5 * g.n));
+            s[m][5] = ldc(sig + c);
+        }
+        const idx ch = ck(base + (idx)map_axis(f, n, g.bc[0], g.bc[1]), g.n);
+        const idx cl = ck(base + (idx)map_axis(f - 1, n, g.bc[0], g.bc[1]), g.n);
+#pragma unroll
+        for (int u = 0; u < 5; u++) {
+            const C hi = per || f < n ? wdt * lout[ckl((size_t)u * (size_t)g.n + ch, 5 * g.n)] : C(0);
+            const C lo = per || f >= 1 ? wdt * lout[ckl((size_t)u * (size_t)g.n + cl, 5 * g.n)] : C(0);
+            Fb[u] = (hi - lo) * inv_dx;
+        }
+        face_rev<0>(s, Fb, gamma, Lb, Rb);
+    }
+    // lane l gathers for cell f = fs + l, on top of what the cell has: its
+    // faces are those of lanes l + 3 .. l - 2
+    const bool in = lane >= 2 && lane <= 28 && f >= max(c0, 0) && f < min(c1, n);
+    const idx c = in ? ck(base + (idx)f, g.n) : 0;
+    C v[6], a0[5];
+#pragma unroll
+    for (int u = 0; u < 5; u++) {
+        a0[u] = in ? lout[ckl((size_t)u * (size_t)g.n + c, 5 * g.n)] : C(0);
+        v[u] = w * a0[u];
+    }
+    v[5] = in ? lsig[c] : C(0);
+#pragma unroll
+    for (int m = 0; m < 6; m++)
+#pragma unroll
+        for (int u = 0; u < 6; u++)
+            v[u] += w_left(m) * __shfl_sync(0xffffffffu, Lb[u], (lane + 3 - m) & 31) +
+                    w_right(m) * __shfl_sync(0xffffffffu, Rb[u], (lane + 3 - m) & 31);
+    if (!per && (seg == 0 || seg == nseg - 1)) {  // the cells past the ends
+#pragma unroll
+        for (int u = 0; u < 6; u++) {
+            C lo = C(0), hi = C(0);
+#pragma unroll
+            for (int m = 1; m <= 3; m++) {
+                lo += __shfl_sync(0xffffffffu, v[u], (lane - m) & 31);
+                hi += __shfl_sync(0xffffffffu, v[u], (lane + m) & 31);
+            }
+            if (f == 0) v[u] += lo;
+            if (f == n - 1) v[u] += hi;
+        }
+    }
+    if (!in) return;
+#pragma unroll
+    for (int u = 0; u < 5; u++) {
+        const size_t at = ckl((size_t)u * (size_t)g.n + c, 5 * g.n);
+        lqs[at] = v[u];
+        lq0[at] = first ? (C(1) - w) * a0[u] : lq0[at] + (C(1) - w) * a0[u];
+    }
+    lsig[c] = v[5];
+}
+
+// The y- and z-faces' reverse: a thread marches along D over a chunk of cells
+// of one line (lanes along x, then the next line), with the six cells of the face's stencil and
+// the sums of the six cells it sends to in registers; a cell is written when
+// the last face that reads it is done. A chunk also evaluates the two faces
+// before and after it that reach its cells. Ends as for the x-faces; the
+// cells below an inflow face send to the cell above it (1 - W) and to the
+// inflow tables (lamJ).
+template <int D>
+__global__ void __launch_bounds__(128) k_adj_rhs_march(const S *q, const S *sig, const C *lout, C *lqs, C *lsig,
+                                                       C *lamJ, Geom g, C gamma, C inv_dx, C wdt, const C *W,
+                                                       const C *J, int chunk)
+{
+    const unsigned t = blockIdx.x * 128u + threadIdx.x, line = t / (unsigned)g.nx, i = t - line * (unsigned)g.nx;
+    if (line >= (unsigned)(D == 1 ? g.nz : g.ny)) return;
+    const int n = D == 1 ? g.ny : g.nz, blo = D == 1 ? g.bc[2] : g.bc[4], bhi = D == 1 ? g.bc[3] : g.bc[5];
+    const bool per = blo == BC_PERIODIC, jet = D == 2 && blo == BC_INFLOW;
+    const idx step = D == 1 ? (idx)g.nx : (idx)g.plane;
+    const idx base = (idx)line * (D == 1 ? (idx)g.plane : (idx)g.nx) + (idx)i;
+    const int c0 = blockIdx.y * chunk, c1 = min(n, c0 + chunk);
+    const int f0 = per ? c0 - 2 : max(0, c0 - 2), f1 = per ? c1 + 2 : min(n, c1 + 2);
+    auto cell = [&](int c) { return ck(base + (idx)map_axis(c, n, blo, bhi) * step, g.n); };
+    auto value = [&](int c, C (&s)[6]) {
+        const idx at = cell(c);
+#pragma unroll
+        for (int u = 0; u < 5; u++) s[u] = ldc(q + ckl((size_t)u * (size_t)g.n + at, 5 * g.n));
+        s[5] = ldc(sig + at);
+        if (jet && c < 0) {
+            const C wf = C(1) - W[ck(base, g.plane)];
+#pragma unroll
+            for (int u = 0; u < 5; u++) s[u] = wf * s[u] + J[ckl((size_t)u * (size_t)g.plane + base, 5 * g.plane)];
+        }
+    };
+    auto adjoint = [&](int c, C (&l)[5]) {
+        const bool in = per || (c >= 0 && c < n);
+        const idx at = cell(c);
+#pragma unroll
+        for (int u = 0; u < 5; u++) l[u] = in ? wdt * lout[ckl((size_t)u * (size_t)g.n + at, 5 * g.n)] : C(0);
+    };
+    // what the cell has so far (0 for one that this thread does not write)
+    auto begin = [&](int c, C (&v)[6]) {
+        const bool mine = c >= c0 && c < c1;
+        const idx at = mine ? cell(c) : 0;
+#pragma unroll
+        for (int u = 0; u < 5; u++) v[u] = mine ? lqs[ckl((size_t)u * (size_t)g.n + at, 5 * g.n)] : C(0);
+        v[5] = mine ? lsig[at] : C(0);
+    };
+    auto write = [&](int c, const C (&v)[6]) {
+        if (c < c0 || c >= c1) return;
+        const idx at = cell(c);
+#pragma unroll
+        for (int u = 0; u < 5; u++) lqs[ckl((size_t)u * (size_t)g.n + at, 5 * g.n)] = v[u];
+        lsig[at] = v[5];
+    };
+    const C wf = jet ? C(1) - W[ck(base, g.plane)] : C(1);
+    // From the last face down: a cell then gathers from the face three above
+    // it first and the face two below it last, as from the x-faces.
+    C s[6][6], acc[6][6], hi[5];
+#pragma unroll
+    for (int m = 1; m < 6; m++) {
+        value(f1 - 3 + m, s[m]);
+        begin(f1 - 3 + m, acc[m]);
+    }
+    adjoint(f1, hi);
+    C below[3][3][5];  // what the faces 0..2 send below an inflow face's first cell
+    for (int f = f1; f >= f0; f--) {
+        C lo[5], Fb[5], Lb[6], Rb[6];
+        value(f - 3, s[0]);
+        begin(f - 3, acc[0]);
+        adjoint(f - 1, lo);
+#pragma unroll
+        for (int u = 0; u < 5; u++) {
+            Fb[u] = (hi[u] - lo[u]) * inv_dx;
+            hi[u] = lo[u];
+        }
+        face_rev<D>(s, Fb, gamma, Lb, Rb);
+        auto sent = [&](int m, int u) { return w_left(m) * Lb[u] + w_right(m) * Rb[u]; };
+        if (!per && f < 3) {  // cells below the line's end: f - 3 .. -1, which stand for cell 0 = f - 3 + e
+#pragma unroll
+            for (int e = 1; e <= 3; e++)
+                if (e == 3 - f) {
+#pragma unroll
+                    for (int m = 0; m < e; m++)
+#pragma unroll
+                        for (int u = 0; u < 6; u++) {
+                            const C a = sent(m, u);
+                            acc[e][u] += u < 5 ? wf * a : a;
+                            if (jet && u < 5) below[3 - e][m][u] = a;
+                        }
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < 6; m++)
+#pragma unroll
+            for (int u = 0; u < 6; u++) acc[m][u] += sent(m, u);
+        if (!per && f > n - 3) {  // cells past the end: n .. f + 2, which stand for cell n - 1 = f - 3 + e
+#pragma unroll
+            for (int e = 2; e <= 4; e++)
+                if (e == n - 1 - f + 3) {
+#pragma unroll
+                    for (int m = e + 1; m < 6; m++)
+#pragma unroll
+                        for (int u = 0; u < 6; u++) acc[e][u] += sent(m, u);
+                }
+        }
+        write(f + 2, acc[5]);  // no face below reads this cell
+        if (f > f0) {
+#pragma unroll
+            for (int m = 5; m > 0; m--)
+#pragma unroll
+                for (int u = 0; u < 6; u++) {
+                    s[m][u] = s[m - 1][u];
+                    acc[m][u] = acc[m - 1][u];
+                }
+        }
+    }
+    if (!per && f0 == 0) {  // below the first face: cells 1 and 0
+        write(1, acc[4]);
+        write(0, acc[3]);
+    }
+    if (jet && c0 == 0) {
+#pragma unroll
+        for (int u = 0; u < 5; u++) {
+            const size_t at = ckl((size_t)u * (size_t)g.plane + base, 5 * g.plane);
+            C v = lamJ[at];
+#pragma unroll
+            for (int m = 0; m < 3; m++)
+#pragma unroll
+                for (int f = 0; f < 3 - m; f++) v += below[f][m][u];
+            lamJ[at] = v;
+        }
+    }
+}
+
+// neighbour of the cell at (i, j, k) across face d (0: -x .. 5: +z); false on
+// a non-periodic domain boundary (no face term there)
+__device__ __forceinline__ bool nbr(const Geom &g, int i, int j, int k, int d, idx &out)
+{
+    int c[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz};
+    int ax = d >> 1;
+    c[ax] += (d & 1) ? 1 : -1;
+    if (c[ax] < 0 || c[ax] >= n[ax]) {
+        if (g.bc[d] != BC_PERIODIC) return false;
+        c[ax] = c[ax] < 0 ? c[ax] + n[ax] : c[ax] - n[ax];
+    }
+    out = ck(((idx)c[2] * (idx)g.ny + (idx)c[1]) * (idx)g.nx + (idx)c[0], g.n);
+    return true;
+}
+// cell-wise kernels: 32 x 4 cells of a plane per block
+constexpr int CBX = 32, CBY = 4;
+__device__ __forceinline__ bool cell_of(const Geom &g, int &i, int &j, int &k, idx &t)
+{
+    const unsigned gx = ((unsigned)g.nx + CBX - 1) / CBX, gy = ((unsigned)g.ny + CBY - 1) / CBY;
+    const unsigned rest = blockIdx.x / gx;
+    i = (int)(blockIdx.x % gx) * CBX + (int)threadIdx.x;
+    j = (int)(rest % gy) * CBY + (int)threadIdx.y;
+    k = (int)(rest / gy);
+    t = ((idx)k * (idx)g.ny + (idx)j) * (idx)g.nx + (idx)i;
+    return i < g.nx && j < g.ny;
+}
+
+// r = 1 / rho and the diagonal D of the sweeps, once per stage (FP64: 1 / D,
+// whose seven divisions per cell and sweep would be slow)
+__device__ __forceinline__ float mu_of(float l, float d) { return l / d; }
+__device__ __forceinline__ double mu_of(double l, double dinv) { return l * dinv; }
+__global__ void __launch_bounds__(CBX *CBY) k_adj_diag(const S *q, C *r, C *dg, Geom g, C beta)
+{
+    int i, j, k;
+    idx t;
+    if (!cell_of(g, i, j, k, t)) return;
+    const C ri = C(1) / ldc(q + t);
+    C diag = ri;
+#pragma unroll
+    for (int d = 0; d < 6; d++) {
+        idx m;
+        if (nbr(g, i, j, k, d, m)) diag += beta * C(0.5) * (ri + C(1) / ldc(q + m));
+    }
+    r[t] = ri;
+    dg[t] = sizeof(C) == 8 ? C(1) / diag : diag;
+}
+
+// One reversed Jacobi sweep s_k -> F, gathered (the neighbour relation is
+// symmetric): with mu = lsig / D (lsig the adjoint of F),
+//   nl_m = sum_i beta c_im mu_i (the adjoint of s_k), lb_m += mu_m,
+//   rb_m += mu_m (beta/2 sum s_nb - F_m (1 + beta nf/2)) + sum_i mu_i beta/2 (s_m - F_i);
+// the neighbours' mu are formed again from lsig and D, which saves a pass.
+__global__ void __launch_bounds__(CBX *CBY) k_adj_jacobi(const C *__restrict__ r, const C *__restrict__ dg,
+                                                         const S *__restrict__ sk, const S *__restrict__ F,
+                                                         const C *__restrict__ lsig, C *nl, C *lb, C *rb, Geom g,
+                                                         C beta, int first)
+{
+    int i, j, k;
+    idx t;
+    if (!cell_of(g, i, j, k, t)) return;
+    const C rm = r[t], sm = ldc(sk + t), Fm = ldc(F + t), mum = mu_of(lsig[t], dg[t]), hb = C(0.5) * beta;
+    C acc = C(0), ssum = C(0), rbm = C(0);
+    int nfc = 0;
+#pragma unroll
+    for (int d = 0; d < 6; d++) {
+        idx n;
+        if (!nbr(g, i, j, k, d, n)) continue;
+        const C mun = mu_of(lsig[n], dg[n]);
+        acc += hb * (rm + r[n]) * mun;
+        ssum += ldc(sk + n);
+        nfc++;
+        rbm += mun * hb * (sm - ldc(F + n));
+    }
+    rbm += mum * (hb * ssum - Fm * (C(1) + hb * C(nfc)));
+    nl[t] = acc;
+    lb[t] = first ? mum : lb[t] + mum;
+    rb[t] = first ? rbm : rb[t] + rbm;
+}
+
+// Reverse of the source, first pass: the adjoints of the nine gradients of u
+// at each cell, Gb[a][c] = alpha (2 G_ca + 2 delta_ac tr G) lb / (2 dx)
+struct Grads {
+    C *p[9];
+};
+__global__ void __launch_bounds__(CBX *CBY) k_adj_grad(const S *q, const C *__restrict__ r, const C *lb, Grads out,
+                                                       Geom g, C alpha, C inv2dx, const C *W, const C *J)
+{
+    int i, j, k;
+    idx t;
+    if (!cell_of(g, i, j, k, t)) return;
+    const C bb = lb[t];
+    C G[3][3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        C u[2][3];
+#pragma unroll
+        for (int s = 0; s < 2; s++) {
+            const int ii = i + (c == 0 ? 1 - 2 * s : 0), jj = j + (c == 1 ? 1 - 2 * s : 0),
+                      kk = k + (c == 2 ? 1 - 2 * s : 0);
+            const idx f = (idx)map_axis(jj, g.ny, g.bc[2], g.bc[3]) * (idx)g.nx + (idx)map_axis(ii, g.nx, g.bc[0], g.bc[1]);
+            C ri;
+            if (kk < 0 && g.bc[4] == BC_INFLOW)
+                ri = C(1) / val_col(q, nullptr, g, W, J, f, kk, 0);
+            else
+                ri = r[ck((idx)zmap(kk, g) * (idx)g.plane + f, g.n)];
+#pragma unroll
+            for (int a = 0; a < 3; a++) u[s][a] = val_col(q, nullptr, g, W, J, f, kk, 1 + a) * ri;
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) G[a][c] = (u[0][a] - u[1][a]) * inv2dx;
+    }
+    const C tr = G[0][0] + G[1][1] + G[2][2], s = alpha * bb * inv2dx;
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int c = 0; c < 3; c++) out.p[3 * a + c][t] = s * (C(2) * G[c][a] + (a == c ? C(2) * tr : C(0)));
+}
+// Second pass: a cell's u is the upper value of the gradient of the cell below
+// it and the lower one of the cell above; at a boundary the cell's own
+// gradient reads it (or, below an inflow face, the blend of it) as the ghost.
+// Then u to (rho, m), and the sweeps' adjoint rb of 1/rho to rho.
+__global__ void __launch_bounds__(CBX *CBY) k_adj_source(const S *q, const C *__restrict__ r, const C *rb, Grads G,
+                                                         C *lq, C *lamJ, Geom g, const C *W, const C *J)
+{
+    int i, j, k;
+    idx t;
+    if (!cell_of(g, i, j, k, t)) return;
+    const C ri = r[t];
+    const bool jet = k == 0 && g.bc[4] == BC_INFLOW;
+    C v[4], m[3], mg[3], rg = C(0), wf = C(0), lj[4];
+#pragma unroll
+    for (int f = 0; f < 4; f++) v[f] = lq[ckl((size_t)f * (size_t)g.n + t, 5 * g.n)];
+#pragma unroll
+    for (int a = 0; a < 3; a++) m[a] = ldc(q + ckl((size_t)(1 + a) * (size_t)g.n + t, 5 * g.n));
+    if (jet) {
+        rg = C(1) / val_col(q, nullptr, g, W, J, t, -1, 0);
+        wf = C(1) - W[ck(t, g.plane)];
+#pragma unroll
+        for (int a = 0; a < 3; a++) mg[a] = val_col(q, nullptr, g, W, J, t, -1, 1 + a);
+#pragma unroll
+        for (int f = 0; f < 4; f++) lj[f] = lamJ[ckl((size_t)f * (size_t)g.plane + t, 5 * g.plane)];
+    }
+    v[0] -= rb[t] * ri * ri;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        idx lo = t, hi = t;
+        const bool has_lo = nbr(g, i, j, k, 2 * c, lo), has_hi = nbr(g, i, j, k, 2 * c + 1, hi);
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const C *p = G.p[3 * a + c];
+            // adjoint us of this cell's u_a, added as that of (rho, m_a)
+            auto add = [&](C us) {
+                const C mb = us * ri;
+                v[1 + a] += mb;
+                v[0] -= mb * m[a] * ri;
+            };
+            add(has_hi ? -p[hi] : p[t]);
+            if (c == 2 && jet) {
+                const C mb = -p[t] * rg, rhob = -mb * mg[a] * rg;
+                v[1 + a] += wf * mb;
+                v[0] += wf * rhob;
+                lj[1 + a] += mb;
+                lj[0] += rhob;
+            } else {
+                add(has_lo ? p[lo] : -p[t]);
+            }
+        }
+    }
+#pragma unroll
+    for (int f = 0; f < 4; f++) {
+        lq[ckl((size_t)f * (size_t)g.n + t, 5 * g.n)] = v[f];
+        if (jet) lamJ[ckl((size_t)f * (size_t)g.plane + t, 5 * g.plane)] = lj[f];
+    }
+}
+
+// out = a + b over n values
+__global__ void k_adj_add(const C *a, const C *b, C *out, long long n)
+{
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
+        out[c] = a[c] + b[c];
+}
+
+// part[n][b] = block b's share of the sum over the inflow face of
+// s_n (rho_n lamJ_mz + rho_n w_n lamJ_E), then gw[n] = the shares in order.
+// Twenty edge widths outside a jet s_n is 0 to the last bit, so those cells
+// skip the FP64 root and tanh; one block per jet took 263 us on a 128^2 face.
+__global__ void __launch_bounds__(256) k_adj_jets(const double *jets, const C *lamJ, double *part, int nx, int ny,
+                                                  double dx)
 {
     const double *jt = jets + 7 * blockIdx.x;
-    long long plane = (long long)nx * ny;
+    const long long plane = (long long)nx * ny;
+    const double reach = jt[2] + 20.0 * jt[6] * dx;
     double acc = 0.0;
-    for (long long f = threadIdx.x; f < plane; f += blockDim.x) {
-        int i = (int)(f % nx), j = (int)(f / nx);
-        double x = (i + 0.5) * dx, y = (j + 0.5) * dx;
-        double r = sqrt((x - jt[0]) * (x - jt[0]) + (y - jt[1]) * (y - jt[1]));
-        double sn = 0.5 * (1.0 - tanh((r - jt[2]) / (jt[6] * dx)));
+    for (long long f = blockIdx.y * 256LL + threadIdx.x; f < plane; f += 256LL * gridDim.y) {
+        const int i = (int)((unsigned)f % (unsigned)nx), j = (int)((unsigned)f / (unsigned)nx);
+        const double x = (i + 0.5) * dx - jt[0], y = (j + 0.5) * dx - jt[1], r2 = x * x + y * y;
+        if (r2 > reach * reach) continue;
+        const double sn = 0.5 * (1.0 - tanh((sqrt(r2) - jt[2]) / (jt[6] * dx)));
         acc += sn * (jt[3] * double(lamJ[ckl(3 * plane + f, 5 * plane)]) +
                      jt[3] * jt[4] * double(lamJ[ckl(4 * plane + f, 5 * plane)]));
     }
     __shared__ double red[256];
     red[threadIdx.x] = acc;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    for (int o = 128; o > 0; o >>= 1) {
         if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) gw[blockIdx.x] += red[0];
+    if (threadIdx.x == 0) part[blockIdx.x * gridDim.y + blockIdx.y] = red[0];
+}
+__global__ void k_adj_jets_sum(const double *part, double *gw, int njets, int nblk)
+{
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= njets) return;
+    double s = 0.0;
+    for (int b = 0; b < nblk; b++) s += part[n * nblk + b];
+    gw[n] = s;
 }
 
 // ------------------------------------------------- grouped launches
@@ -3128,55 +3612,127 @@ cudaError_t launch_rk_combine(const void *qn, const void *qs, const void *L, voi
     return cudaGetLastError();
 }
 
-int adj_blocks(long long n)
+// blocks of a grid-stride launch over n values
+int flat_blocks(long long n)
 {
     long long b = (n + 255) / 256;
     return (int)(b < 152 * 32 ? (b > 0 ? b : 1) : 152 * 32);
+}
+unsigned cell_blocks(const Geom &g)
+{
+    return (unsigned)(((long long)g.nx + CBX - 1) / CBX * ((g.ny + CBY - 1) / CBY) * g.nz);
+}
+// cells per chunk of a march over n cells in `lines` blocks: a chunk evaluates
+// five faces beyond its cells; three blocks fit an SM in FP32, and one fills
+// its FP64 units (as choose_zc)
+int march_chunk(long long lines, int n)
+{
+    int best = n;
+    double tbest = 1e300;
+    const long long slots = sizeof(C) == 8 ? 152 : 456;
+    for (int m = (n + 65534) / 65535; m <= (n + 3) / 4; m++) {
+        const int zc = (n + m - 1) / m;
+        const long long blocks = lines * ((n + zc - 1) / zc);
+        const double t = (zc + 5.0) * (double)((blocks + slots - 1) / slots);
+        if (t < tbest * 0.999) {
+            tbest = t;
+            best = zc;
+        }
+        if (blocks > 16 * slots) break;
+    }
+    return best;
+}
+
+cudaError_t launch_adj_rhs(const Geom &g, const Phys &p, const Inflow &in, const void *qs, const void *sig,
+                           const void *lout, void *lqs, void *lq0, void *lsig, void *lamJ, double w, double dt,
+                           int first, cudaStream_t st)
+{
+    const C *W = (const C *)in.W, *J = (const C *)in.J, *lo = (const C *)lout;
+    const S *q = (const S *)qs, *s = (const S *)sig;
+    const C gamma = C(p.gamma), inv_dx = C(1.0 / p.dx), wdt = C(w) * C(dt);
+    const long long rows = (long long)g.ny * g.nz;
+    const int nseg = g.bc[0] == BC_PERIODIC ? (g.nx + XCELLS - 1) / XCELLS : (g.nx + 6 + XCELLS - 1) / XCELLS;
+    k_adj_rhs_x<<<(unsigned)((rows * nseg + XWARPS - 1) / XWARPS), 32 * XWARPS, 0, st>>>(
+        q, s, lo, (C *)lqs, (C *)lq0, (C *)lsig, g, gamma, inv_dx, C(w), wdt, first, nseg);
+    const long long by = ((long long)g.nx * g.nz + 127) / 128, bz = (g.plane + 127) / 128;
+    const int cy = march_chunk(by, g.ny), cz = march_chunk(bz, g.nz);
+    k_adj_rhs_march<1><<<dim3((unsigned)by, (g.ny + cy - 1) / cy), 128, 0, st>>>(
+        q, s, lo, (C *)lqs, (C *)lsig, (C *)lamJ, g, gamma, inv_dx, wdt, W, J, cy);
+    k_adj_rhs_march<2><<<dim3((unsigned)bz, (g.nz + cz - 1) / cz), 128, 0, st>>>(
+        q, s, lo, (C *)lqs, (C *)lsig, (C *)lamJ, g, gamma, inv_dx, wdt, W, J, cz);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_adj_rk(const void *lout, void *lq0, void *lqs, void *Lb, long long n5, double w,
                           double dt, cudaStream_t st)
 {
-    k_adj_rk<<<adj_blocks(n5), 256, 0, st>>>((const C *)lout, (C *)lq0, (C *)lqs, (C *)Lb, n5, C(w), C(dt));
+    k_adj_rk<<<flat_blocks(n5), 256, 0, st>>>((const C *)lout, (C *)lq0, (C *)lqs, (C *)Lb, n5, C(w), C(dt));
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_rhs(const Geom &g, const Phys &p, const Inflow &in, const void *qs, const void *sig,
+cudaError_t launch_adj_rhs_scatter(const Geom &g, const Phys &p, const Inflow &in, const void *qs, const void *sig,
                            const void *Lb, void *lqs, void *lsig, void *lamJ, cudaStream_t st)
 {
     long long nfx = (long long)(g.nx + 1) * g.ny * g.nz, nfy = (long long)g.nx * (g.ny + 1) * g.nz,
               nfz = (long long)g.nx * g.ny * (g.nz + 1);
     const C *W = (const C *)in.W, *J = (const C *)in.J;
-    k_adj_rhs<0><<<adj_blocks(nfx), 256, 0, st>>>((const S *)qs, (const S *)sig, (const C *)Lb, (C *)lqs,
+    k_adj_rhs_scatter<0><<<flat_blocks(nfx), 256, 0, st>>>((const S *)qs, (const S *)sig, (const C *)Lb, (C *)lqs,
                                                    (C *)lsig, (C *)lamJ, g, C(p.gamma), C(1.0 / p.dx), W, J);
-    k_adj_rhs<1><<<adj_blocks(nfy), 256, 0, st>>>((const S *)qs, (const S *)sig, (const C *)Lb, (C *)lqs,
+    k_adj_rhs_scatter<1><<<flat_blocks(nfy), 256, 0, st>>>((const S *)qs, (const S *)sig, (const C *)Lb, (C *)lqs,
                                                    (C *)lsig, (C *)lamJ, g, C(p.gamma), C(1.0 / p.dx), W, J);
-    k_adj_rhs<2><<<adj_blocks(nfz), 256, 0, st>>>((const S *)qs, (const S *)sig, (const C *)Lb, (C *)lqs,
+    k_adj_rhs_scatter<2><<<flat_blocks(nfz), 256, 0, st>>>((const S *)qs, (const S *)sig, (const C *)Lb, (C *)lqs,
                                                    (C *)lsig, (C *)lamJ, g, C(p.gamma), C(1.0 / p.dx), W, J);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_adj_jacobi(const Geom &g, const Phys &p, const void *q, const void *sk, const void *F,
-                              const void *lsig, void *nl, void *lb, void *rb, void *mu, cudaStream_t st)
-{
-    C beta = C(p.alpha / (p.dx * p.dx));
-    k_adj_jac_mu<<<adj_blocks(g.n), 256, 0, st>>>((const S *)q, (const C *)lsig, (C *)mu, (C *)lb, g, beta);
-    k_adj_jac_gather<<<adj_blocks(g.n), 256, 0, st>>>((const S *)q, (const S *)sk, (const S *)F,
-                                                       (const C *)mu, (C *)nl, (C *)rb, g, beta);
     return cudaGetLastError();
 }
 
 cudaError_t launch_adj_rho(const Geom &g, const void *q, void *rb, void *lqs, cudaStream_t st)
 {
-    k_adj_rho<<<adj_blocks(g.n), 256, 0, st>>>((const S *)q, (C *)rb, (C *)lqs, g.n);
+    k_adj_rho<<<flat_blocks(g.n), 256, 0, st>>>((const S *)q, (C *)rb, (C *)lqs, g.n);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_source(const Geom &g, const Phys &p, const Inflow &in, const void *q, const void *lb,
+cudaError_t launch_adj_source_scatter(const Geom &g, const Phys &p, const Inflow &in, const void *q, const void *lb,
                               void *lqs, void *lamJ, cudaStream_t st)
 {
-    k_adj_source<<<adj_blocks(g.n), 256, 0, st>>>((const S *)q, (const C *)lb, (C *)lqs, (C *)lamJ, g,
+    k_adj_source_scatter<<<flat_blocks(g.n), 256, 0, st>>>((const S *)q, (const C *)lb, (C *)lqs, (C *)lamJ, g,
                                                    C(p.alpha), C(0.5 / p.dx), (const C *)in.W, (const C *)in.J);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adj_diag(const Geom &g, const Phys &p, const void *q, void *r, void *dinv, cudaStream_t st)
+{
+    k_adj_diag<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const S *)q, (C *)r, (C *)dinv, g,
+                                                          C(p.alpha / (p.dx * p.dx)));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adj_jacobi(const Geom &g, const Phys &p, const void *r, const void *dinv, const void *sk,
+                              const void *F, const void *lsig, void *nl, void *lb, void *rb, int first,
+                              cudaStream_t st)
+{
+    k_adj_jacobi<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const C *)r, (const C *)dinv, (const S *)sk,
+                                                            (const S *)F, (const C *)lsig, (C *)nl, (C *)lb, (C *)rb,
+                                                            g, C(p.alpha / (p.dx * p.dx)), first);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adj_source(const Geom &g, const Phys &p, const Inflow &in, const void *q, const void *r,
+                              const void *lb, const void *rb, void *const grads[9], void *lqs, void *lamJ,
+                              cudaStream_t st)
+{
+    Grads G;
+    for (int t = 0; t < 9; t++) G.p[t] = (C *)grads[t];
+    const C *W = (const C *)in.W, *J = (const C *)in.J;
+    k_adj_grad<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const S *)q, (const C *)r, (const C *)lb, G, g,
+                                                          C(p.alpha), C(0.5 / p.dx), W, J);
+    k_adj_source<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const S *)q, (const C *)r, (const C *)rb, G, (C *)lqs,
+                                                            (C *)lamJ, g, W, J);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adj_add(const void *a, const void *b, void *out, long long n, cudaStream_t st)
+{
+    k_adj_add<<<flat_blocks(n), 256, 0, st>>>((const C *)a, (const C *)b, (C *)out, n);
     return cudaGetLastError();
 }
 
@@ -3184,7 +3740,9 @@ cudaError_t launch_adj_jets(const Geom &g, const Phys &p, const double *jets, in
                             double *gw, cudaStream_t st)
 {
     if (njets <= 0) return cudaSuccess;
-    k_adj_jets<<<njets, 256, 0, st>>>(jets, (const C *)lamJ, gw, g.nx, g.ny, p.dx);
+    double *part = gw + njets;
+    k_adj_jets<<<dim3(njets, ADJ_JET_BLOCKS), 256, 0, st>>>(jets, (const C *)lamJ, part, g.nx, g.ny, p.dx);
+    k_adj_jets_sum<<<(njets + 31) / 32, 32, 0, st>>>(part, gw, njets, ADJ_JET_BLOCKS);
     return cudaGetLastError();
 }
 
@@ -3233,8 +3791,9 @@ cudaError_t bounds_selftest(int *sink, cudaStream_t st)
 
 extern const Ops IGR_OPS = {
     (int)sizeof(S), (int)sizeof(C), (int)sizeof(QB), launch_source, launch_jacobi, launch_flux, flux_blocks,
-    launch_speed, launch_rk_combine, launch_adj_rk, launch_adj_rhs, launch_adj_jacobi, launch_adj_rho,
-    launch_adj_source, launch_adj_jets, launch_diag, bounds_hits, bounds_selftest,
+    launch_speed, launch_rk_combine, launch_adj_rhs, launch_adj_diag, launch_adj_jacobi, launch_adj_source,
+    launch_adj_add, launch_adj_jets, launch_adj_rk, launch_adj_rhs_scatter, launch_adj_rho,
+    launch_adj_source_scatter, launch_diag, bounds_hits, bounds_selftest,
     launch_source_group, launch_jacobi_group, launch_flux_group, source_shape, jacobi_shape,
 };
 
