@@ -207,10 +207,14 @@ __device__ __forceinline__ void finalize_dt_body(const double *blockmax, int nbl
     if (fixed_dt <= 0.0)
         for (int t = threadIdx.x; t < nblocks; t += blockDim.x) m = nanmax_d(m, blockmax[t]);
     for (int o = 16; o > 0; o >>= 1) m = nanmax_d(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
+    if (warps > 1) {
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+        __syncthreads();
+        if (threadIdx.x >= 32) return;
+        m = (int)threadIdx.x < warps ? red[threadIdx.x] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) m = nanmax_d(m, __shfl_xor_sync(0xffffffffu, m, o));
+    }
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); w++) m = nanmax_d(m, red[w]);
         double dt = fixed_dt > 0.0 ? fixed_dt : cfl_dx / m;
         if (fixed_dt <= 0.0) sc->speed = m;
         if (!(dt > 0.0) || isinf(dt)) sc->err |= ERRF_NONFINITE;
@@ -218,6 +222,8 @@ __device__ __forceinline__ void finalize_dt_body(const double *blockmax, int nbl
         sc->t += dt;
     }
 }
+// threads of the finaliser's block
+static int dt_threads(int nblocks) { return nblocks >= 1024 ? 1024 : nblocks <= 32 ? 32 : (nblocks + 31) / 32 * 32; }
 
 // ------------------------------------------------------------ helpers
 
@@ -800,7 +806,7 @@ igr_status igr_get_state(igr_ctx *c, void *q, void *sigma, igr_dtype dtype, int 
 static igr_status finalize_dt(igr_ctx *c, double fixed_dt)
 {
     prof_begin(c, KC_OTHER);
-    k_finalize_dt<<<1, 1024, 0, c->st>>>(c->blockmax, c->speed_nblocks, c->sc, c->cfg.cfl * c->cfg.dx,
+    k_finalize_dt<<<1, dt_threads(c->speed_nblocks), 0, c->st>>>(c->blockmax, c->speed_nblocks, c->sc, c->cfg.cfl * c->cfg.dx,
                                         fixed_dt);
     CU(c, cudaGetLastError());
     prof_end(c);
@@ -971,7 +977,7 @@ igr_status igr_get_dt(igr_ctx *c, double *dt)
     // reduce into the second scalar slot so the step's scalars are untouched
     Scalars *tmp = c->sc + 1;
     CU(c, cudaMemsetAsync(tmp, 0, sizeof(Scalars), c->st));
-    k_finalize_dt<<<1, 1024, 0, c->st>>>(c->blockmax, c->speed_nblocks, tmp, c->cfg.cfl * c->cfg.dx, 0.0);
+    k_finalize_dt<<<1, dt_threads(c->speed_nblocks), 0, c->st>>>(c->blockmax, c->speed_nblocks, tmp, c->cfg.cfl * c->cfg.dx, 0.0);
     CU(c, cudaGetLastError());
     Scalars h;
     CU(c, cudaMemcpyAsync(&h, tmp, sizeof(Scalars), cudaMemcpyDeviceToHost, c->st));
@@ -1237,8 +1243,9 @@ static igr_status step_grouped(igr_batch *b)
         for (int i = 0; i < a.count; i++) {
             igr_ctx *c = b->inst[i0 + i];
             a.d[i] = {c->blockmax, c->speed_nblocks, c->sc, c->cfg.cfl * c->cfg.dx};
+            threads = std::max(threads, dt_threads(c->speed_nblocks));
         }
-        k_finalize_dt_group<<<a.count, 1024, 0, st>>>(a);
+        k_finalize_dt_group<<<a.count, threads, 0, st>>>(a);
         if (cudaGetLastError() != cudaSuccess) return bfail(b, IGR_ERR_CUDA, "grouped dt launch");
     }
     int maxs = 0;
