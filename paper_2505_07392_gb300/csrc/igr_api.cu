@@ -202,7 +202,10 @@ __global__ void k_finalize_dt_group(const __grid_constant__ DtGroup a)
 __device__ __forceinline__ void finalize_dt_body(const double *blockmax, int nblocks, Scalars *sc, double cfl_dx,
                                                  double fixed_dt)
 {
+    // one warp per 32 maxima up to 32 warps, then one warp over the warps (a
+    // thread walking them took 8 us of dependent FP64 comparisons)
     __shared__ double red[32];
+    const int warps = blockDim.x >> 5;
     double m = 0.0;
     if (fixed_dt <= 0.0)
         for (int t = threadIdx.x; t < nblocks; t += blockDim.x) m = nanmax_d(m, blockmax[t]);
@@ -1240,6 +1243,7 @@ static igr_status step_grouped(igr_batch *b)
     for (int i0 = 0; i0 < n; i0 += kGroupMax) {
         DtGroup a;
         a.count = std::min(n - i0, (int)kGroupMax);
+        int threads = 32;
         for (int i = 0; i < a.count; i++) {
             igr_ctx *c = b->inst[i0 + i];
             a.d[i] = {c->blockmax, c->speed_nblocks, c->sc, c->cfg.cfl * c->cfg.dx};
