@@ -429,15 +429,23 @@ static Inflow inflow_of(igr_ctx *c)
 
 // `sweeps` sweeps warm-started from s_first: Jacobi ping-pongs between
 // s_first and s_other; red-black Gauss-Seidel updates s_first in place (two
-// half-sweeps each). *result is the buffer holding the solution.
+// half-sweeps each). *result is the buffer holding the solution. coefs: 5 n
+// scratch values in the state type, for FP64's stored coefficients (from the
+// first sweep on: forming them costs less than one sweep without).
 static igr_status launch_sweeps(igr_ctx *c, const Tiles &t, const void *q, const void *b,
-                                void *s_first, void *s_other, int sweeps, void **result)
+                                void *s_first, void *s_other, int sweeps, void **result, void *coefs)
 {
+    const Ops *o = c->ops;
+    auto sweep = [&](const void *s_in, void *s_out, int colour, bool first) -> cudaError_t {
+        if (!o->sweep) return o->jacobi(c->g, c->p, t, q, b, s_in, s_out, colour, c->st);
+        cudaError_t e = first ? o->coefs(c->g, c->p, q, coefs, c->st) : cudaSuccess;
+        return e == cudaSuccess ? o->sweep(c->g, coefs, b, s_in, s_out, colour, c->st) : e;
+    };
     if (c->cfg.sigma_solver == SOLVER_RBGS) {
         for (int it = 0; it < sweeps; it++)
             for (int colour = 0; colour < 2; colour++) {
                 prof_begin(c, KC_JACOBI);
-                CU(c, c->ops->jacobi(c->g, c->p, t, q, b, s_first, s_first, colour, c->st));
+                CU(c, sweep(s_first, s_first, colour, it == 0 && colour == 0));
                 prof_end(c);
             }
         *result = s_first;
@@ -446,7 +454,7 @@ static igr_status launch_sweeps(igr_ctx *c, const Tiles &t, const void *q, const
     void *src = s_first, *dst = s_other;
     for (int it = 0; it < sweeps; it++) {
         prof_begin(c, KC_JACOBI);
-        CU(c, c->ops->jacobi(c->g, c->p, t, q, b, src, dst, -1, c->st));
+        CU(c, sweep(src, dst, -1, it == 0));
         prof_end(c);
         void *t = src;
         src = dst;
@@ -478,7 +486,10 @@ static igr_status run_stage(igr_ctx *c, int mode, const void *qs, const void *qd
     // the sweeps read the density as field 0 of their q: the state itself, or
     // the stage density the source kernel stored (increment modes)
     const void *qj = c->inc ? c->rho16 : qs;
-    igr_status s = launch_sweeps(c, c->tiles, qj, c->b, c->sig[c->cur], c->sig[1 - c->cur], c->cfg.sweeps, &res);
+    // scratch of the sweeps: the flux's output, or where that is q^n (stage 3) stage 1's
+    void *free5 = out != qs && out != qn ? out : c->q[1];
+    igr_status s = launch_sweeps(c, c->tiles, qj, c->b, c->sig[c->cur], c->sig[1 - c->cur], c->cfg.sweeps, &res,
+                                 free5);
     if (s != IGR_OK) return s;
     c->cur = res == c->sig[0] ? 0 : 1;
     if (q_ready) {
@@ -933,7 +944,7 @@ igr_status igr_solve_sigma(igr_ctx *c, const void *q, void *sigma_inout, int swe
     // the caller's buffer and it, and an odd count copies the result back
     void *scratch = c->sig[1 - c->cur];
     void *res;
-    igr_status s = launch_sweeps(c, t, c->inc ? c->rho16 : q, c->b, sigma_inout, scratch, sweeps, &res);
+    igr_status s = launch_sweeps(c, t, c->inc ? c->rho16 : q, c->b, sigma_inout, scratch, sweeps, &res, c->q[1]);
     if (s != IGR_OK) return s;
     if (res != sigma_inout)
         CU(c, cudaMemcpyAsync(sigma_inout, res, c->g.n * (size_t)c->ops->storage_bytes,
@@ -1649,8 +1660,10 @@ igr_status igr_adjoint_step(igr_ctx *c, const void *q_n, const void *sigma_n, co
     CU(c, cudaMemcpyAsync(it(0, 0), sigma_n, n * sb, cudaMemcpyDeviceToDevice, c->st));
     for (int st = 0; st < 3; st++) {
         CU(c, o->source(c->g, c->p, c->tiles, inflow_of(c), qs[st], nullptr, A.b, nullptr, c->st));
+        if (o->sweep) CU(c, o->coefs(c->g, c->p, qs[st], c->q[1], c->st));
         for (int k = 0; k < S; k++)
-            CU(c, o->jacobi(c->g, c->p, c->tiles, qs[st], A.b, it(st, k), it(st, k + 1), -1, c->st));
+            CU(c, o->sweep ? o->sweep(c->g, c->q[1], A.b, it(st, k), it(st, k + 1), -1, c->st)
+                           : o->jacobi(c->g, c->p, c->tiles, qs[st], A.b, it(st, k), it(st, k + 1), -1, c->st));
         if (st < 2) {
             CU(c, o->flux(c->g, c->p, c->tiles, inflow_of(c), st == 0 ? FLUX_STAGE1 : FLUX_STAGE2, qs[st],
                           nullptr, it(st, S), q_n, (void *)qs[st + 1], nullptr, nullptr, A.sc, c->blockmax,

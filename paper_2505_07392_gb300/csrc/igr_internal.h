@@ -218,6 +218,11 @@ struct Ops {
     // their registers allow (for the choice of the z-chunks)
     void (*source_shape)(const Geom &, long long *cols, int *resident);
     void (*jacobi_shape)(const Geom &, long long *cols, int *resident);
+    // FP64 (NULL in the other modes): the sweeps' coefficients of the density q into
+    // coefs (5 n scratch values), and a sweep with them; arguments and results as jacobi
+    cudaError_t (*coefs)(const Geom &, const Phys &, const void *q, void *coefs, cudaStream_t st);
+    cudaError_t (*sweep)(const Geom &, const void *coefs, const void *b, const void *s_in, void *s_out, int colour,
+                         cudaStream_t st);
 };
 
 // One instance's arguments of a grouped launch (the same as the single

@@ -1207,6 +1207,111 @@ __global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS) k_jacobi_pairs(const S
     jacobi_pairs(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), R, SG);
 }
 
+// FP64 sweeps from stored coefficients. An FP64 instruction holds an SM's units
+// for 16 cycles here, so the sweeps above are bound by the 40 or so that a cell
+// takes (two divisions, 14 for the faces, 6 for the diagonal). None of these
+// depend on Sigma, so where 5 n scratch values are free (a context's RK buffers)
+// they are formed once per stage: the three low-face factors, the diagonal d and
+// its inverse. That leaves 10: the sum and num / d by the inverse with one
+// remainder step (Markstein, IBM J. R&D 34, 1990), which gives the division's
+// rounding, so the results are those of the sweeps above. All else is free
+// beside the FP64 units (64 bytes per cell from memory take half their time):
+// one thread per cell, neighbours from L1, no alignment and no tile shape.
+// 96^3: 82 us per sweep above, 17.6 here and 42 per stage for the coefficients;
+// 48^3: 27, 3.8 and 10.
+template <class T> struct Coefs {
+    T *cx, *cy, *cz, *d, *inv;
+};
+// a cell, its neighbours (wrapped) and whether the faces to them exist
+struct Stencil {
+    idx c, xl, xh, yl, yh, zl, zh;
+    bool hxl, hxh, hyl, hyh, hzl, hzh;
+};
+__device__ __forceinline__ Stencil stencil_of(int i, int j, int k, const Geom &g)
+{
+    const bool px = g.bc[0] == BC_PERIODIC, py = g.bc[2] == BC_PERIODIC, pz = g.bc[4] == BC_PERIODIC;
+    const idx nx = (idx)g.nx, pl = (idx)g.plane;
+    Stencil t;
+    t.c = (idx)k * pl + (idx)j * nx + (idx)i;
+    t.xl = i > 0 ? t.c - 1 : t.c + (nx - 1);
+    t.xh = i + 1 < g.nx ? t.c + 1 : t.c - (nx - 1);
+    t.yl = j > 0 ? t.c - nx : t.c + (pl - nx);
+    t.yh = j + 1 < g.ny ? t.c + nx : t.c - (pl - nx);
+    t.zl = k > 0 ? t.c - pl : t.c + (idx)(g.nz - 1) * pl;
+    t.zh = k + 1 < g.nz ? t.c + pl : t.c - (idx)(g.nz - 1) * pl;
+    t.hxl = px || i > 0;
+    t.hxh = px || i + 1 < g.nx;
+    t.hyl = py || j > 0;
+    t.hyh = py || j + 1 < g.ny;
+    t.hzl = pz || k > 0;
+    t.hzh = pz || k + 1 < g.nz;
+    return t;
+}
+// fn(i, j, k) over the cells (colour >= 0: those of that colour), one per
+// thread and plane: blocks of 256 along a plane (x), planes over y
+template <class F> __device__ __forceinline__ void for_cells(const Geom &g, int colour, F fn)
+{
+    const unsigned w = colour < 0 ? g.nx : (g.nx + 1) / 2, p = blockIdx.x * 256u + threadIdx.x;
+    const int j = (int)(p / w), h = (int)(p % w);
+    if (j >= g.ny) return;
+    for (int k = blockIdx.y; k < g.nz; k += gridDim.y) {
+        const int i = colour < 0 ? h : 2 * h + ((colour + j + k) & 1);
+        if (i < g.nx) fn(i, j, k);
+    }
+}
+template <class T> __global__ void __launch_bounds__(256) k_coef_rcp(const T *__restrict__ q, T *r, Geom g)
+{
+    for_cells(g, -1, [&](int i, int j, int k) {
+        const idx c = ck((idx)k * (idx)g.plane + (idx)j * (idx)g.nx + (idx)i, g.n);
+        r[c] = rcp(q[c]);
+    });
+}
+// 1 / rho is in a.d
+template <class T> __global__ void __launch_bounds__(256) k_coef_faces(Coefs<T> a, Geom g, T hb)
+{
+    for_cells(g, -1, [&](int i, int j, int k) {
+        const Stencil t = stencil_of(i, j, k, g);
+        const idx c = ck(t.c, g.n);
+        const T r = a.d[c];
+        a.cx[c] = t.hxl ? mul_rn(hb, add_rn(r, a.d[ck(t.xl, g.n)])) : T(0);
+        a.cy[c] = t.hyl ? mul_rn(hb, add_rn(r, a.d[ck(t.yl, g.n)])) : T(0);
+        a.cz[c] = t.hzl ? mul_rn(hb, add_rn(r, a.d[ck(t.zl, g.n)])) : T(0);
+    });
+}
+// the diagonal in place of 1 / rho, and its inverse (an outer face has the factor 0)
+template <class T> __global__ void __launch_bounds__(256) k_coef_diag(Coefs<T> a, Geom g)
+{
+    for_cells(g, -1, [&](int i, int j, int k) {
+        const Stencil t = stencil_of(i, j, k, g);
+        const idx c = ck(t.c, g.n);
+        T d = add_rn(add_rn(a.d[c], a.cx[c]), a.cx[ck(t.xh, g.n)]);
+        d = add_rn(add_rn(d, a.cy[c]), a.cy[ck(t.yh, g.n)]);
+        d = add_rn(add_rn(d, a.cz[c]), a.cz[ck(t.zh, g.n)]);
+        a.d[c] = d;
+        a.inv[c] = rcp(d);
+    });
+}
+// (RB: s_in == s_out; a launch reads the cells of the other colour)
+template <class T>
+__global__ void __launch_bounds__(256) k_sweep(Coefs<const T> a, const T *__restrict__ b, const T *sin, T *sout, Geom g,
+                                              int colour)
+{
+    for_cells(g, colour, [&](int i, int j, int k) {
+        const Stencil t = stencil_of(i, j, k, g);
+        const idx c = ck(t.c, g.n), xh = ck(t.xh, g.n), yh = ck(t.yh, g.n), zh = ck(t.zh, g.n);
+        auto s = [&](bool face, idx at) { return face ? sin[ck(at, g.n)] : T(0); };
+        T off = mul_rn(__ldg(a.cx + c), s(t.hxl, t.xl));
+        off = fma_rn(__ldg(a.cx + xh), s(t.hxh, t.xh), off);
+        off = fma_rn(__ldg(a.cy + c), s(t.hyl, t.yl), off);
+        off = fma_rn(__ldg(a.cy + yh), s(t.hyh, t.yh), off);
+        off = fma_rn(__ldg(a.cz + c), s(t.hzl, t.zl), off);
+        off = fma_rn(__ldg(a.cz + zh), s(t.hzh, t.zh), off);
+        const T num = add_rn(__ldg(b + c), off), y = __ldg(a.inv + c), v = mul_rn(num, y);
+        const T rem = fma_rn(-__ldg(a.d + c), v, num);  // NaN where num or d is infinite: v is the quotient then
+        sout[c] = (__double2hiint(rem) & 0x7ff00000) == 0x7ff00000 ? v : fma_rn(rem, y, v);
+    });
+}
+
 // --------------------------------------------------------------- source
 // b = alpha [tr(G^2) + tr(G)^2] (Eq. igrelliptic) from the undivided central
 // differences D = 2 dx G of u, with alpha_s = alpha / (2 dx)^2:
@@ -3378,6 +3483,47 @@ cudaError_t launch_jacobi(const Geom &g, const Phys &p, const Tiles &t, const vo
     return cudaGetLastError();
 }
 
+template <class T> Coefs<T> coefs_at(void *p, long long n)
+{
+    T *a = (T *)p;
+    return {a, a + n, a + 2 * n, a + 3 * n, a + 4 * n};
+}
+dim3 cells_grid(const Geom &g, int colour)
+{
+    const long long w = colour < 0 ? g.nx : (g.nx + 1) / 2;
+    return dim3((unsigned)((w * g.ny + 255) / 256), (unsigned)std::min(g.nz, 65535));
+}
+template <class T>
+cudaError_t launch_coefs(const Geom &g, const Phys &p, const void *q, void *coefs, cudaStream_t st)
+{
+    const Coefs<T> a = coefs_at<T>(coefs, g.n);
+    const dim3 gr = cells_grid(g, -1);
+    k_coef_rcp<T><<<gr, 256, 0, st>>>((const T *)q, a.d, g);
+    k_coef_faces<T><<<gr, 256, 0, st>>>(a, g, T(0.5) * T(p.alpha / (p.dx * p.dx)));
+    k_coef_diag<T><<<gr, 256, 0, st>>>(a, g);
+    return cudaGetLastError();
+}
+template <class T>
+cudaError_t launch_sweep(const Geom &g, const void *coefs, const void *b, const void *s_in, void *s_out, int colour,
+                         cudaStream_t st)
+{
+    const Coefs<T> a = coefs_at<T>((void *)coefs, g.n);
+    k_sweep<T><<<cells_grid(g, colour), 256, 0, st>>>({a.cx, a.cy, a.cz, a.d, a.inv}, (const T *)b, (const T *)s_in,
+                                                      (T *)s_out, g, colour);
+    return cudaGetLastError();
+}
+// Ops::coefs and Ops::sweep: FP64 only
+template <class T> constexpr auto coefs_op()
+{
+    if constexpr (sizeof(T) == 8) return &launch_coefs<T>;
+    else return nullptr;
+}
+template <class T> constexpr auto sweep_op()
+{
+    if constexpr (sizeof(T) == 8) return &launch_sweep<T>;
+    else return nullptr;
+}
+
 long long flux_blocks(const Geom &g, const Tiles &t)
 {
     dim3 gr = grid_of(g, TX, TY, t.zc_flux);
@@ -3818,6 +3964,7 @@ extern const Ops IGR_OPS = {
     launch_adj_add, launch_adj_jets, launch_adj_rk, launch_adj_rhs_scatter, launch_adj_rho,
     launch_adj_source_scatter, launch_diag, bounds_hits, bounds_selftest,
     launch_source_group, launch_jacobi_group, launch_flux_group, source_shape, jacobi_shape,
+    coefs_op<S>(), sweep_op<S>(),
 };
 
 }  // namespace igr
