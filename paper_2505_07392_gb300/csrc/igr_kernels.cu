@@ -1182,6 +1182,8 @@ __device__ __forceinline__ void jacobi_pairs(const S *__restrict__ q, const S *_
 // resident blocks per SM that the registers are held to
 template <int NR> constexpr int kJacobiBlocks = sizeof(S) == 8 ? 1 : sizeof(S) == 2 && NR == 1 ? 3 : 2;
 constexpr int JACOBI_FIT_BLOCKS = sizeof(C) == 8 ? 1 : 2;
+// four blocks of pairs (1022 x 255 x 255 FP32: 265 us; five: 252, six: 342; but
+// 254 x 201 x 130: 34.7, 36.9 and 45.1)
 constexpr int JACOBI_PAIR_BLOCKS = sizeof(C) == 8 ? 2 : 4;
 template <bool RB, int NR>
 __global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full(const S *__restrict__ q, const S *__restrict__ b,
@@ -1217,8 +1219,6 @@ __global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS) k_jacobi_pairs(const S
 // rounding, so the results are those of the sweeps above. All else is free
 // beside the FP64 units (64 bytes per cell from memory take half their time):
 // one thread per cell, neighbours from L1, no alignment and no tile shape.
-// 96^3: 82 us per sweep above, 17.6 here and 42 per stage for the coefficients;
-// 48^3: 27, 3.8 and 10.
 template <class T> struct Coefs {
     T *cx, *cy, *cz, *d, *inv;
 };
@@ -1621,8 +1621,13 @@ __global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source(QIn q, S *__restri
     __shared__ __align__(16) C U2[SOURCE_BUFS * 3 * TILEV];
     source_quads<HASD, FULL>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch(), wq, rows, U2);
 }
+// The pairs wait on latency more (element loads, 24 per thread and plane in the
+// increment modes): four blocks (64 registers, a few spilled) against three and
+// two, 510 x 399 x 200: FP32 196, 221 and 262 us, BF16 increments 328, 378 and
+// 448; only the smallest grids prefer fewer (33 x 35 x 37: 11.4, 10.5, 9.9).
+constexpr int SOURCE_PAIR_BLOCKS = sizeof(C) == 8 ? 1 : 4;
 template <bool HASD>
-__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_pairs(QIn q, S *__restrict__ b, S *__restrict__ rho_out,
+__global__ void __launch_bounds__(32 * PWARPS, SOURCE_PAIR_BLOCKS) k_source_pairs(QIn q, S *__restrict__ b, S *__restrict__ rho_out,
                                                                     Geom g, C alpha_s, const C *W, const C *J, int zc)
 {
     __shared__ C U2[2 * 3 * TILEP];
@@ -3316,7 +3321,7 @@ __global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_group(const __grid
                              BlockPos::of_index(blockIdx.x - d.blk0, d.gx, d.gy), d.wq, d.rows, U2);
 }
 template <bool HASD>
-__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_pairs_group(const __grid_constant__ Group<SourceInst> a)
+__global__ void __launch_bounds__(32 * PWARPS, SOURCE_PAIR_BLOCKS) k_source_pairs_group(const __grid_constant__ Group<SourceInst> a)
 {
     __shared__ C U2[2 * 3 * TILEP];
     const SourceInst &d = a.d[group_find(a, blockIdx.x)];
@@ -3420,7 +3425,7 @@ void source_shape(const Geom &g, long long *cols, int *resident)
     const int form = quad_form(g, Tiles{});
     const dim3 gr = quad_grid(g, form, g.nz);
     *cols = (long long)gr.x * gr.y;
-    *resident = (sizeof(C) == 8 ? 256 : 512) / quad_threads(g, form);
+    *resident = !form ? SOURCE_PAIR_BLOCKS : (sizeof(C) == 8 ? 256 : 512) / quad_threads(g, form);
 }
 void jacobi_shape(const Geom &g, long long *cols, int *resident)
 {
