@@ -179,6 +179,7 @@ __device__ __forceinline__ void finalize_dt_body(const double *blockmax, int nbl
 __global__ void k_finalize_dt(const double *blockmax, int nblocks, Scalars *sc, double cfl_dx,
                               double fixed_dt)
 {
+    launched();
     finalize_dt_body(blockmax, nblocks, sc, cfl_dx, fixed_dt);
 }
 
@@ -195,6 +196,7 @@ struct DtGroup {
 };
 __global__ void k_finalize_dt_group(const __grid_constant__ DtGroup a)
 {
+    launched();
     const DtInst &d = a.d[blockIdx.x];
     finalize_dt_body(d.blockmax, d.nblocks, d.sc, d.cfl_dx, 0.0);
 }
@@ -820,9 +822,8 @@ igr_status igr_get_state(igr_ctx *c, void *q, void *sigma, igr_dtype dtype, int 
 static igr_status finalize_dt(igr_ctx *c, double fixed_dt)
 {
     prof_begin(c, KC_OTHER);
-    k_finalize_dt<<<1, dt_threads(c->speed_nblocks), 0, c->st>>>(c->blockmax, c->speed_nblocks, c->sc, c->cfg.cfl * c->cfg.dx,
-                                        fixed_dt);
-    CU(c, cudaGetLastError());
+    CU(c, launch(k_finalize_dt, 1, dt_threads(c->speed_nblocks), 0, c->st, c->blockmax, c->speed_nblocks, c->sc,
+                 c->cfg.cfl * c->cfg.dx, fixed_dt));
     prof_end(c);
     return IGR_OK;
 }
@@ -991,8 +992,8 @@ igr_status igr_get_dt(igr_ctx *c, double *dt)
     // reduce into the second scalar slot so the step's scalars are untouched
     Scalars *tmp = c->sc + 1;
     CU(c, cudaMemsetAsync(tmp, 0, sizeof(Scalars), c->st));
-    k_finalize_dt<<<1, dt_threads(c->speed_nblocks), 0, c->st>>>(c->blockmax, c->speed_nblocks, tmp, c->cfg.cfl * c->cfg.dx, 0.0);
-    CU(c, cudaGetLastError());
+    CU(c, launch(k_finalize_dt, 1, dt_threads(c->speed_nblocks), 0, c->st, c->blockmax, c->speed_nblocks, tmp,
+                 c->cfg.cfl * c->cfg.dx, 0.0));
     Scalars h;
     CU(c, cudaMemcpyAsync(&h, tmp, sizeof(Scalars), cudaMemcpyDeviceToHost, c->st));
     CU(c, cudaStreamSynchronize(c->st));
@@ -1260,8 +1261,7 @@ static igr_status step_grouped(igr_batch *b)
             a.d[i] = {c->blockmax, c->speed_nblocks, c->sc, c->cfg.cfl * c->cfg.dx};
             threads = std::max(threads, dt_threads(c->speed_nblocks));
         }
-        k_finalize_dt_group<<<a.count, threads, 0, st>>>(a);
-        if (cudaGetLastError() != cudaSuccess) return bfail(b, IGR_ERR_CUDA, "grouped dt launch");
+        if (launch(k_finalize_dt_group, a.count, threads, 0, st, a) != cudaSuccess) return bfail(b, IGR_ERR_CUDA, "grouped dt launch");
     }
     int maxs = 0;
     for (igr_ctx *c : b->inst) maxs = std::max(maxs, c->cfg.sweeps);

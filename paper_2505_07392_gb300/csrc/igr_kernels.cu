@@ -1190,6 +1190,7 @@ __global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full(const S *
                                                                   const S *sin, S *sout, Geom g, C beta, int zc,
                                                                   int colour)
 {
+    launched();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     jacobi_quads<true, RB, NR>(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), FQ, FR, smem_raw);
 }
@@ -1197,6 +1198,7 @@ __global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit(const S *_
                                                                      const S *sin, S *sout, Geom g, C beta, int zc,
                                                                      int colour, int wq, int rows)
 {
+    launched();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     jacobi_quads<false, false, 1>(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), wq, rows, smem_raw);
 }
@@ -1204,6 +1206,7 @@ __global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS) k_jacobi_pairs(const S
                                                                         const S *__restrict__ b, const S *sin,
                                                                         S *sout, Geom g, C beta, int zc, int colour)
 {
+    launched();
     __shared__ C R[2 * TILEP];
     __shared__ C SG[2 * TILEP];
     jacobi_pairs(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), R, SG);
@@ -1261,6 +1264,7 @@ template <class F> __device__ __forceinline__ void for_cells(const Geom &g, int 
 }
 template <class T> __global__ void __launch_bounds__(256) k_coef_rcp(const T *__restrict__ q, T *r, Geom g)
 {
+    launched();
     for_cells(g, -1, [&](int i, int j, int k) {
         const idx c = ck((idx)k * (idx)g.plane + (idx)j * (idx)g.nx + (idx)i, g.n);
         r[c] = rcp(q[c]);
@@ -1269,6 +1273,7 @@ template <class T> __global__ void __launch_bounds__(256) k_coef_rcp(const T *__
 // 1 / rho is in a.d
 template <class T> __global__ void __launch_bounds__(256) k_coef_faces(Coefs<T> a, Geom g, T hb)
 {
+    launched();
     for_cells(g, -1, [&](int i, int j, int k) {
         const Stencil t = stencil_of(i, j, k, g);
         const idx c = ck(t.c, g.n);
@@ -1281,6 +1286,7 @@ template <class T> __global__ void __launch_bounds__(256) k_coef_faces(Coefs<T> 
 // the diagonal in place of 1 / rho, and its inverse (an outer face has the factor 0)
 template <class T> __global__ void __launch_bounds__(256) k_coef_diag(Coefs<T> a, Geom g)
 {
+    launched();
     for_cells(g, -1, [&](int i, int j, int k) {
         const Stencil t = stencil_of(i, j, k, g);
         const idx c = ck(t.c, g.n);
@@ -1296,6 +1302,7 @@ template <class T>
 __global__ void __launch_bounds__(256) k_sweep(Coefs<const T> a, const T *__restrict__ b, const T *sin, T *sout, Geom g,
                                               int colour)
 {
+    launched();
     for_cells(g, colour, [&](int i, int j, int k) {
         const Stencil t = stencil_of(i, j, k, g);
         const idx c = ck(t.c, g.n), xh = ck(t.xh, g.n), yh = ck(t.yh, g.n), zh = ck(t.zh, g.n);
@@ -1618,6 +1625,7 @@ __global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source(QIn q, S *__restri
                                                               C alpha_s, const C *W, const C *J, int zc, int wq,
                                                               int rows)
 {
+    launched();
     __shared__ __align__(16) C U2[SOURCE_BUFS * 3 * TILEV];
     source_quads<HASD, FULL>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch(), wq, rows, U2);
 }
@@ -1630,6 +1638,7 @@ template <bool HASD>
 __global__ void __launch_bounds__(32 * PWARPS, SOURCE_PAIR_BLOCKS) k_source_pairs(QIn q, S *__restrict__ b, S *__restrict__ rho_out,
                                                                     Geom g, C alpha_s, const C *W, const C *J, int zc)
 {
+    launched();
     __shared__ C U2[2 * 3 * TILEP];
     source_pairs<HASD>(q, b, rho_out, g, alpha_s, W, J, zc, BlockPos::of_launch(), U2);
 }
@@ -2276,6 +2285,7 @@ __global__ void __maxnreg__(FLUX_MAXREG)
            Geom g, C gamma, C half_inv_dx, const Scalars *sc, double *blockmax, int *err, const C *W,
            const C *J, int zc, int cz0, C mu, C lamv)
 {
+    launched();
     flux_body<mode, ORD, VISC>(qin, sig, qn, out, outb, rhs, base_out, g, gamma, half_inv_dx, sc, blockmax, err,
                                W, J, zc, cz0, mu, lamv, BlockPos::of_launch());
 }
@@ -2314,6 +2324,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(SPEED_NT) k_speed(const QB *__restrict__ q, long long n, C gamma,
                                                      double *blockmax)
 {
+    launched();
     C m = C(0);
     const C gm1 = gamma - C(1);
     auto take = [&](C rho, C mx, C my, C mz, C E) {
@@ -3315,6 +3326,7 @@ template <class I> __device__ __forceinline__ int group_find(const Group<I> &a, 
 template <bool HASD, bool FULL>
 __global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_group(const __grid_constant__ Group<SourceInst> a)
 {
+    launched();
     __shared__ __align__(16) C U2[SOURCE_BUFS * 3 * TILEV];
     const SourceInst &d = a.d[group_find(a, blockIdx.x)];
     source_quads<HASD, FULL>(d.q, d.b, d.rho_out, d.g, d.alpha_s, d.W, d.J, d.zc,
@@ -3323,6 +3335,7 @@ __global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source_group(const __grid
 template <bool HASD>
 __global__ void __launch_bounds__(32 * PWARPS, SOURCE_PAIR_BLOCKS) k_source_pairs_group(const __grid_constant__ Group<SourceInst> a)
 {
+    launched();
     __shared__ C U2[2 * 3 * TILEP];
     const SourceInst &d = a.d[group_find(a, blockIdx.x)];
     source_pairs<HASD>(d.q, d.b, d.rho_out, d.g, d.alpha_s, d.W, d.J, d.zc,
@@ -3332,6 +3345,7 @@ template <bool RB, int NR>
 __global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full_group(const __grid_constant__ Group<JacobiInst> a,
                                                                         int colour)
 {
+    launched();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const JacobiInst &d = a.d[group_find(a, blockIdx.x)];
     jacobi_quads<true, RB, NR>(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
@@ -3340,6 +3354,7 @@ __global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full_group(con
 __global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit_group(const __grid_constant__ Group<JacobiInst> a,
                                                                            int colour)
 {
+    launched();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const JacobiInst &d = a.d[group_find(a, blockIdx.x)];
     jacobi_quads<false, false, 1>(d.q, d.b, d.sin, d.sout, d.g, d.beta, d.zc, colour,
@@ -3348,6 +3363,7 @@ __global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit_group(cons
 __global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS)
     k_jacobi_pairs_group(const __grid_constant__ Group<JacobiInst> a, int colour)
 {
+    launched();
     __shared__ C R[2 * TILEP];
     __shared__ C SG[2 * TILEP];
     const JacobiInst &d = a.d[group_find(a, blockIdx.x)];
@@ -3357,6 +3373,7 @@ __global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS)
 template <int mode, int ORD, bool VISC>
 __global__ void __maxnreg__(FLUX_MAXREG) k_flux_group(const __grid_constant__ Group<FluxInst> a)
 {
+    launched();
     const FluxInst &d = a.d[group_find(a, blockIdx.x)];
     const Frhs none_rhs = {};
     const Fout<5> none_base = {};
@@ -3450,12 +3467,11 @@ cudaError_t launch_source(const Geom &g, const Phys &p, const Tiles &t, const In
     if (form) {
         auto kern = source_full(form) ? (qd ? k_source<kInc, true> : k_source<false, true>)
                               : (qd ? k_source<kInc, false> : k_source<false, false>);
-        kern<<<gr, threads, 0, st>>>(qi, (S *)b, (S *)rho_out, g, as, W, J, t.zc_source, f.wq, f.rows);
+        return launch(kern, gr, threads, 0, st, qi, (S *)b, (S *)rho_out, g, as, W, J, t.zc_source, f.wq, f.rows);
     } else {
         auto kern = qd ? k_source_pairs<kInc> : k_source_pairs<false>;
-        kern<<<gr, threads, 0, st>>>(qi, (S *)b, (S *)rho_out, g, as, W, J, t.zc_source);
+        return launch(kern, gr, threads, 0, st, qi, (S *)b, (S *)rho_out, g, as, W, J, t.zc_source);
     }
-    return cudaGetLastError();
 }
 
 constexpr int kRows = sizeof(S) == 2 ? 2 : 1;  // rows per thread of form 3
@@ -3477,15 +3493,15 @@ cudaError_t launch_jacobi(const Geom &g, const Phys &p, const Tiles &t, const vo
         const int smem = form == 3 ? JShape<kRows>::SMEM : JShape<1>::SMEM;
         cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        kern<<<gr, threads, smem, st>>>(qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour);
+        return launch(kern, gr, threads, smem, st, qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour);
     } else if (form) {
         cudaError_t e = allow_smem(k_jacobi_fit, JShape<1>::SMEM);
         if (e != cudaSuccess) return e;
-        k_jacobi_fit<<<gr, threads, JShape<1>::SMEM, st>>>(qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour, f.wq, f.rows);
+        return launch(k_jacobi_fit, gr, threads, JShape<1>::SMEM, st, qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi,
+                      colour, f.wq, f.rows);
     } else {
-        k_jacobi_pairs<<<gr, threads, 0, st>>>(qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour);
+        return launch(k_jacobi_pairs, gr, threads, 0, st, qs, bs, si, (S *)s_out, g, beta, t.zc_jacobi, colour);
     }
-    return cudaGetLastError();
 }
 
 template <class T> Coefs<T> coefs_at(void *p, long long n)
@@ -3503,19 +3519,17 @@ cudaError_t launch_coefs(const Geom &g, const Phys &p, const void *q, void *coef
 {
     const Coefs<T> a = coefs_at<T>(coefs, g.n);
     const dim3 gr = cells_grid(g, -1);
-    k_coef_rcp<T><<<gr, 256, 0, st>>>((const T *)q, a.d, g);
-    k_coef_faces<T><<<gr, 256, 0, st>>>(a, g, T(0.5) * T(p.alpha / (p.dx * p.dx)));
-    k_coef_diag<T><<<gr, 256, 0, st>>>(a, g);
-    return cudaGetLastError();
+    cudaError_t e = launch(k_coef_rcp<T>, gr, 256, 0, st, (const T *)q, a.d, g);
+    if (e == cudaSuccess) e = launch(k_coef_faces<T>, gr, 256, 0, st, a, g, T(0.5) * T(p.alpha / (p.dx * p.dx)));
+    return e == cudaSuccess ? launch(k_coef_diag<T>, gr, 256, 0, st, a, g) : e;
 }
 template <class T>
 cudaError_t launch_sweep(const Geom &g, const void *coefs, const void *b, const void *s_in, void *s_out, int colour,
                          cudaStream_t st)
 {
     const Coefs<T> a = coefs_at<T>((void *)coefs, g.n);
-    k_sweep<T><<<cells_grid(g, colour), 256, 0, st>>>({a.cx, a.cy, a.cz, a.d, a.inv}, (const T *)b, (const T *)s_in,
-                                                      (T *)s_out, g, colour);
-    return cudaGetLastError();
+    const Coefs<const T> k = {a.cx, a.cy, a.cz, a.d, a.inv};
+    return launch(k_sweep<T>, cells_grid(g, colour), 256, 0, st, k, (const T *)b, (const T *)s_in, (T *)s_out, g, colour);
 }
 // Ops::coefs and Ops::sweep: FP64 only
 template <class T> constexpr auto coefs_op()
@@ -3565,10 +3579,9 @@ cudaError_t launch_flux(const Geom &g, const Phys &p, const Tiles &t, const Infl
         dim3 gr = grid_of(g, TX, TY, t.zc_flux);
         const int cz0 = t.z_begin / t.zc_flux;
         if (t.z_end > 0) gr.z = (t.z_end - t.z_begin + t.zc_flux - 1) / t.zc_flux;
-        kern<<<gr, NT, smem, st>>>(fi, (const S *)sig, fn, fo, fob, fr, fb, g, C(p.gamma), C(0.5 / p.dx), sc,
+        e = launch(kern, gr, NT, smem, st, fi, (const S *)sig, fn, fo, fob, fr, fb, g, C(p.gamma), C(0.5 / p.dx), sc,
                                    blockmax, err, (const C *)in.W, (const C *)in.J, t.zc_flux, cz0, C(p.mu),
                                    C(p.zeta - 2.0 * p.mu / 3.0));
-        e = cudaGetLastError();
         if (e != cudaSuccess) {
             cudaFuncAttributes fa;
             if (cudaFuncGetAttributes(&fa, kern) == cudaSuccess)
@@ -3653,8 +3666,7 @@ cudaError_t launch_source_group(const SourceCall *calls, int n, cudaStream_t st)
         auto kern = source_full(form) ? (cs[0].qd ? k_source_group<kInc, true> : k_source_group<false, true>)
                     : form ? (cs[0].qd ? k_source_group<kInc, false> : k_source_group<false, false>)
                            : (cs[0].qd ? k_source_pairs_group<kInc> : k_source_pairs_group<false>);
-        kern<<<blk, threads, 0, st>>>(a);
-        return cudaGetLastError();
+        return launch(kern, blk, threads, 0, st, a);
     });
 }
 
@@ -3691,8 +3703,7 @@ cudaError_t launch_jacobi_group(const JacobiCall *calls, int n, int colour, cuda
         const int smem = form == 3 ? JShape<kRows>::SMEM : form ? JShape<1>::SMEM : 0;
         cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        kern<<<blk, threads, smem, st>>>(a, colour);
-        return cudaGetLastError();
+        return launch(kern, blk, threads, smem, st, a, colour);
     });
 }
 
@@ -3742,8 +3753,7 @@ cudaError_t launch_flux_group(const FluxCall *calls, int n, int mode, cudaStream
         auto go = [&](auto kern) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            kern<<<blk, NT, smem, st>>>(a);
-            return cudaGetLastError();
+            return launch(kern, blk, NT, smem, st, a);
         };
         auto by_mode = [&](auto k1, auto k2, auto k3) {
             return mode == FLUX_STAGE1 ? go(k1) : mode == FLUX_STAGE2 ? go(k2) : go(k3);
@@ -3772,9 +3782,8 @@ cudaError_t launch_speed(const Geom &g, const Phys &p, const void *q, double *bl
     const long long want = (g.n / (vec ? 4 : 1) + SPEED_NT - 1) / SPEED_NT;
     const int nb = (int)std::min<long long>(want, SPEED_MAXBLOCKS);
     auto kern = vec ? k_speed<true> : k_speed<false>;
-    kern<<<nb, SPEED_NT, 0, st>>>((const QB *)q, g.n, C(p.gamma), blockmax);
     *nblocks = nb;
-    return cudaGetLastError();
+    return launch(kern, nb, SPEED_NT, 0, st, (const QB *)q, g.n, C(p.gamma), blockmax);
 }
 
 cudaError_t launch_rk_combine(const void *qn, const void *qs, const void *L, void *out,
