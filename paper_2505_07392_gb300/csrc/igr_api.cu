@@ -435,13 +435,14 @@ static Inflow inflow_of(igr_ctx *c)
 // scratch values in the state type, for FP64's stored coefficients (from the
 // first sweep on: forming them costs less than one sweep without).
 static igr_status launch_sweeps(igr_ctx *c, const Tiles &t, const void *q, const void *b,
-                                void *s_first, void *s_other, int sweeps, void **result, void *coefs)
+                                void *s_first, void *s_other, int sweeps, void **result, void *coefs,
+                                cudaStream_t st)
 {
     const Ops *o = c->ops;
     auto sweep = [&](const void *s_in, void *s_out, int colour, bool first) -> cudaError_t {
-        if (!o->sweep) return o->jacobi(c->g, c->p, t, q, b, s_in, s_out, colour, c->st);
-        cudaError_t e = first ? o->coefs(c->g, c->p, q, coefs, c->st) : cudaSuccess;
-        return e == cudaSuccess ? o->sweep(c->g, coefs, b, s_in, s_out, colour, c->st) : e;
+        if (!o->sweep) return o->jacobi(c->g, c->p, t, q, b, s_in, s_out, colour, st);
+        cudaError_t e = first ? o->coefs(c->g, c->p, q, coefs, st) : cudaSuccess;
+        return e == cudaSuccess ? o->sweep(c->g, coefs, b, s_in, s_out, colour, st) : e;
     };
     if (c->cfg.sigma_solver == SOLVER_RBGS) {
         for (int it = 0; it < sweeps; it++)
@@ -466,6 +467,12 @@ static igr_status launch_sweeps(igr_ctx *c, const Tiles &t, const void *q, const
     return IGR_OK;
 }
 
+// scratch of a stage's sweeps: the flux's output, or where that is q^n (stage 3) stage 1's
+static void *sweep_scratch(const igr_ctx *c, const void *qs, const void *qn, void *out)
+{
+    return out != qs && out != qn ? out : c->q[1];
+}
+
 static igr_status refresh_speed(igr_ctx *c);
 static igr_status finalize_dt(igr_ctx *c, double fixed_dt);
 
@@ -488,10 +495,8 @@ static igr_status run_stage(igr_ctx *c, int mode, const void *qs, const void *qd
     // the sweeps read the density as field 0 of their q: the state itself, or
     // the stage density the source kernel stored (increment modes)
     const void *qj = c->inc ? c->rho16 : qs;
-    // scratch of the sweeps: the flux's output, or where that is q^n (stage 3) stage 1's
-    void *free5 = out != qs && out != qn ? out : c->q[1];
     igr_status s = launch_sweeps(c, c->tiles, qj, c->b, c->sig[c->cur], c->sig[1 - c->cur], c->cfg.sweeps, &res,
-                                 free5);
+                                 sweep_scratch(c, qs, qn, out), c->st);
     if (s != IGR_OK) return s;
     c->cur = res == c->sig[0] ? 0 : 1;
     if (q_ready) {
@@ -945,7 +950,8 @@ igr_status igr_solve_sigma(igr_ctx *c, const void *q, void *sigma_inout, int swe
     // the caller's buffer and it, and an odd count copies the result back
     void *scratch = c->sig[1 - c->cur];
     void *res;
-    igr_status s = launch_sweeps(c, t, c->inc ? c->rho16 : q, c->b, sigma_inout, scratch, sweeps, &res, c->q[1]);
+    igr_status s = launch_sweeps(c, t, c->inc ? c->rho16 : q, c->b, sigma_inout, scratch, sweeps, &res, c->q[1],
+                                 c->st);
     if (s != IGR_OK) return s;
     if (res != sigma_inout)
         CU(c, cudaMemcpyAsync(sigma_inout, res, c->g.n * (size_t)c->ops->storage_bytes,
@@ -1280,13 +1286,27 @@ static igr_status step_grouped(igr_batch *b)
                 }
             if (o->source_group(sc.data(), (int)sc.size(), st) != cudaSuccess)
                 return bfail(b, IGR_ERR_CUDA, "grouped source launch");
+            // FP64 from 32^3 cells: each instance's own sweeps on stored coefficients, a
+            // quarter of the grouped ones' operations for more launches (twelve
+            // instances of 32^3: 2545 us per step against 2769, four of 96^3: 13464
+            // against 16027; twelve of 16^3: 1099 against 991)
+            auto own = [&](const igr_ctx *c) { return o->sweep && c->g.n >= 32768; };
+            for (igr_ctx *c : inst) {
+                if (c->ops != o || !own(c)) continue;
+                const StageIO io = stage_io(c, stage);
+                void *res;
+                igr_status s = launch_sweeps(c, c->tiles, io.qs, c->b, c->sig[c->cur], c->sig[1 - c->cur], c->cfg.sweeps,
+                                             &res, sweep_scratch(c, io.qs, io.qn, io.out), st);
+                if (s != IGR_OK) return bfail(b, s, igr_last_error(c));
+                c->cur = res == c->sig[0] ? 0 : 1;
+            }
             // sweep k of every instance that makes at least k + 1 sweeps
             for (int k = 0; k < maxs; k++)
                 for (int colour = -1; colour < 2; colour++) {
                     jc.clear();
                     for (igr_ctx *c : inst) {
                         const bool rb = c->cfg.sigma_solver == SOLVER_RBGS;
-                        if (c->ops != o || k >= c->cfg.sweeps || (rb ? colour < 0 : colour >= 0)) continue;
+                        if (c->ops != o || own(c) || k >= c->cfg.sweeps || (rb ? colour < 0 : colour >= 0)) continue;
                         const void *qj = c->inc ? c->rho16 : stage_io(c, stage).qs;
                         void *src = c->sig[c->cur], *dst = rb ? src : c->sig[1 - c->cur];
                         jc.push_back({c->g, c->p, c->tiles, qj, c->b, src, dst});
@@ -1295,7 +1315,7 @@ static igr_status step_grouped(igr_batch *b)
                     if (o->jacobi_group(jc.data(), (int)jc.size(), colour, st) != cudaSuccess)
                         return bfail(b, IGR_ERR_CUDA, "grouped sweep launch");
                     for (igr_ctx *c : inst)  // Jacobi sweeps alternate the two Sigma buffers
-                        if (c->ops == o && k < c->cfg.sweeps && c->cfg.sigma_solver != SOLVER_RBGS && colour < 0)
+                        if (c->ops == o && !own(c) && k < c->cfg.sweeps && c->cfg.sigma_solver != SOLVER_RBGS && colour < 0)
                             c->cur = 1 - c->cur;
                 }
             fc.clear();

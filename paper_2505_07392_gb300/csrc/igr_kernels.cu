@@ -3414,7 +3414,7 @@ template <class K> cudaError_t allow_smem(K kern, int bytes)
 
 // Kernel form of a source or sweep launch: 2 full quad tiles, 1 fitted quad
 // tiles, 0 pairs; a sweep's form 3: full tiles with two rows per thread
-// (16-bit storage; from 16M cells: FP16, 512 x 512 x 128: 74 us against 80
+// (16-bit storage; from 16M cells: FP16, 512 x 512 x 128: 73 us against 79
 // with one; 256 x 256 x 192: 32 against 29.5). Its grid and block.
 int quad_form(const Geom &g, const Tiles &t)
 {

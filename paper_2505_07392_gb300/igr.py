@@ -413,8 +413,8 @@ class Solver:
         return a.value, b.value, c.value
 
     def set_kernel_forms(self, source_vec4: int = -1, jacobi_vec4: int = -1):
-        """Forms of the source and Jacobi kernels: -1 default rule, 0 one
-        cell per thread, 1 four cells per thread (nx % 4 == 0)."""
+        """Accepted as -1, 0 or 1 (1: nx % 4 == 0) and returned by kernel_forms;
+        the kernels' form follows from the row length and the alignment."""
         self._check(lib().igr_set_kernel_forms(self.h, int(source_vec4), int(jacobi_vec4)))
 
     def kernel_forms(self):
