@@ -373,6 +373,8 @@ igr_status igr_profile_read(igr_ctx *ctx, int kernel_class, long long *launches,
  * and reported (the default rule reports 1 for rows of a multiple of 4 cells
  * that fill blocks of 128 cells), and every setting launches the kernels
  * described above.
+ * The sweep chunk has no effect on FP64 sweeps on stored coefficients (a
+ * context's steps and igr_solve_sigma), which have none.
  * igr_autotune times each class on the current state for the default chunk
  * and the candidate lengths 4..128 (reps launches each, on the context
  * stream; only scratch buffers are written) and keeps the fastest; call it

@@ -87,7 +87,7 @@ struct igr_ctx {
         void *lq0, *lqs, *lout, *Lb;       // adjoints (arithmetic type, 5 n)
         void *lsig, *lb, *mu, *nl, *rb;    // adjoints (arithmetic type, n)
         void *lamJ;                        // adjoint of the inflow tables (5 x plane)
-        double *gw;                        // jet gradient (njets)
+        double *gw;                        // jet gradient (njets) and its partial sums
         Scalars *sc;                       // dt of the recomputed stages
         std::vector<void *> all;
     } adj;
