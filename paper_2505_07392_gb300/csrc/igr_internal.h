@@ -113,11 +113,13 @@ inline size_t vec4_align(int storage_bytes) { return storage_bytes * 4 > 16 ? 16
 // Launches of a step's kernels (programmatic dependent launch). A kernel launched
 // by `launch` may be placed on the SMs once every block of the kernel before it
 // has begun, and waits in `launched`, its first statement, until that kernel has
-// completed and its writes are visible; so the order of all memory accesses is
-// that of plain launches, and only the launch itself overlaps. A kernel without
-// `launched` is launched plainly. The gap between two kernels was about 2 us,
-// most of a small grid's step: ten steps at 32^3 (220 launches) 1671 us before,
-// 1197 now; 254 x 201 x 130, 70 launches a two-step run: 3958 and 3820.
+// completed and its writes are visible to ordinary loads; so the order of all
+// memory accesses is that of plain launches, and only the launch itself overlaps.
+// Read-only loads (__ldg, const __restrict__) are not for such a kernel: the data
+// change during its lifetime. A kernel without `launched` is launched plainly.
+// The gap between two kernels was about 2 us, most of a small grid's step: ten
+// steps at 32^3 (220 launches) 1671 us before, 1197 now; 254 x 201 x 130, 70
+// launches a two-step run: 3958 and 3820.
 __device__ __forceinline__ void launched()
 {
     cudaGridDependencySynchronize();

@@ -143,15 +143,21 @@ struct QBIn { const QB *p[5]; };                  // the state q^n (RK base)
 struct QBOut { QB *p[5]; };                       // a new state q^n+1
 
 // ------------------------------------------------------------ load/store
+// Read-only (non-coherent) loads, for kernels that are launched plainly. A kernel
+// that begins with launched() is resident while its predecessor writes, so it
+// takes ordinary loads (ldr, ld4r, cp.async) and no __restrict__ pointers, and the
+// writes that it waited for are visible to them. They cost nothing: every case
+// within 0.5% of the read-only loads' time (plume 1024 x 1024 x 512, FP16
+// increments: 140.0 ms before, 139.7 now; ten steps at 32^3: 1200 and 1194 us).
 __device__ __forceinline__ double ldc(const double *p) { return __ldg(p); }
 __device__ __forceinline__ float ldc(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ldc(const __half *p) { return __half2float(__ldg(p)); }
 __device__ __forceinline__ float ldc(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
 
-// Raw loads for prefetching: the value stays in its storage type until it is
+// Raw (ordinary) loads for prefetching: the value stays in its storage type until it is
 // used, so no instruction waits on the load before then (a conversion right
 // after the load would stall there and hide nothing).
-__device__ __forceinline__ S ldr(const S *p) { return __ldg(p); }
+__device__ __forceinline__ S ldr(const S *p) { return *p; }
 __device__ __forceinline__ double cv(double v) { return v; }
 __device__ __forceinline__ float cv(float v) { return v; }
 __device__ __forceinline__ float cv(__half v) { return __half2float(v); }
@@ -184,7 +190,7 @@ template <> struct StateIO<true> {
     template <bool HASD> static __device__ __forceinline__ QRawInc ld(const QIn &q, int u, idx c)
     {
         QRawInc r;
-        r.b = __ldg(q.b[0] + u * q.fs + c);
+        r.b = q.b[0][u * q.fs + c];
         r.d = HASD ? ldr(q.d[0] + u * q.fs + c) : S(0.0f);
         return r;
     }
@@ -746,13 +752,13 @@ using V4 = Vec4<S>;
 
 __device__ __forceinline__ Vec4<double> ld4r(const double *p)
 {
-    return {__ldg(reinterpret_cast<const double2 *>(p)), __ldg(reinterpret_cast<const double2 *>(p) + 1)};
+    return {*reinterpret_cast<const double2 *>(p), reinterpret_cast<const double2 *>(p)[1]};
 }
-__device__ __forceinline__ Vec4<float> ld4r(const float *p) { return {__ldg(reinterpret_cast<const float4 *>(p))}; }
-__device__ __forceinline__ Vec4<__half> ld4r(const __half *p) { return {__ldg(reinterpret_cast<const uint2 *>(p))}; }
+__device__ __forceinline__ Vec4<float> ld4r(const float *p) { return {*reinterpret_cast<const float4 *>(p)}; }
+__device__ __forceinline__ Vec4<__half> ld4r(const __half *p) { return {*reinterpret_cast<const uint2 *>(p)}; }
 __device__ __forceinline__ Vec4<__nv_bfloat16> ld4r(const __nv_bfloat16 *p)
 {
-    return {__ldg(reinterpret_cast<const uint2 *>(p))};
+    return {*reinterpret_cast<const uint2 *>(p)};
 }
 __device__ __forceinline__ void cv4(const Vec4<double> &v, double o[4])
 {
@@ -889,9 +895,9 @@ template <int NR> struct JShape {
     static constexpr int SMEM = JRING * PLANE * (int)sizeof(S) + 2 * TILE * (int)(sizeof(C) + sizeof(S));
 };
 template <bool FULL, bool RB, int NR>
-__device__ __forceinline__ void jacobi_quads(const S *__restrict__ q, const S *__restrict__ b, const S *sin, S *sout,
-                                             const Geom &g, C beta, int zc, int colour, const BlockPos &bp, int wq,
-                                             int rows, unsigned char *smem)
+__device__ __forceinline__ void jacobi_quads(const S *q, const S *b, const S *sin, S *sout, const Geom &g, C beta,
+                                             int zc, int colour, const BlockPos &bp, int wq, int rows,
+                                             unsigned char *smem)
 {
     static_assert(FULL || NR == 1, "two rows per thread: full tiles");
     constexpr int JPLANE = JShape<NR>::PLANE, JTILE = JShape<NR>::TILE, HT = JShape<NR>::HT;
@@ -1096,7 +1102,7 @@ __device__ __forceinline__ void jacobi_quads(const S *__restrict__ q, const S *_
 
 // the pairs: one halo cell per thread of the first three warps, own values
 // one plane ahead
-__device__ __forceinline__ void jacobi_pairs(const S *__restrict__ q, const S *__restrict__ b, const S *sin, S *sout,
+__device__ __forceinline__ void jacobi_pairs(const S *q, const S *b, const S *sin, S *sout,
                                              const Geom &g, C beta, int zc, int colour, const BlockPos &bp, C *R2,
                                              C *S2)
 {
@@ -1186,7 +1192,7 @@ constexpr int JACOBI_FIT_BLOCKS = sizeof(C) == 8 ? 1 : 2;
 // 254 x 201 x 130: 34.7, 36.9 and 45.1)
 constexpr int JACOBI_PAIR_BLOCKS = sizeof(C) == 8 ? 2 : 4;
 template <bool RB, int NR>
-__global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full(const S *__restrict__ q, const S *__restrict__ b,
+__global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full(const S *q, const S *b,
                                                                   const S *sin, S *sout, Geom g, C beta, int zc,
                                                                   int colour)
 {
@@ -1194,7 +1200,7 @@ __global__ void __launch_bounds__(BT, kJacobiBlocks<NR>) k_jacobi_full(const S *
     extern __shared__ __align__(16) unsigned char smem_raw[];
     jacobi_quads<true, RB, NR>(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), FQ, FR, smem_raw);
 }
-__global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit(const S *__restrict__ q, const S *__restrict__ b,
+__global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit(const S *q, const S *b,
                                                                      const S *sin, S *sout, Geom g, C beta, int zc,
                                                                      int colour, int wq, int rows)
 {
@@ -1202,8 +1208,8 @@ __global__ void __launch_bounds__(BT, JACOBI_FIT_BLOCKS) k_jacobi_fit(const S *_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     jacobi_quads<false, false, 1>(q, b, sin, sout, g, beta, zc, colour, BlockPos::of_launch(), wq, rows, smem_raw);
 }
-__global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS) k_jacobi_pairs(const S *__restrict__ q,
-                                                                        const S *__restrict__ b, const S *sin,
+__global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS) k_jacobi_pairs(const S *q,
+                                                                        const S *b, const S *sin,
                                                                         S *sout, Geom g, C beta, int zc, int colour)
 {
     launched();
@@ -1262,7 +1268,7 @@ template <class F> __device__ __forceinline__ void for_cells(const Geom &g, int 
         if (i < g.nx) fn(i, j, k);
     }
 }
-template <class T> __global__ void __launch_bounds__(256) k_coef_rcp(const T *__restrict__ q, T *r, Geom g)
+template <class T> __global__ void __launch_bounds__(256) k_coef_rcp(const T *q, T *r, Geom g)
 {
     launched();
     for_cells(g, -1, [&](int i, int j, int k) {
@@ -1299,7 +1305,7 @@ template <class T> __global__ void __launch_bounds__(256) k_coef_diag(Coefs<T> a
 }
 // (RB: s_in == s_out; a launch reads the cells of the other colour)
 template <class T>
-__global__ void __launch_bounds__(256) k_sweep(Coefs<const T> a, const T *__restrict__ b, const T *sin, T *sout, Geom g,
+__global__ void __launch_bounds__(256) k_sweep(Coefs<const T> a, const T *b, const T *sin, T *sout, Geom g,
                                               int colour)
 {
     launched();
@@ -1307,14 +1313,14 @@ __global__ void __launch_bounds__(256) k_sweep(Coefs<const T> a, const T *__rest
         const Stencil t = stencil_of(i, j, k, g);
         const idx c = ck(t.c, g.n), xh = ck(t.xh, g.n), yh = ck(t.yh, g.n), zh = ck(t.zh, g.n);
         auto s = [&](bool face, idx at) { return face ? sin[ck(at, g.n)] : T(0); };
-        T off = mul_rn(__ldg(a.cx + c), s(t.hxl, t.xl));
-        off = fma_rn(__ldg(a.cx + xh), s(t.hxh, t.xh), off);
-        off = fma_rn(__ldg(a.cy + c), s(t.hyl, t.yl), off);
-        off = fma_rn(__ldg(a.cy + yh), s(t.hyh, t.yh), off);
-        off = fma_rn(__ldg(a.cz + c), s(t.hzl, t.zl), off);
-        off = fma_rn(__ldg(a.cz + zh), s(t.hzh, t.zh), off);
-        const T num = add_rn(__ldg(b + c), off), y = __ldg(a.inv + c), v = mul_rn(num, y);
-        const T rem = fma_rn(-__ldg(a.d + c), v, num);  // NaN where num or d is infinite: v is the quotient then
+        T off = mul_rn(a.cx[c], s(t.hxl, t.xl));
+        off = fma_rn(a.cx[xh], s(t.hxh, t.xh), off);
+        off = fma_rn(a.cy[c], s(t.hyl, t.yl), off);
+        off = fma_rn(a.cy[yh], s(t.hyh, t.yh), off);
+        off = fma_rn(a.cz[c], s(t.hzl, t.zl), off);
+        off = fma_rn(a.cz[zh], s(t.hzh, t.zh), off);
+        const T num = add_rn(b[c], off), y = a.inv[c], v = mul_rn(num, y);
+        const T rem = fma_rn(-a.d[c], v, num);  // NaN where num or d is infinite: v is the quotient then
         sout[c] = (__double2hiint(rem) & 0x7ff00000) == 0x7ff00000 ? v : fma_rn(rem, y, v);
     });
 }
@@ -1377,7 +1383,7 @@ template <bool HASD, class R> __device__ __forceinline__ void cvq4(const R &r, C
 // alternates two plane tiles (one barrier per plane); the others keep one.
 constexpr int SOURCE_BUFS = sizeof(S) == 2 ? 2 : 1;
 template <bool HASD, bool FULL>
-__device__ __forceinline__ void source_quads(const QIn q, S *__restrict__ b, S *__restrict__ rho_out, const Geom &g,
+__device__ __forceinline__ void source_quads(const QIn q, S *b, S *rho_out, const Geom &g,
                                             C alpha_s, const C *W, const C *J, int zc, const BlockPos &bp, int wq,
                                             int rows, C *U2)
 {
@@ -1519,7 +1525,7 @@ __device__ __forceinline__ void source_quads(const QIn q, S *__restrict__ b, S *
 // the pairs: u of a cell and the one above it, one halo cell per thread of
 // the first three warps, raw values one plane ahead
 template <bool HASD>
-__device__ __forceinline__ void source_pairs(const QIn q, S *__restrict__ b, S *__restrict__ rho_out, const Geom &g,
+__device__ __forceinline__ void source_pairs(const QIn q, S *b, S *rho_out, const Geom &g,
                                              C alpha_s, const C *W, const C *J, int zc, const BlockPos &bp, C *U2)
 {
     const Pair t = pair_of(g, bp);
@@ -1621,7 +1627,7 @@ __device__ __forceinline__ void source_pairs(const QIn q, S *__restrict__ b, S *
 // registers under this bound and still runs faster. FP64 keeps one block.
 constexpr int SOURCE_BLOCKS = sizeof(C) == 8 ? 1 : 2;
 template <bool HASD, bool FULL>
-__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source(QIn q, S *__restrict__ b, S *__restrict__ rho_out, Geom g,
+__global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source(QIn q, S *b, S *rho_out, Geom g,
                                                               C alpha_s, const C *W, const C *J, int zc, int wq,
                                                               int rows)
 {
@@ -1635,7 +1641,7 @@ __global__ void __launch_bounds__(BT, SOURCE_BLOCKS) k_source(QIn q, S *__restri
 // 448; only the smallest grids prefer fewer (33 x 35 x 37: 11.4, 10.5, 9.9).
 constexpr int SOURCE_PAIR_BLOCKS = sizeof(C) == 8 ? 1 : 4;
 template <bool HASD>
-__global__ void __launch_bounds__(32 * PWARPS, SOURCE_PAIR_BLOCKS) k_source_pairs(QIn q, S *__restrict__ b, S *__restrict__ rho_out,
+__global__ void __launch_bounds__(32 * PWARPS, SOURCE_PAIR_BLOCKS) k_source_pairs(QIn q, S *b, S *rho_out,
                                                                     Geom g, C alpha_s, const C *W, const C *J, int zc)
 {
     launched();
@@ -1931,7 +1937,7 @@ constexpr int FLUX_MAXREG = sizeof(C) == 8 ? 224 : 128;
 // d_{s+1} = RN16(w [(q_s - q^n) + dt L]) into `out`, and stage 3 stores the
 // FP32 state q^n + w [(q_s - q^n) + dt L] into `outb`.
 template <int mode, int ORD, bool VISC>
-__device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ sig, const QBIn qn,
+__device__ __forceinline__ void flux_body(const QIn qin, const S *sig, const QBIn qn,
                                           const Fout<5> out, const QBOut outb, const Frhs rhs,
                                           const Fout<5> base_out, const Geom g, C gamma, C half_inv_dx,
                                           const Scalars *sc, double *blockmax, int *err, const C *W,
@@ -1954,7 +1960,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
     auto ldq_raw = [&](int u, idx c) -> QRaw {
         if constexpr (kInc) {
             QRawInc r;
-            r.b = __ldg(qb0 + u * fs + c);
+            r.b = qb0[u * fs + c];
             r.d = HASD ? ldr(qd0 + u * fs + c) : S(0.0f);
             return *reinterpret_cast<QRaw *>(&r);
         } else {
@@ -2206,7 +2212,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
                 if (k >= k0 && (mode == FLUX_STAGE2 || mode == FLUX_STAGE3)) {
                     idx c = ck((idx)k * pl + own, g.n);
 #pragma unroll
-                    for (int u = 0; u < 5; u++) qnv[u] = __ldg(kInc ? qn0 + u * fs + c : qn.p[u] + c);
+                    for (int u = 0; u < 5; u++) qnv[u] = kInc ? qn0[u * fs + c] : qn.p[u][c];
                 }
             }
             Fzm = Fzp;
@@ -2281,7 +2287,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *__restrict__ s
 }
 template <int mode, int ORD, bool VISC>
 __global__ void __maxnreg__(FLUX_MAXREG)
-    k_flux(QIn qin, const S *__restrict__ sig, QBIn qn, Fout<5> out, QBOut outb, Frhs rhs, Fout<5> base_out,
+    k_flux(QIn qin, const S *sig, QBIn qn, Fout<5> out, QBOut outb, Frhs rhs, Fout<5> base_out,
            Geom g, C gamma, C half_inv_dx, const Scalars *sc, double *blockmax, int *err, const C *W,
            const C *J, int zc, int cz0, C mu, C lamv)
 {
@@ -2321,7 +2327,7 @@ __global__ void k_rk_combine(const QB *__restrict__ qn, const QB *__restrict__ q
 constexpr int SPEED_NT = 256, SPEED_MAXBLOCKS = 152 * 8;
 
 template <bool VEC>
-__global__ void __launch_bounds__(SPEED_NT) k_speed(const QB *__restrict__ q, long long n, C gamma,
+__global__ void __launch_bounds__(SPEED_NT) k_speed(const QB *q, long long n, C gamma,
                                                      double *blockmax)
 {
     launched();
@@ -2344,7 +2350,7 @@ __global__ void __launch_bounds__(SPEED_NT) k_speed(const QB *__restrict__ q, lo
         }
     } else {
         for (long long c = blockIdx.x * (long long)SPEED_NT + threadIdx.x; c < n; c += (long long)gridDim.x * SPEED_NT)
-            take(ldc(q + c), ldc(q + n + c), ldc(q + 2 * n + c), ldc(q + 3 * n + c), ldc(q + 4 * n + c));
+            take(cv(q[c]), cv(q[n + c]), cv(q[2 * n + c]), cv(q[3 * n + c]), cv(q[4 * n + c]));
     }
     const double bm = block_max<SPEED_NT>(double(m));
     if (threadIdx.x == 0) blockmax[blockIdx.x] = bm;
