@@ -32,7 +32,7 @@
  *  - Alignment: a device pointer must be aligned to its element size (2, 4
  *    or 8 bytes), else the call returns IGR_ERR_INVALID_ARG before any
  *    launch. Where a call could take 4-wide loads (igr_solve_sigma,
- *    igr_solve_sigma_noalloc), pointers that are element-aligned but not
+ *    igr_solve_sigma_noalloc, igr_adjoint_step), pointers that are element-aligned but not
  *    aligned to 4 elements (8 bytes at 16-bit storage, 16 bytes for FP32 and
  *    FP64; a sliced tensor can start anywhere) make that call load element by
  *    element, with the same bits. Buffers from cudaMalloc or a

@@ -1679,11 +1679,13 @@ igr_status igr_adjoint_step(igr_ctx *c, const void *q_n, const void *sigma_n, co
     const void *qs[3] = {q_n, A.qs[0], A.qs[1]};
     CU(c, cudaMemcpyAsync(it(0, 0), sigma_n, n * sb, cudaMemcpyDeviceToDevice, c->st));
     for (int st = 0; st < 3; st++) {
-        CU(c, o->source(c->g, c->p, c->tiles, inflow_of(c), qs[st], nullptr, A.b, nullptr, c->st));
+        Tiles t = c->tiles;
+        t.elem = st == 0 && !is_aligned(q_n, vec4_align((int)sb));  // the caller's q: the others are the context's
+        CU(c, o->source(c->g, c->p, t, inflow_of(c), qs[st], nullptr, A.b, nullptr, c->st));
         if (o->sweep) CU(c, o->coefs(c->g, c->p, qs[st], c->q[1], c->st));
         for (int k = 0; k < S; k++)
             CU(c, o->sweep ? o->sweep(c->g, c->q[1], A.b, it(st, k), it(st, k + 1), -1, c->st)
-                           : o->jacobi(c->g, c->p, c->tiles, qs[st], A.b, it(st, k), it(st, k + 1), -1, c->st));
+                           : o->jacobi(c->g, c->p, t, qs[st], A.b, it(st, k), it(st, k + 1), -1, c->st));
         if (st < 2) {
             CU(c, o->flux(c->g, c->p, c->tiles, inflow_of(c), st == 0 ? FLUX_STAGE1 : FLUX_STAGE2, qs[st],
                           nullptr, it(st, S), q_n, (void *)qs[st + 1], nullptr, nullptr, A.sc, c->blockmax,
