@@ -251,7 +251,7 @@ __device__ __forceinline__ double sqrt_c(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_c(float x)
 {
     float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 
