@@ -1223,11 +1223,26 @@ __global__ void __launch_bounds__(BT, JACOBI_PAIR_BLOCKS) k_jacobi_pairs(const S
 // takes (two divisions, 14 for the faces, 6 for the diagonal). None of these
 // depend on Sigma, so where 5 n scratch values are free (a context's RK buffers)
 // they are formed once per stage: the three low-face factors, the diagonal d and
-// its inverse. That leaves 10: the sum and num / d by the inverse with one
-// remainder step (Markstein, IBM J. R&D 34, 1990), which gives the division's
-// rounding, so the results are those of the sweeps above. All else is free
-// beside the FP64 units (64 bytes per cell from memory take half their time):
-// one thread per cell, neighbours from L1, no alignment and no tile shape.
+// its inverse. That leaves 10: the sum and num / d (quot), so the results are those
+// of the sweeps above. All else is free beside the FP64 units (64 bytes per cell
+// from memory take half their time): one thread per cell, neighbours from L1, no
+// alignment and no tile shape.
+//
+// num / d rounded to nearest from inv = 1 / d: v = num inv and one remainder step
+// (Markstein, IBM J. R&D 34, 1990). The remainder is exact and inv normal where
+// both num and v lie in [2^-500, 2^500) (tested on the exponents, by integer
+// instructions); zero is 0 inv, and the rest (far smaller or larger, infinities,
+// NaN) divides.
+__device__ __forceinline__ bool mid_range(double x)
+{
+    return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 523u < 1000u;
+}
+__device__ __forceinline__ double quot(double num, double d, double inv)
+{
+    const double v = __dmul_rn(num, inv);
+    if (mid_range(num) && mid_range(v)) return __fma_rn(__fma_rn(-d, v, num), inv, v);
+    return num == 0.0 && mid_range(inv) ? v : __ddiv_rn(num, d);
+}
 template <class T> struct Coefs {
     T *cx, *cy, *cz, *d, *inv;
 };
@@ -1319,9 +1334,7 @@ __global__ void __launch_bounds__(256) k_sweep(Coefs<const T> a, const T *b, con
         off = fma_rn(a.cy[yh], s(t.hyh, t.yh), off);
         off = fma_rn(a.cz[c], s(t.hzl, t.zl), off);
         off = fma_rn(a.cz[zh], s(t.hzh, t.zh), off);
-        const T num = add_rn(b[c], off), y = a.inv[c], v = mul_rn(num, y);
-        const T rem = fma_rn(-a.d[c], v, num);  // NaN where num or d is infinite: v is the quotient then
-        sout[c] = (__double2hiint(rem) & 0x7ff00000) == 0x7ff00000 ? v : fma_rn(rem, y, v);
+        sout[c] = quot(add_rn(b[c], off), a.d[c], a.inv[c]);
     });
 }
 
