@@ -1696,8 +1696,9 @@ igr_status igr_adjoint_step(igr_ctx *c, const void *q_n, const void *sigma_n, co
     // reverse, stage by stage: `in` the adjoint of the stage's output, `out` that of its
     // input (lq0 gathers that of the step's input), by gathering or, in FP32 arithmetic
     // with jets, scattering (igr_kernels.cu says why). Scratch: once the faces are done,
-    // the buffer `free5` (5 n) and Lb (5 n) hold 1 / rho, the diagonal and, with mu, the
-    // nine gradient adjoints of the gathered source.
+    // Lb (5 n) holds 1 / rho and, during the sweeps, the diagonal and its inverse; the buffer
+    // `free5` (5 n), the rest of Lb and mu then hold the nine gradient adjoints of the
+    // gathered source.
     const bool gather = cb == 8 || c->cfg.njets == 0;
     const void *in = lam_q_np1;
     void *out = A.lqs, *free5 = A.lout, *lsig = A.lsig, *nl = A.nl;
@@ -1705,7 +1706,7 @@ igr_status igr_adjoint_step(igr_ctx *c, const void *q_n, const void *sigma_n, co
     CU(c, cudaMemcpyAsync(lsig, lam_sigma_np1, n * cb, cudaMemcpyDeviceToDevice, c->st));
     CU(c, cudaMemsetAsync(A.lamJ, 0, 5 * (size_t)c->g.plane * cb, c->st));
     if (!gather) CU(c, cudaMemsetAsync(A.lq0, 0, 5 * n * cb, c->st));
-    void *r = at(A.Lb, 0), *diag = at(A.Lb, 1);
+    void *r = at(A.Lb, 0), *diag = at(A.Lb, 1), *dinv = at(A.Lb, 2);
     for (int st = 2; st >= 0; st--) {
         if (gather) {
             CU(c, o->adj_rhs(c->g, c->p, inflow_of(c), qs[st], it(st, S), in, out, A.lq0, lsig, A.lamJ, wst[st], dt,
@@ -1715,10 +1716,10 @@ igr_status igr_adjoint_step(igr_ctx *c, const void *q_n, const void *sigma_n, co
             CU(c, o->adj_rhs_scatter(c->g, c->p, inflow_of(c), qs[st], it(st, S), A.Lb, out, lsig, A.lamJ, c->st));
         }
         if (st < 2) free5 = (void *)in;  // (stage 3's `in` is the caller's)
-        CU(c, o->adj_diag(c->g, c->p, qs[st], r, diag, c->st));
+        CU(c, o->adj_diag(c->g, c->p, qs[st], r, diag, dinv, c->st));
         for (int k = S - 1; k >= 0; k--) {
-            CU(c, o->adj_jacobi(c->g, c->p, r, diag, it(st, k), it(st, k + 1), lsig, nl, A.lb, A.rb, k == S - 1,
-                                c->st));
+            CU(c, o->adj_jacobi(c->g, c->p, r, diag, dinv, it(st, k), it(st, k + 1), lsig, nl, A.lb, A.rb,
+                                k == S - 1, c->st));
             std::swap(lsig, nl);
         }
         if (gather) {

@@ -192,13 +192,14 @@ struct Ops {
     cudaError_t (*adj_rhs)(const Geom &, const Phys &, const Inflow &, const void *qs, const void *sig,
                            const void *lout, void *lqs, void *lq0, void *lsig, void *lamJ, double w, double dt,
                            int first, cudaStream_t st);
-    // r = 1 / rho and the diagonal of the sweeps (FP64: its inverse)
-    cudaError_t (*adj_diag)(const Geom &, const Phys &, const void *q, void *r, void *diag, cudaStream_t st);
+    // r = 1 / rho, the diagonal of the sweeps and (FP64 only) its inverse
+    cudaError_t (*adj_diag)(const Geom &, const Phys &, const void *q, void *r, void *diag, void *dinv,
+                            cudaStream_t st);
     // one reversed Jacobi sweep s_k -> F: lsig (adjoint of F) -> nl (adjoint of s_k);
     // lb += mu, rb += d/d(1/rho) (first: =)
-    cudaError_t (*adj_jacobi)(const Geom &, const Phys &, const void *r, const void *diag, const void *sk,
-                              const void *F, const void *lsig, void *nl, void *lb, void *rb, int first,
-                              cudaStream_t st);
+    cudaError_t (*adj_jacobi)(const Geom &, const Phys &, const void *r, const void *diag, const void *dinv,
+                              const void *sk, const void *F, const void *lsig, void *nl, void *lb, void *rb,
+                              int first, cudaStream_t st);
     // reverse of the IGR source and of 1 / rho: lb, rb -> lqs (rho, m), lamJ; grads: nine
     // scratch arrays of n values
     cudaError_t (*adj_source)(const Geom &, const Phys &, const Inflow &, const void *q, const void *r,

@@ -3099,11 +3099,15 @@ __device__ __forceinline__ bool cell_of(const Geom &g, int &i, int &j, int &k, i
     return i < g.nx && j < g.ny;
 }
 
-// r = 1 / rho and the diagonal D of the sweeps, once per stage (FP64: 1 / D,
-// whose seven divisions per cell and sweep would be slow)
-__device__ __forceinline__ float mu_of(float l, float d) { return l / d; }
-__device__ __forceinline__ double mu_of(double l, double dinv) { return l * dinv; }
-__global__ void __launch_bounds__(CBX *CBY) k_adj_diag(const S *q, C *r, C *dg, Geom g, C beta)
+// r = 1 / rho, the diagonal D of the sweeps and, in FP64, its inverse, once per
+// stage. mu = lsig / D is the division's rounding in both (quot): seven divisions
+// per cell and sweep would hold the FP64 units.
+__device__ __forceinline__ float mu_of(const float *l, const float *d, const float *, idx t) { return l[t] / d[t]; }
+__device__ __forceinline__ double mu_of(const double *l, const double *d, const double *inv, idx t)
+{
+    return quot(l[t], d[t], inv[t]);
+}
+__global__ void __launch_bounds__(CBX *CBY) k_adj_diag(const S *q, C *r, C *dg, C *dinv, Geom g, C beta)
 {
     int i, j, k;
     idx t;
@@ -3116,7 +3120,8 @@ __global__ void __launch_bounds__(CBX *CBY) k_adj_diag(const S *q, C *r, C *dg, 
         if (nbr(g, i, j, k, d, m)) diag += beta * C(0.5) * (ri + C(1) / ldc(q + m));
     }
     r[t] = ri;
-    dg[t] = sizeof(C) == 8 ? C(1) / diag : diag;
+    dg[t] = diag;
+    if (sizeof(C) == 8) dinv[t] = C(1) / diag;
 }
 
 // One reversed Jacobi sweep s_k -> F, gathered (the neighbour relation is
@@ -3125,21 +3130,21 @@ __global__ void __launch_bounds__(CBX *CBY) k_adj_diag(const S *q, C *r, C *dg, 
 //   rb_m += mu_m (beta/2 sum s_nb - F_m (1 + beta nf/2)) + sum_i mu_i beta/2 (s_m - F_i);
 // the neighbours' mu are formed again from lsig and D, which saves a pass.
 __global__ void __launch_bounds__(CBX *CBY) k_adj_jacobi(const C *__restrict__ r, const C *__restrict__ dg,
-                                                         const S *__restrict__ sk, const S *__restrict__ F,
+                                                         const C *__restrict__ dinv, const S *__restrict__ sk, const S *__restrict__ F,
                                                          const C *__restrict__ lsig, C *nl, C *lb, C *rb, Geom g,
                                                          C beta, int first)
 {
     int i, j, k;
     idx t;
     if (!cell_of(g, i, j, k, t)) return;
-    const C rm = r[t], sm = ldc(sk + t), Fm = ldc(F + t), mum = mu_of(lsig[t], dg[t]), hb = C(0.5) * beta;
+    const C rm = r[t], sm = ldc(sk + t), Fm = ldc(F + t), mum = mu_of(lsig, dg, dinv, t), hb = C(0.5) * beta;
     C acc = C(0), ssum = C(0), rbm = C(0);
     int nfc = 0;
 #pragma unroll
     for (int d = 0; d < 6; d++) {
         idx n;
         if (!nbr(g, i, j, k, d, n)) continue;
-        const C mun = mu_of(lsig[n], dg[n]);
+        const C mun = mu_of(lsig, dg, dinv, n);
         acc += hb * (rm + r[n]) * mun;
         ssum += ldc(sk + n);
         nfc++;
@@ -3901,20 +3906,21 @@ cudaError_t launch_adj_source_scatter(const Geom &g, const Phys &p, const Inflow
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_diag(const Geom &g, const Phys &p, const void *q, void *r, void *dinv, cudaStream_t st)
+cudaError_t launch_adj_diag(const Geom &g, const Phys &p, const void *q, void *r, void *diag, void *dinv,
+                            cudaStream_t st)
 {
-    k_adj_diag<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const S *)q, (C *)r, (C *)dinv, g,
+    k_adj_diag<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const S *)q, (C *)r, (C *)diag, (C *)dinv, g,
                                                           C(p.alpha / (p.dx * p.dx)));
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_jacobi(const Geom &g, const Phys &p, const void *r, const void *dinv, const void *sk,
-                              const void *F, const void *lsig, void *nl, void *lb, void *rb, int first,
-                              cudaStream_t st)
+cudaError_t launch_adj_jacobi(const Geom &g, const Phys &p, const void *r, const void *diag, const void *dinv,
+                              const void *sk, const void *F, const void *lsig, void *nl, void *lb, void *rb,
+                              int first, cudaStream_t st)
 {
-    k_adj_jacobi<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const C *)r, (const C *)dinv, (const S *)sk,
-                                                            (const S *)F, (const C *)lsig, (C *)nl, (C *)lb, (C *)rb,
-                                                            g, C(p.alpha / (p.dx * p.dx)), first);
+    k_adj_jacobi<<<cell_blocks(g), dim3(CBX, CBY), 0, st>>>((const C *)r, (const C *)diag, (const C *)dinv,
+                                                            (const S *)sk, (const S *)F, (const C *)lsig, (C *)nl,
+                                                            (C *)lb, (C *)rb, g, C(p.alpha / (p.dx * p.dx)), first);
     return cudaGetLastError();
 }
 
