@@ -3262,7 +3262,8 @@ __global__ void k_adj_add(const C *a, const C *b, C *out, long long n)
 // part[n][b] = block b's share of the sum over the inflow face of
 // s_n (rho_n lamJ_mz + rho_n w_n lamJ_E), then gw[n] = the shares in order.
 // Twenty edge widths outside a jet s_n is 0 to the last bit, so those cells
-// skip the FP64 root and tanh; one block per jet took 263 us on a 128^2 face.
+// skip the FP64 root and tanh (not the product: an infinity or a NaN in lamJ
+// reaches the sum); one block per jet took 263 us on a 128^2 face.
 __global__ void __launch_bounds__(256) k_adj_jets(const double *jets, const C *lamJ, double *part, int nx, int ny,
                                                   double dx)
 {
@@ -3273,8 +3274,7 @@ __global__ void __launch_bounds__(256) k_adj_jets(const double *jets, const C *l
     for (long long f = blockIdx.y * 256LL + threadIdx.x; f < plane; f += 256LL * gridDim.y) {
         const int i = (int)((unsigned)f % (unsigned)nx), j = (int)((unsigned)f / (unsigned)nx);
         const double x = (i + 0.5) * dx - jt[0], y = (j + 0.5) * dx - jt[1], r2 = x * x + y * y;
-        if (r2 > reach * reach) continue;
-        const double sn = 0.5 * (1.0 - tanh((sqrt(r2) - jt[2]) / (jt[6] * dx)));
+        const double sn = r2 > reach * reach ? 0.0 : 0.5 * (1.0 - tanh((sqrt(r2) - jt[2]) / (jt[6] * dx)));
         acc += sn * (jt[3] * double(lamJ[ckl(3 * plane + f, 5 * plane)]) +
                      jt[3] * jt[4] * double(lamJ[ckl(4 * plane + f, 5 * plane)]));
     }
