@@ -247,7 +247,7 @@ def run_form(case, precision, steps, warmup, sync_all, e2e_steps=0, host_rk_base
             s.set_kernel_forms(*forms)
         if autotune:
             s.autotune(reps=2)
-        res["tiles"], res["forms"] = s.tiles(), s.kernel_forms()
+        res["tiles"], res["forms"] = s.tiles(), s.launch_forms()
         s.step(warmup)
         stream = s.stream
         sync_all()
@@ -467,7 +467,7 @@ def run_batch(args, sync_all=lambda: None):
         torch.cuda.synchronize()
         b.autotune(reps=3)
         for c, inst in zip(cases, b.instances):
-            tuned.setdefault((c.nx, c.ny, c.nz), (inst.tiles(), inst.kernel_forms()))
+            tuned.setdefault((c.nx, c.ny, c.nz), (inst.tiles(), inst.launch_forms()))
         b.step(args.warmup, sync=True)
         sync_all()
         torch.cuda.synchronize()
@@ -582,7 +582,7 @@ def main():
     ap.add_argument("--mu", type=float, default=0.0, help="shear viscosity (0: Euler)")
     ap.add_argument("--zeta", type=float, default=0.0, help="bulk viscosity")
     ap.add_argument("--forms", type=int, nargs=2, default=None, metavar=("SOURCE", "JACOBI"),
-                    help="kernel forms of the source and Jacobi kernels (1: four cells per thread, 0: one)")
+                    help="forms of the source and Jacobi kernels (1: quads, 0: pairs)")
     ap.add_argument("--autotune", action="store_true", help="autotune the launch shape before timing")
     ap.add_argument("--host-rk-base", action="store_true",
                     help="keep the RK base q^n in host memory (read over NVLink-C2C)")

@@ -32,11 +32,11 @@
  *  - Alignment: a device pointer must be aligned to its element size (2, 4
  *    or 8 bytes), else the call returns IGR_ERR_INVALID_ARG before any
  *    launch. Where a call could take 4-wide loads (igr_solve_sigma,
- *    igr_solve_sigma_noalloc, igr_adjoint_step), pointers that are element-aligned but not
- *    aligned to 4 elements (8 bytes at 16-bit storage, 16 bytes for FP32 and
- *    FP64; a sliced tensor can start anywhere) make that call load element by
- *    element, with the same bits. Buffers from cudaMalloc or a
- *    caching allocator are 256-byte aligned.
+ *    igr_solve_sigma_noalloc, igr_adjoint_step), pointers that are
+ *    element-aligned but not aligned to 4 elements (8 bytes at 16-bit storage,
+ *    16 bytes for FP32 and FP64; a sliced tensor can start anywhere) make that
+ *    call load element by element, with the same bits. Buffers from cudaMalloc
+ *    or a caching allocator are 256-byte aligned.
  *  - A context is not thread-safe; distinct contexts are independent.
  *  - Asynchronous faults (CUDA errors, non-finite results) surface at the
  *    next call that synchronises: igr_get_state, igr_sync, igr_step_host,
@@ -360,29 +360,35 @@ igr_status igr_profile_read(igr_ctx *ctx, int kernel_class, long long *launches,
  * Each kernel class marches blocks up chunks of z-planes; the chunk length
  * is the tunable launch shape (>= 4 planes, at most nz). The default is the
  * chunk that a count of waves of resident blocks makes the fastest.
- * The source and Jacobi kernels give a thread four consecutive cells of a
- * row with 4-wide loads where rows are a multiple of 4 cells and the buffers
- * aligned to 4 values, else two cells, one above the other, loaded element by
- * element; blocks are fitted to the row length.
+ * The source and Jacobi kernels have two forms: quads, four consecutive cells
+ * of a row per thread with 4-wide loads, for rows of a multiple of 4 cells in
+ * buffers aligned to 4 values, and pairs, two cells one above the other, loaded
+ * element by element; blocks of quads are fitted to the row length.
  * Results do not depend on the launch shape: every face flux comes out of
  * the same instructions whatever the chunking, both forms evaluate the same
  * sequence of rounded operations, and there are no atomics, so outputs are
  * bitwise identical for every choice.
- * igr_set_kernel_forms: source_vec4 and jacobi_vec4 each -1 (the default
- * rule), 0 or 1 (IGR_ERR_INVALID_ARG when nx % 4 != 0). The setting is kept
- * and reported (the default rule reports 1 for rows of a multiple of 4 cells
- * that fill blocks of 128 cells), and every setting launches the kernels
- * described above.
+ * igr_set_kernel_forms: source_vec4 and jacobi_vec4 each -1 (the default:
+ * quads where rows are a multiple of 4 cells), 0 (pairs) or 1 (quads;
+ * IGR_ERR_INVALID_ARG when nx % 4 != 0). Fields that are not aligned to 4
+ * values take pairs whatever the setting.
+ * igr_get_kernel_forms returns the settings; for the default not -1 but 1
+ * where rows fill blocks of 128 cells about as well as blocks of 32, else 0: a
+ * property of nx that earlier kernels were chosen by and callers compare.
+ * igr_get_launch_forms tells what the context's steps launch under the
+ * present setting: 1 quads, 0 pairs; sweeps -1 in FP64, whose sweeps on stored
+ * coefficients have one form.
  * The sweep chunk has no effect on FP64 sweeps on stored coefficients (a
  * context's steps and igr_solve_sigma), which have none.
  * igr_autotune times each class on the current state for the default chunk
- * and the candidate lengths 4..128 (reps launches each, on the context
- * stream; only scratch buffers are written) and keeps the fastest; call it
- * after igr_set_state. It synchronises. */
+ * and the candidate lengths 4..128 and, where nx % 4 == 0, both forms (reps
+ * launches each, on the context stream; only scratch buffers are written) and
+ * keeps the fastest; call it after igr_set_state. It synchronises. */
 igr_status igr_set_tiles(igr_ctx *ctx, int zc_source, int zc_jacobi, int zc_flux);
 igr_status igr_get_tiles(igr_ctx *ctx, int *zc_source, int *zc_jacobi, int *zc_flux);
 igr_status igr_set_kernel_forms(igr_ctx *ctx, int source_vec4, int jacobi_vec4);
 igr_status igr_get_kernel_forms(igr_ctx *ctx, int *source_vec4, int *jacobi_vec4);
+igr_status igr_get_launch_forms(igr_ctx *ctx, int *source, int *sweeps);
 igr_status igr_autotune(igr_ctx *ctx, int reps);
 
 /* ---- Batches of independent instances -----------------------------------

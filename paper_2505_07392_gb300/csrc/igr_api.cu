@@ -285,8 +285,7 @@ static int choose_zc(long long cols, int nz, int resident, double c0)
 Tiles igr::default_tiles(const Geom &g, const Ops *o)
 {
     Tiles t = {};
-    t.vec_source = vec4_default_source(g.nx);
-    t.vec_jacobi = vec4_default_jacobi(g.nx);
+    t.vec_source = t.vec_jacobi = -1;
     long long cols;
     int resident;
     o->source_shape(g, &cols, &resident);
@@ -1065,19 +1064,27 @@ igr_status igr_set_kernel_forms(igr_ctx *c, int source_vec4, int jacobi_vec4)
 {
     if (!c) return fail(c, IGR_ERR_INVALID_ARG, "ctx is NULL");
     if (source_vec4 < -1 || source_vec4 > 1 || jacobi_vec4 < -1 || jacobi_vec4 > 1)
-        return fail(c, IGR_ERR_INVALID_ARG, "forms are -1 (default), 0 (1 cell) or 1 (4 cells)");
+        return fail(c, IGR_ERR_INVALID_ARG, "forms are -1 (default), 0 (pairs) or 1 (quads)");
     if ((source_vec4 == 1 || jacobi_vec4 == 1) && c->g.nx % 4)
-        return fail(c, IGR_ERR_INVALID_ARG, "the 4-cell form needs nx %% 4 == 0 (nx = %d)", c->g.nx);
-    c->tiles.vec_source = source_vec4 < 0 ? vec4_default_source(c->g.nx) : source_vec4;
-    c->tiles.vec_jacobi = jacobi_vec4 < 0 ? vec4_default_jacobi(c->g.nx) : jacobi_vec4;
+        return fail(c, IGR_ERR_INVALID_ARG, "quads need nx %% 4 == 0 (nx = %d)", c->g.nx);
+    c->tiles.vec_source = source_vec4;
+    c->tiles.vec_jacobi = jacobi_vec4;
     return IGR_OK;
 }
 
 igr_status igr_get_kernel_forms(igr_ctx *c, int *source_vec4, int *jacobi_vec4)
 {
     if (!c || !source_vec4 || !jacobi_vec4) return fail(c, IGR_ERR_INVALID_ARG, "null argument");
-    *source_vec4 = c->tiles.vec_source;
-    *jacobi_vec4 = c->tiles.vec_jacobi;
+    *source_vec4 = c->tiles.vec_source < 0 ? vec4_default_source(c->g.nx) : c->tiles.vec_source;
+    *jacobi_vec4 = c->tiles.vec_jacobi < 0 ? vec4_default_jacobi(c->g.nx) : c->tiles.vec_jacobi;
+    return IGR_OK;
+}
+
+igr_status igr_get_launch_forms(igr_ctx *c, int *source, int *sweeps)
+{
+    if (!c || !source || !sweeps) return fail(c, IGR_ERR_INVALID_ARG, "null argument");
+    *source = c->ops->source_form(c->g, c->tiles);
+    *sweeps = c->ops->sweep ? -1 : c->ops->sweep_form(c->g, c->tiles);
     return IGR_OK;
 }
 
@@ -1107,7 +1114,8 @@ igr_status igr_autotune(igr_ctx *c, int reps)
 {
     if (!c || reps < 1) return fail(c, IGR_ERR_INVALID_ARG, "ctx and reps >= 1 are required");
     if (c->profiling) return fail(c, IGR_ERR_INVALID_ARG, "disable profiling before tuning");
-    // the default shape and chunks of 4..128 planes
+    // the default shape and chunks of 4..128 planes, pairs and, where rows allow, quads
+    const int nforms = c->g.nx % 4 == 0 ? 2 : 1;
     const Tiles dflt = default_tiles(c->g, c->ops);
     const int cand[] = {0, 4, 8, 16, 32, 64, 128};
     Tiles best = c->tiles;
@@ -1125,20 +1133,23 @@ igr_status igr_autotune(igr_ctx *c, int reps)
         float ms;
         igr_status s;
         // each kernel class writes only scratch: b, the other Sigma buffer, the stage-1 output
-        s = time_launches(c, reps, [&] {
-            return c->ops->source(c->g, c->p, t, inflow_of(c), c->q[0], nullptr, c->b, c->rho16, c->st);
-        }, &ms);
-        if (s != IGR_OK) return s;
-        if (ms < tbest[0]) { tbest[0] = ms; best.zc_source = t.zc_source; }
-        s = time_launches(c, reps, [&] {
-            // red-black: a half-sweep in place on a copy of Sigma in the stage-1 output buffer
-            const void *qj = c->inc ? c->rho16 : c->q[0];
-            return c->cfg.sigma_solver == SOLVER_RBGS
-                       ? c->ops->jacobi(c->g, c->p, t, qj, c->b, c->q[1], c->q[1], 0, c->st)
-                       : c->ops->jacobi(c->g, c->p, t, qj, c->b, sig, scratch, -1, c->st);
-        }, &ms);
-        if (s != IGR_OK) return s;
-        if (ms < tbest[1]) { tbest[1] = ms; best.zc_jacobi = t.zc_jacobi; }
+        for (int v = 0; v < nforms; v++) {
+            t.vec_source = t.vec_jacobi = v;
+            s = time_launches(c, reps, [&] {
+                return c->ops->source(c->g, c->p, t, inflow_of(c), c->q[0], nullptr, c->b, c->rho16, c->st);
+            }, &ms);
+            if (s != IGR_OK) return s;
+            if (ms < tbest[0]) { tbest[0] = ms; best.zc_source = t.zc_source; best.vec_source = v; }
+            s = time_launches(c, reps, [&] {
+                // red-black: a half-sweep in place on a copy of Sigma in the stage-1 output buffer
+                const void *qj = c->inc ? c->rho16 : c->q[0];
+                return c->cfg.sigma_solver == SOLVER_RBGS
+                           ? c->ops->jacobi(c->g, c->p, t, qj, c->b, c->q[1], c->q[1], 0, c->st)
+                           : c->ops->jacobi(c->g, c->p, t, qj, c->b, sig, scratch, -1, c->st);
+            }, &ms);
+            if (s != IGR_OK) return s;
+            if (ms < tbest[1]) { tbest[1] = ms; best.zc_jacobi = t.zc_jacobi; best.vec_jacobi = v; }
+        }
         s = time_launches(c, reps, [&] {
             return c->ops->flux(c->g, c->p, t, inflow_of(c), FLUX_STAGE1, c->q[0], nullptr, sig, c->q[0], c->q[1],
                                 nullptr, nullptr, c->sc, c->blockmax, &c->sc->err, c->st);

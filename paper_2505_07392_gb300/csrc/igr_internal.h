@@ -53,17 +53,19 @@ struct Tiles {
     int zc_source;  // z-planes per block of the source kernel
     int zc_jacobi;  // z-planes per block of the Jacobi kernel
     int zc_flux;    // z-planes per block of the flux kernel
-    int vec_source; // the form igr_get_kernel_forms reports (both forms launch the same kernel
-    int vec_jacobi; // where rows are a multiple of 4 cells)
+    int vec_source; // the source's and the sweeps' form: 0 pairs, 1 quads, -1 quads where
+    int vec_jacobi; // rows are a multiple of 4 cells (igr_set_kernel_forms)
     int elem;       // 1: the source and the sweeps load element by element (pointers that are not
                     // aligned to 4 values)
     int z_begin;    // a flux launch covers planes [z_begin, z_end) only (z_begin a multiple
     int z_end;      // of zc_flux, z_end a multiple or nz); z_end = 0: all planes
 };
 
-// The form the default rule of igr_set_kernel_forms reports: 1 where rows of
-// nx cells fill blocks of 128 cells at least num / den times as well as
-// blocks of 32.
+// What igr_get_kernel_forms returns for the default setting: 1 where rows of nx
+// cells fill blocks of 128 cells at least num / den times as well as blocks of 32,
+// the rule by which kernels of one and four cells per thread were chosen. It
+// chooses nothing now (igr_get_launch_forms says what is launched); callers
+// compare the value.
 inline int vec4_default(int nx, int num, int den)
 {
     if (nx % 4) return 0;
@@ -250,6 +252,9 @@ struct Ops {
 
     // blocks per plane of the source / of a sweep, and the blocks per SM that
     // their registers allow (for the choice of the z-chunks)
+    // (source_form, sweep_form: 1 where the launch takes quads, 0 pairs)
+    int (*source_form)(const Geom &, const Tiles &);
+    int (*sweep_form)(const Geom &, const Tiles &);
     void (*source_shape)(const Geom &, long long *cols, int *resident);
     void (*jacobi_shape)(const Geom &, long long *cols, int *resident);
     // FP64 (NULL in the other modes): the sweeps' coefficients of the density q into

@@ -3440,14 +3440,15 @@ template <class K> cudaError_t allow_smem(K kern, int bytes)
 // tiles, 0 pairs; a sweep's form 3: full tiles with two rows per thread
 // (16-bit storage; from 16M cells: FP16, 512 x 512 x 128: 73 us against 79
 // with one; 256 x 256 x 192: 32 against 29.5). Its grid and block.
-int quad_form(const Geom &g, const Tiles &t)
+int quad_form(const Geom &g, const Tiles &t, int vec)
 {
-    if (t.elem || g.nx % VX != 0) return 0;
+    if (t.elem || vec == 0 || g.nx % VX != 0) return 0;
     return quad_fit(g).full ? 2 : 1;
 }
+int source_form(const Geom &g, const Tiles &t) { return quad_form(g, t, t.vec_source); }
 int sweep_form(const Geom &g, const Tiles &t)
 {
-    const int form = quad_form(g, t);
+    const int form = quad_form(g, t, t.vec_jacobi);
     return form == 2 && sizeof(S) == 2 && g.ny % (2 * FR) == 0 && g.n >= (1 << 24) ? 3 : form;
 }
 // the source takes the compiled-in tile in the 16-bit forms only (FP32, 256^3:
@@ -3460,17 +3461,20 @@ dim3 quad_grid(const Geom &g, int form, int zc)
     return dim3(f.gx, form == 3 ? f.gy / 2 : f.gy, (g.nz + zc - 1) / zc);
 }
 int quad_threads(const Geom &g, int form) { return form ? quad_fit(g).threads : 32 * PWARPS; }
-// blocks per plane and blocks per SM (Ops::source_shape, Ops::jacobi_shape)
+int takes_quads_source(const Geom &g, const Tiles &t) { return source_form(g, t) > 0; }
+int takes_quads_sweep(const Geom &g, const Tiles &t) { return sweep_form(g, t) > 0; }
+// blocks per plane and blocks per SM (Ops::source_shape, Ops::jacobi_shape), default forms
+constexpr Tiles kDefaultForms = {0, 0, 0, -1, -1, 0, 0, 0};
 void source_shape(const Geom &g, long long *cols, int *resident)
 {
-    const int form = quad_form(g, Tiles{});
+    const int form = source_form(g, kDefaultForms);
     const dim3 gr = quad_grid(g, form, g.nz);
     *cols = (long long)gr.x * gr.y;
     *resident = !form ? SOURCE_PAIR_BLOCKS : (sizeof(C) == 8 ? 256 : 512) / quad_threads(g, form);
 }
 void jacobi_shape(const Geom &g, long long *cols, int *resident)
 {
-    const int form = sweep_form(g, Tiles{});
+    const int form = sweep_form(g, kDefaultForms);
     const dim3 gr = quad_grid(g, form, g.nz);
     *cols = (long long)gr.x * gr.y;
     const int blocks = form == 3 ? kJacobiBlocks<2> : form == 2 ? kJacobiBlocks<1> : form ? JACOBI_FIT_BLOCKS : JACOBI_PAIR_BLOCKS;
@@ -3486,7 +3490,7 @@ cudaError_t launch_source(const Geom &g, const Phys &p, const Tiles &t, const In
     const C as = C(p.alpha * 0.25 / (p.dx * p.dx));
     const C *W = (const C *)in.W, *J = (const C *)in.J;
     const QuadFit f = quad_fit(g);
-    const int form = quad_form(g, t), threads = quad_threads(g, form);
+    const int form = source_form(g, t), threads = quad_threads(g, form);
     const dim3 gr = quad_grid(g, form, t.zc_source);
     if (form) {
         auto kern = source_full(form) ? (qd ? k_source<kInc, true> : k_source<false, true>)
@@ -3660,7 +3664,7 @@ cudaError_t launch_source_group(const SourceCall *calls, int n, cudaStream_t st)
 {
     for (int i = 0; i < n; i++)
         if ((kInc != (calls[i].rho_out != nullptr)) || (!kInc && calls[i].qd)) return cudaErrorInvalidValue;
-    auto key = [](const SourceCall &c) { return 2 * quad_form(c.g, c.t) + (c.qd ? 1 : 0); };
+    auto key = [](const SourceCall &c) { return 2 * source_form(c.g, c.t) + (c.qd ? 1 : 0); };
     return by_runs(calls, n, key, [&](const SourceCall *cs, int m) {
         Group<SourceInst> a;
         a.count = m;
@@ -4002,7 +4006,8 @@ extern const Ops IGR_OPS = {
     launch_speed, launch_rk_combine, launch_adj_rhs, launch_adj_diag, launch_adj_jacobi, launch_adj_source,
     launch_adj_add, launch_adj_jets, launch_adj_rk, launch_adj_rhs_scatter, launch_adj_rho,
     launch_adj_source_scatter, launch_diag, bounds_hits, bounds_selftest,
-    launch_source_group, launch_jacobi_group, launch_flux_group, source_shape, jacobi_shape,
+    launch_source_group, launch_jacobi_group, launch_flux_group, takes_quads_source, takes_quads_sweep,
+    source_shape, jacobi_shape,
     coefs_op<S>(), sweep_op<S>(),
 };
 

@@ -96,6 +96,7 @@ def lib():
             "igr_get_tiles": (i, [p, C.POINTER(i), C.POINTER(i), C.POINTER(i)]),
             "igr_set_kernel_forms": (i, [p, i, i]),
             "igr_get_kernel_forms": (i, [p, C.POINTER(i), C.POINTER(i)]),
+            "igr_get_launch_forms": (i, [p, C.POINTER(i), C.POINTER(i)]),
             "igr_autotune": (i, [p, i]),
             "igr_create_batch": (i, [C.POINTER(Config), i, C.POINTER(Allocator), p, C.POINTER(p)]),
             "igr_batch_instance": (p, [p, i]),
@@ -413,13 +414,20 @@ class Solver:
         return a.value, b.value, c.value
 
     def set_kernel_forms(self, source_vec4: int = -1, jacobi_vec4: int = -1):
-        """Accepted as -1, 0 or 1 (1: nx % 4 == 0) and returned by kernel_forms;
-        the kernels' form follows from the row length and the alignment."""
+        """Forms of the source and sweep kernels: 0 pairs, 1 quads (nx % 4 == 0),
+        -1 quads where nx % 4 == 0."""
         self._check(lib().igr_set_kernel_forms(self.h, int(source_vec4), int(jacobi_vec4)))
 
     def kernel_forms(self):
         a, b = C.c_int(), C.c_int()
         self._check(lib().igr_get_kernel_forms(self.h, C.byref(a), C.byref(b)))
+        return a.value, b.value
+
+    def launch_forms(self):
+        """What the steps launch for (source, sweeps): 1 quads, 0 pairs; sweeps
+        -1 in FP64 (one form, on stored coefficients)."""
+        a, b = C.c_int(), C.c_int()
+        self._check(lib().igr_get_launch_forms(self.h, C.byref(a), C.byref(b)))
         return a.value, b.value
 
     def autotune(self, reps: int = 3, cache: Optional[str] = None):
