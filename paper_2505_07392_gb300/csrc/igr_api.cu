@@ -1108,14 +1108,21 @@ template <typename F> static igr_status time_launches(igr_ctx *c, int reps, F fn
     return IGR_OK;
 }
 
-extern "C" {
+// Whether a grouped step runs this instance's sweeps by itself, on stored
+// coefficients: FP64 from 32^3 cells, a quarter of the grouped ones' operations
+// for more launches (twelve instances of 32^3: 2545 us per step against 2769,
+// four of 96^3: 13464 against 16027; twelve of 16^3: 1099 against 991)
+static bool own_sweeps(const igr_ctx *c) { return c->ops->sweep && c->g.n >= 32768; }
 
-igr_status igr_autotune(igr_ctx *c, int reps)
+// igr_autotune; grouped: the context's steps are those of a batch. Sweeps on
+// stored coefficients have neither chunk nor form, so theirs are left as they are.
+static igr_status tune(igr_ctx *c, int reps, bool grouped)
 {
     if (!c || reps < 1) return fail(c, IGR_ERR_INVALID_ARG, "ctx and reps >= 1 are required");
     if (c->profiling) return fail(c, IGR_ERR_INVALID_ARG, "disable profiling before tuning");
     // the default shape and chunks of 4..128 planes, pairs and, where rows allow, quads
     const int nforms = c->g.nx % 4 == 0 ? 2 : 1;
+    const bool sweeps = !c->ops->sweep || (grouped && !own_sweeps(c));
     const Tiles dflt = default_tiles(c->g, c->ops);
     const int cand[] = {0, 4, 8, 16, 32, 64, 128};
     Tiles best = c->tiles;
@@ -1140,6 +1147,7 @@ igr_status igr_autotune(igr_ctx *c, int reps)
             }, &ms);
             if (s != IGR_OK) return s;
             if (ms < tbest[0]) { tbest[0] = ms; best.zc_source = t.zc_source; best.vec_source = v; }
+            if (!sweeps) continue;
             s = time_launches(c, reps, [&] {
                 // red-black: a half-sweep in place on a copy of Sigma in the stage-1 output buffer
                 const void *qj = c->inc ? c->rho16 : c->q[0];
@@ -1160,6 +1168,10 @@ igr_status igr_autotune(igr_ctx *c, int reps)
     c->tiles = best;
     return IGR_OK;
 }
+
+extern "C" {
+
+igr_status igr_autotune(igr_ctx *c, int reps) { return tune(c, reps, false); }
 
 // ------------------------------------------------------------ batches
 
@@ -1297,13 +1309,8 @@ static igr_status step_grouped(igr_batch *b)
                 }
             if (o->source_group(sc.data(), (int)sc.size(), st) != cudaSuccess)
                 return bfail(b, IGR_ERR_CUDA, "grouped source launch");
-            // FP64 from 32^3 cells: each instance's own sweeps on stored coefficients, a
-            // quarter of the grouped ones' operations for more launches (twelve
-            // instances of 32^3: 2545 us per step against 2769, four of 96^3: 13464
-            // against 16027; twelve of 16^3: 1099 against 991)
-            auto own = [&](const igr_ctx *c) { return o->sweep && c->g.n >= 32768; };
             for (igr_ctx *c : inst) {
-                if (c->ops != o || !own(c)) continue;
+                if (c->ops != o || !own_sweeps(c)) continue;
                 const StageIO io = stage_io(c, stage);
                 void *res;
                 igr_status s = launch_sweeps(c, c->tiles, io.qs, c->b, c->sig[c->cur], c->sig[1 - c->cur], c->cfg.sweeps,
@@ -1317,7 +1324,7 @@ static igr_status step_grouped(igr_batch *b)
                     jc.clear();
                     for (igr_ctx *c : inst) {
                         const bool rb = c->cfg.sigma_solver == SOLVER_RBGS;
-                        if (c->ops != o || own(c) || k >= c->cfg.sweeps || (rb ? colour < 0 : colour >= 0)) continue;
+                        if (c->ops != o || own_sweeps(c) || k >= c->cfg.sweeps || (rb ? colour < 0 : colour >= 0)) continue;
                         const void *qj = c->inc ? c->rho16 : stage_io(c, stage).qs;
                         void *src = c->sig[c->cur], *dst = rb ? src : c->sig[1 - c->cur];
                         jc.push_back({c->g, c->p, c->tiles, qj, c->b, src, dst});
@@ -1326,7 +1333,7 @@ static igr_status step_grouped(igr_batch *b)
                     if (o->jacobi_group(jc.data(), (int)jc.size(), colour, st) != cudaSuccess)
                         return bfail(b, IGR_ERR_CUDA, "grouped sweep launch");
                     for (igr_ctx *c : inst)  // Jacobi sweeps alternate the two Sigma buffers
-                        if (c->ops == o && !own(c) && k < c->cfg.sweeps && c->cfg.sigma_solver != SOLVER_RBGS && colour < 0)
+                        if (c->ops == o && !own_sweeps(c) && k < c->cfg.sweeps && c->cfg.sigma_solver != SOLVER_RBGS && colour < 0)
                             c->cur = 1 - c->cur;
                 }
             fc.clear();
@@ -1425,7 +1432,7 @@ static igr_status time_class(igr_batch *b, int cls, const std::vector<Tiles> &t,
                     for (int i : b->order) {
                         igr_ctx *c = b->inst[i];
                         const bool rb = c->cfg.sigma_solver == SOLVER_RBGS;
-                        if (c->ops != o || rb != (colour == 0)) continue;
+                        if (c->ops != o || own_sweeps(c) || rb != (colour == 0)) continue;
                         const void *qj = c->inc ? c->rho16 : c->q[0];
                         if (rb)  // a half-sweep in place on the copy of Sigma in the stage-1 output buffer
                             jc.push_back({c->g, c->p, t[i], qj, c->b, c->q[1], c->q[1]});
@@ -1490,7 +1497,7 @@ igr_status igr_autotune_batch(igr_batch *b, int reps)
             c->tiles = b->inst[same]->tiles;
             continue;
         }
-        igr_status s = igr_autotune(c, reps);
+        igr_status s = tune(c, reps, true);
         if (s != IGR_OK) return bfail(b, s, igr_last_error(c));
     }
     // 2. the batch together: per kernel class, every instance's z-chunk
@@ -1507,6 +1514,7 @@ igr_status igr_autotune_batch(igr_batch *b, int reps)
     }
     const int factors[] = {1, 2, 4, 8, 16, 32};
     for (int cls : {KC_FLUX, KC_JACOBI, KC_SOURCE}) {
+        if (cls == KC_JACOBI && std::all_of(b->inst.begin(), b->inst.end(), own_sweeps)) continue;
         std::vector<Tiles> base(n), t(n), best;
         for (int i = 0; i < n; i++) base[i] = b->inst[i]->tiles;
         float tbest = 1e30f;
@@ -1517,7 +1525,7 @@ igr_status igr_autotune_batch(igr_batch *b, int reps)
                 const int nz = b->inst[i]->g.nz;
                 int &z = cls == KC_FLUX ? t[i].zc_flux : cls == KC_JACOBI ? t[i].zc_jacobi : t[i].zc_source;
                 const int z0 = z;
-                z = clamp_zc(z0 * f, nz);
+                if (cls != KC_JACOBI || !own_sweeps(b->inst[i])) z = clamp_zc(z0 * f, nz);
                 changed = changed || z != z0;
             }
             if (!changed) break;  // every chunk already spans its grid
