@@ -9,6 +9,8 @@ it raises if libigr.so has not been built (there is no CPU fallback).
 from __future__ import annotations
 
 import ctypes as C
+import functools
+import hashlib
 import os
 from typing import Optional, Sequence
 
@@ -171,13 +173,26 @@ def _dt_code(t):
 _NP_DT = {np.dtype(np.float64): DT_F64, np.dtype(np.float32): DT_F32, np.dtype(np.float16): DT_F16}
 
 
+@functools.lru_cache(maxsize=None)
+def _kernel_tag() -> str:
+    """Changes with the kernels that a stored launch shape was timed on (the
+    digest of their source, or of the library where it is installed alone): a
+    shape from other kernels is not a choice for these."""
+    source = [os.path.join(HERE, "csrc", f) for f in ("igr_internal.h", "igr_kernels.cu")]
+    h = hashlib.sha256()
+    for path in source if all(map(os.path.exists, source)) else [LIB_PATH]:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
 def autotune_key(case, precision: str, host_rk_base: bool, device_name: str) -> str:
     """What a tuned launch shape depends on: grid shape, storage precision,
-    scheme variant, RK base placement and GPU model."""
+    scheme variant, RK base placement, GPU model and the kernels."""
     visc = float(getattr(case, "mu", 0.0)) > 0 or float(getattr(case, "zeta", 0.0)) > 0
-    return "%dx%dx%d:%s:order%d:solver%d:visc%d:hostbase%d:%s" % (
+    return "%dx%dx%d:%s:order%d:solver%d:visc%d:hostbase%d:%s:kernels %s" % (
         case.nx, case.ny, case.nz, precision, int(getattr(case, "order", 5)),
-        int(getattr(case, "sigma_solver", 0)), int(visc), int(bool(host_rk_base)), device_name)
+        int(getattr(case, "sigma_solver", 0)), int(visc), int(bool(host_rk_base)), device_name, _kernel_tag())
 
 
 def autotune_cache_load(path: str) -> dict:
