@@ -264,14 +264,15 @@ const Ops *igr::ops_for(int p)
 // `resident` fit on an SM. A block spends c0 planes' time on the planes below
 // its chunk, and every wave of blocks the time of one, so a launch takes about
 // ceil(blocks / (152 resident)) (zc + c0); the chunk count with the least of
-// it is taken, chunks of 4 to 128 planes.
+// it is taken, chunks of 4 to 128 planes and, beyond the longest, no more of them
+// than a grid has along z.
 static int choose_zc(long long cols, int nz, int resident, double c0)
 {
     int best = nz < 4 ? nz : 4;
     double tbest = 1e300;
     for (int m = (nz + 127) / 128; m <= (nz + 3) / 4; m++) {
         const int zc = (nz + m - 1) / m;
-        if (zc < 4 && m > 1) break;
+        if (m > (nz + 127) / 128 && (zc < 4 || (nz + zc - 1) / zc > 65535)) break;
         const long long slots = 152LL * resident, blocks = cols * ((nz + zc - 1) / zc);
         const double t = (zc + c0) * (double)((blocks + slots - 1) / slots);
         if (t < tbest * 0.999) {
