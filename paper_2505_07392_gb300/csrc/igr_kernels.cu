@@ -136,7 +136,6 @@ __device__ __forceinline__ int cks(int c, int) { return c; }
 __device__ __forceinline__ int cks4(int c, int) { return c; }
 #endif
 
-template <int N> struct Fin { const S *p[N]; };   // fields read
 template <int N> struct Fout { S *p[N]; };        // fields written
 struct Frhs { C *p[5]; };
 struct QBIn { const QB *p[5]; };                  // the state q^n (RK base)
@@ -3410,13 +3409,6 @@ __global__ void __maxnreg__(FLUX_MAXREG) k_flux_group(const __grid_constant__ Gr
 dim3 grid_of(const Geom &g, int bx, int by, int zc)
 {
     return dim3((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, (g.nz + zc - 1) / zc);
-}
-
-template <int N> Fin<N> fields_in(const void *base, long long n)
-{
-    Fin<N> f;
-    for (int u = 0; u < N; u++) f.p[u] = base ? (const S *)base + u * n : nullptr;
-    return f;
 }
 
 // state input: base fields q (type QB) and increments qd (type S, or NULL)
