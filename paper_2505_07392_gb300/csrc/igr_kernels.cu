@@ -30,6 +30,7 @@
 
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "igr_internal.h"
 
@@ -3635,17 +3636,19 @@ cudaError_t launch_flux(const Geom &g, const Phys &p, const Tiles &t, const Infl
                    k_flux<FLUX_STAGE2, 5, false>, k_flux<FLUX_STAGE3, 5, false>);
 }
 
-// ---- grouped launches: calls are split by kernel form and in chunks of
+// ---- grouped launches: calls are grouped by kernel form and in chunks of
 // kGroupMax; each chunk is one launch over all its instances' blocks
 
-// run fn(first, count) over the runs of consecutive calls with equal key(call)
+// run fn(first, count) over the calls of each key(call), in their order
 template <class T, class K, class F>
-cudaError_t by_runs(const T *calls, int n, K key, F fn)
+cudaError_t by_key(const T *calls, int n, K key, F fn)
 {
+    std::vector<T> sorted(calls, calls + n);
+    std::stable_sort(sorted.begin(), sorted.end(), [&](const T &x, const T &y) { return key(x) < key(y); });
     for (int i = 0; i < n;) {
         int j = i + 1;
-        while (j < n && j - i < kGroupMax && key(calls[j]) == key(calls[i])) j++;
-        cudaError_t e = fn(calls + i, j - i);
+        while (j < n && j - i < kGroupMax && key(sorted[j]) == key(sorted[i])) j++;
+        cudaError_t e = fn(sorted.data() + i, j - i);
         if (e != cudaSuccess) return e;
         i = j;
     }
@@ -3657,7 +3660,7 @@ cudaError_t launch_source_group(const SourceCall *calls, int n, cudaStream_t st)
     for (int i = 0; i < n; i++)
         if ((kInc != (calls[i].rho_out != nullptr)) || (!kInc && calls[i].qd)) return cudaErrorInvalidValue;
     auto key = [](const SourceCall &c) { return 2 * source_form(c.g, c.t) + (c.qd ? 1 : 0); };
-    return by_runs(calls, n, key, [&](const SourceCall *cs, int m) {
+    return by_key(calls, n, key, [&](const SourceCall *cs, int m) {
         Group<SourceInst> a;
         a.count = m;
         int blk = 0, threads = 0;
@@ -3693,7 +3696,7 @@ cudaError_t launch_source_group(const SourceCall *calls, int n, cudaStream_t st)
 cudaError_t launch_jacobi_group(const JacobiCall *calls, int n, int colour, cudaStream_t st)
 {
     auto key = [](const JacobiCall &c) { return sweep_form(c.g, c.t); };
-    return by_runs(calls, n, key, [&](const JacobiCall *cs, int m) {
+    return by_key(calls, n, key, [&](const JacobiCall *cs, int m) {
         Group<JacobiInst> a;
         a.count = m;
         int blk = 0, threads = 0;
@@ -3738,7 +3741,7 @@ cudaError_t launch_flux_group(const FluxCall *calls, int n, int mode, cudaStream
         return 2 * (c.p.order == 3 ? 1 : 0) + (c.p.mu != 0.0 || c.p.zeta != 0.0 ? 1 : 0);
     };
     const size_t smem = flux_smem_bytes();
-    return by_runs(calls, n, kind, [&](const FluxCall *cs, int m) {
+    return by_key(calls, n, kind, [&](const FluxCall *cs, int m) {
         Group<FluxInst> a;
         a.count = m;
         int blk = 0;
