@@ -3429,6 +3429,7 @@ template <class K> cudaError_t allow_smem(K kern, int bytes)
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
+constexpr int kRows = sizeof(S) == 2 ? 2 : 1;  // rows per thread of form 3
 // Kernel form of a source or sweep launch: 2 full quad tiles, 1 fitted quad
 // tiles, 0 pairs; a sweep's form 3: full tiles with two rows per thread
 // (16-bit storage; from 16M cells: FP16, 512 x 512 x 128: 73 us against 79
@@ -3471,7 +3472,11 @@ void jacobi_shape(const Geom &g, long long *cols, int *resident)
     const dim3 gr = quad_grid(g, form, g.nz);
     *cols = (long long)gr.x * gr.y;
     const int blocks = form == 3 ? kJacobiBlocks<2> : form == 2 ? kJacobiBlocks<1> : form ? JACOBI_FIT_BLOCKS : JACOBI_PAIR_BLOCKS;
-    *resident = blocks * BT / quad_threads(g, form);
+    // shared memory holds two blocks of fitted quads in FP32 and FP64, four at 16 bits,
+    // however few threads they have (8 x 300 x 300, FP16: 54 us per five sweeps with
+    // the chunk for 16 blocks, 42 for 4; 4 x 4 x 2000, FP32: 46 and 36)
+    const int smem = form == 3 ? JShape<kRows>::SMEM : form ? JShape<1>::SMEM : 4 * TILEP * (int)sizeof(C);
+    *resident = std::min(blocks * BT / quad_threads(g, form), 227 * 1024 / (smem + 1024));
 }
 
 cudaError_t launch_source(const Geom &g, const Phys &p, const Tiles &t, const Inflow &in,
@@ -3495,7 +3500,6 @@ cudaError_t launch_source(const Geom &g, const Phys &p, const Tiles &t, const In
     }
 }
 
-constexpr int kRows = sizeof(S) == 2 ? 2 : 1;  // rows per thread of form 3
 template <int NR> auto full_sweep(int colour) { return colour < 0 ? k_jacobi_full<false, NR> : k_jacobi_full<true, NR>; }
 template <int NR> auto full_sweep_group(int colour)
 {
