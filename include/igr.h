@@ -379,8 +379,9 @@ igr_status igr_profile_read(igr_ctx *ctx, int kernel_class, long long *launches,
  * present setting: 1 quads, 0 pairs; sweeps -1 in FP64, whose sweeps on stored
  * coefficients have one form.
  * The sweep chunk has no effect on FP64 sweeps on stored coefficients (a
- * context's steps and igr_solve_sigma, and batch instances of 32768 cells and
- * more), which have none; the autotuners leave their chunk and form alone.
+ * context's steps and igr_solve_sigma; in a batch all but instances below 32768
+ * cells where more than ten are), which have none; the autotuners leave their
+ * chunk and form alone.
  * igr_autotune times each class on the current state for the default chunk
  * and the candidate lengths 4..128 and, where nx % 4 == 0, both forms (reps
  * launches each, on the context stream; only scratch buffers are written) and

@@ -54,6 +54,8 @@ struct igr_ctx {
     void *qalt;         // increment modes: the FP32 buffer stage 3 writes q^n+1 into
     void *rho16;        // increment modes: the stage density in the storage type
     bool inc;           // an increment mode
+    bool own_sweeps;    // a step's sweeps are the context's own, on stored coefficients (FP64; see
+                        // igr_create_batch for the instances whose sweeps are grouped)
     void *hbase;        // host_rk_base: pinned host buffer of the RK base (5 n values)
     void *hbase_dev;    // its device-mapped address
     void *sig[2];
@@ -626,6 +628,7 @@ igr_status igr_create(const igr_config *cfg, const igr_allocator *allocator, voi
     Layout L = layout_of(cfg);
     igr_status s = IGR_OK;
     c->inc = is_inc(cfg->prec);
+    c->own_sweeps = c->ops->sweep != nullptr;
     const int nstate = cfg->host_rk_base ? 2 : 3;
     for (int n = 0; n < nstate && s == IGR_OK; n++) s = ctx_alloc(c, &c->q[n], c->inc && n > 0 ? L.incr : L.state);
     if (s == IGR_OK && c->inc) s = ctx_alloc(c, &c->qalt, L.state);
@@ -1109,21 +1112,16 @@ template <typename F> static igr_status time_launches(igr_ctx *c, int reps, F fn
     return IGR_OK;
 }
 
-// Whether a grouped step runs this instance's sweeps by itself, on stored
-// coefficients: FP64 from 32^3 cells, a quarter of the grouped ones' operations
-// for more launches (twelve instances of 32^3: 2545 us per step against 2769,
-// four of 96^3: 13464 against 16027; twelve of 16^3: 1099 against 991)
-static bool own_sweeps(const igr_ctx *c) { return c->ops->sweep && c->g.n >= 32768; }
+extern "C" {
 
-// igr_autotune; grouped: the context's steps are those of a batch. Sweeps on
-// stored coefficients have neither chunk nor form, so theirs are left as they are.
-static igr_status tune(igr_ctx *c, int reps, bool grouped)
+// Sweeps on stored coefficients have neither chunk nor form: theirs are left alone.
+igr_status igr_autotune(igr_ctx *c, int reps)
 {
     if (!c || reps < 1) return fail(c, IGR_ERR_INVALID_ARG, "ctx and reps >= 1 are required");
     if (c->profiling) return fail(c, IGR_ERR_INVALID_ARG, "disable profiling before tuning");
     // the default shape and chunks of 4..128 planes, pairs and, where rows allow, quads
     const int nforms = c->g.nx % 4 == 0 ? 2 : 1;
-    const bool sweeps = !c->ops->sweep || (grouped && !own_sweeps(c));
+    const bool sweeps = !c->own_sweeps;
     const Tiles dflt = default_tiles(c->g, c->ops);
     const int cand[] = {0, 4, 8, 16, 32, 64, 128};
     Tiles best = c->tiles;
@@ -1169,10 +1167,6 @@ static igr_status tune(igr_ctx *c, int reps, bool grouped)
     c->tiles = best;
     return IGR_OK;
 }
-
-extern "C" {
-
-igr_status igr_autotune(igr_ctx *c, int reps) { return tune(c, reps, false); }
 
 // ------------------------------------------------------------ batches
 
@@ -1311,7 +1305,7 @@ static igr_status step_grouped(igr_batch *b)
             if (o->source_group(sc.data(), (int)sc.size(), st) != cudaSuccess)
                 return bfail(b, IGR_ERR_CUDA, "grouped source launch");
             for (igr_ctx *c : inst) {
-                if (c->ops != o || !own_sweeps(c)) continue;
+                if (c->ops != o || !c->own_sweeps) continue;
                 const StageIO io = stage_io(c, stage);
                 void *res;
                 igr_status s = launch_sweeps(c, c->tiles, io.qs, c->b, c->sig[c->cur], c->sig[1 - c->cur], c->cfg.sweeps,
@@ -1325,7 +1319,7 @@ static igr_status step_grouped(igr_batch *b)
                     jc.clear();
                     for (igr_ctx *c : inst) {
                         const bool rb = c->cfg.sigma_solver == SOLVER_RBGS;
-                        if (c->ops != o || own_sweeps(c) || k >= c->cfg.sweeps || (rb ? colour < 0 : colour >= 0)) continue;
+                        if (c->ops != o || c->own_sweeps || k >= c->cfg.sweeps || (rb ? colour < 0 : colour >= 0)) continue;
                         const void *qj = c->inc ? c->rho16 : stage_io(c, stage).qs;
                         void *src = c->sig[c->cur], *dst = rb ? src : c->sig[1 - c->cur];
                         jc.push_back({c->g, c->p, c->tiles, qj, c->b, src, dst});
@@ -1334,7 +1328,7 @@ static igr_status step_grouped(igr_batch *b)
                     if (o->jacobi_group(jc.data(), (int)jc.size(), colour, st) != cudaSuccess)
                         return bfail(b, IGR_ERR_CUDA, "grouped sweep launch");
                     for (igr_ctx *c : inst)  // Jacobi sweeps alternate the two Sigma buffers
-                        if (c->ops == o && !own_sweeps(c) && k < c->cfg.sweeps && c->cfg.sigma_solver != SOLVER_RBGS && colour < 0)
+                        if (c->ops == o && !c->own_sweeps && k < c->cfg.sweeps && c->cfg.sigma_solver != SOLVER_RBGS && colour < 0)
                             c->cur = 1 - c->cur;
                 }
             fc.clear();
@@ -1395,6 +1389,17 @@ igr_status igr_create_batch(const igr_config *cfgs, int n, const igr_allocator *
         snprintf(g_create_err, sizeof g_create_err, "%s", msg);
         return s;
     }
+    // FP64 instances below 32^3 cells sweep together, dividing, where they are more
+    // than ten: four times the operations in launches that all share, against eight
+    // of 3 us each per instance and stage (us per step, together and each its own:
+    // twelve of 16^3: 984 and 1073, eight: 960 and 876; twelve of 24^3: 1460 and 1531;
+    // ten of 13^3 to 31^3: 1874 and 1438; 64^3 and five smaller: 3217 and 2538).
+    // Larger ones gain either way (twelve of 32^3: 2769 and 2545, four of 96^3: 16027
+    // and 13464).
+    int small = 0;
+    for (const igr_ctx *c : b->inst) small += c->ops->sweep && c->g.n < 32768;
+    for (igr_ctx *c : b->inst)
+        if (c->g.n < 32768 && small > 10) c->own_sweeps = false;
     b->order.resize(n);
     for (int i = 0; i < n; i++) b->order[i] = i;
     std::stable_sort(b->order.begin(), b->order.end(),
@@ -1433,7 +1438,7 @@ static igr_status time_class(igr_batch *b, int cls, const std::vector<Tiles> &t,
                     for (int i : b->order) {
                         igr_ctx *c = b->inst[i];
                         const bool rb = c->cfg.sigma_solver == SOLVER_RBGS;
-                        if (c->ops != o || own_sweeps(c) || rb != (colour == 0)) continue;
+                        if (c->ops != o || c->own_sweeps || rb != (colour == 0)) continue;
                         const void *qj = c->inc ? c->rho16 : c->q[0];
                         if (rb)  // a half-sweep in place on the copy of Sigma in the stage-1 output buffer
                             jc.push_back({c->g, c->p, t[i], qj, c->b, c->q[1], c->q[1]});
@@ -1498,7 +1503,7 @@ igr_status igr_autotune_batch(igr_batch *b, int reps)
             c->tiles = b->inst[same]->tiles;
             continue;
         }
-        igr_status s = tune(c, reps, true);
+        igr_status s = igr_autotune(c, reps);
         if (s != IGR_OK) return bfail(b, s, igr_last_error(c));
     }
     // 2. the batch together: per kernel class, every instance's z-chunk
@@ -1515,7 +1520,8 @@ igr_status igr_autotune_batch(igr_batch *b, int reps)
     }
     const int factors[] = {1, 2, 4, 8, 16, 32};
     for (int cls : {KC_FLUX, KC_JACOBI, KC_SOURCE}) {
-        if (cls == KC_JACOBI && std::all_of(b->inst.begin(), b->inst.end(), own_sweeps)) continue;
+        if (cls == KC_JACOBI && std::all_of(b->inst.begin(), b->inst.end(), [](igr_ctx *c) { return c->own_sweeps; }))
+            continue;
         std::vector<Tiles> base(n), t(n), best;
         for (int i = 0; i < n; i++) base[i] = b->inst[i]->tiles;
         float tbest = 1e30f;
@@ -1526,7 +1532,7 @@ igr_status igr_autotune_batch(igr_batch *b, int reps)
                 const int nz = b->inst[i]->g.nz;
                 int &z = cls == KC_FLUX ? t[i].zc_flux : cls == KC_JACOBI ? t[i].zc_jacobi : t[i].zc_source;
                 const int z0 = z;
-                if (cls != KC_JACOBI || !own_sweeps(b->inst[i])) z = clamp_zc(z0 * f, nz);
+                if (cls != KC_JACOBI || !b->inst[i]->own_sweeps) z = clamp_zc(z0 * f, nz);
                 changed = changed || z != z0;
             }
             if (!changed) break;  // every chunk already spans its grid

@@ -1,6 +1,6 @@
 """The autotuners leave the sweep chunk alone where the sweeps have none (FP64 on
-stored coefficients: a lone context, a batch instance of 32^3 cells or more) and
-still choose it for the small instances of an FP64 batch and in FP32."""
+stored coefficients: a lone context, a large batch instance or one of few) and
+still choose it for the many small instances of an FP64 batch and in FP32."""
 import pytest
 
 from paper_2505_07392_gb300 import inputs
@@ -39,12 +39,19 @@ def test_lone_contexts():
 def test_batch():
     import torch
     from paper_2505_07392_gb300 import igr
-    cases = [inputs.tgv(32), inputs.tgv(16, instance=1), inputs.tgv(33, instance=2)]
+    # more than ten below 32^3 cells: those sweep together, by chunks
+    cases = [inputs.tgv(32), inputs.tgv(33, instance=1)] + [inputs.tgv(16, instance=i) for i in range(2, 13)]
     with igr.Batch(cases, "f64") as b:
         for inst, c in zip(b.instances, cases):
             inst.set_state(torch.from_numpy(inputs.initial_state(c)).cuda())
             inst.set_tiles(7, 7, 7)
         torch.cuda.synchronize()
         tiles = b.autotune(reps=1)
-        assert tiles[0][1] == 7 and tiles[2][1] == 7 and tiles[1][1] != 7
+        assert tiles[0][1] == 7 and tiles[1][1] == 7 and all(t[1] != 7 for t in tiles[2:])
         b.step(3, sync=True)
+    with igr.Batch(cases[:4], "f64") as b:  # few: each sweeps on its own
+        for inst, c in zip(b.instances, cases):
+            inst.set_state(torch.from_numpy(inputs.initial_state(c)).cuda())
+            inst.set_tiles(7, 7, 7)
+        torch.cuda.synchronize()
+        assert all(t[1] == 7 for t in b.autotune(reps=1))
