@@ -2017,8 +2017,13 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *sig, const QBI
             int lx, ly;
             plane_cell(e, lx, ly);
             soff[r] = ly * PW + lx;
-            goff[r] = (idx)(map_axis(y0 + ly - 3, g.ny, g.bc[2], g.bc[3]) * g.nx +
-                            map_axis(x0 + lx - 3, g.nx, g.bc[0], g.bc[1]));
+            // Columns that no cell of the grid reads (past nx + 2) mirror the last ones
+            // instead of repeating the last: a warp's cp.async copies of one address are
+            // served one by one, which made the ragged blocks of an outflow edge twice as
+            // long (right-hand side, FP32, 130 x 126 x 122: 138 us, 77 now; 75 periodic).
+            int x = x0 + lx - 3;
+            if (x > g.nx + 2 && g.bc[1] != BC_PERIODIC) x = max(2 * g.nx + 1 - x, 0);
+            goff[r] = (idx)(map_axis(y0 + ly - 3, g.ny, g.bc[2], g.bc[3]) * g.nx + map_axis(x, g.nx, g.bc[0], g.bc[1]));
         }
     }
 
