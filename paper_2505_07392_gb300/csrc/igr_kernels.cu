@@ -2944,23 +2944,27 @@ __global__ void __launch_bounds__(32 * XWARPS) k_adj_rhs_x(const S *q, const S *
     lsig[c] = v[5];
 }
 
-// The y- and z-faces' reverse: a thread marches along D over a chunk of cells
-// of one line (lanes along x, then the next line), with the six cells of the face's stencil and
-// the sums of the six cells it sends to in registers; a cell is written when
-// the last face that reads it is done. A chunk also evaluates the two faces
-// before and after it that reach its cells. Ends as for the x-faces; the
-// cells below an inflow face send to the cell above it (1 - W) and to the
-// inflow tables (lamJ).
+// The y- and z-faces' reverse, and in FP64 the x-faces' of short rows: a thread
+// marches along D over a chunk of cells of one line (lanes along x, then the next
+// line; along D = 0 a row per lane), with the six cells of the face's stencil and
+// the sums of the six cells it sends to; a cell is written when the last face that
+// reads it is done. A chunk also evaluates the two faces before and after it that
+// reach its cells. Ends as for the x-faces; the cells below an inflow face send to
+// the cell above it (1 - W) and to the inflow tables (lamJ). Along x it does the
+// stage combination's reverse as well. Not all of the sums are in registers: the
+// ends' additions index them, so one 6 x 6 array and `below` are in local memory
+// (stack frame: FP64 288 bytes along y, 656 along z; FP32 144 and 336).
 template <int D>
 __global__ void __launch_bounds__(128) k_adj_rhs_march(const S *q, const S *sig, const C *lout, C *lqs, C *lsig,
-                                                       C *lamJ, Geom g, C gamma, C inv_dx, C wdt, const C *W,
-                                                       const C *J, int chunk)
+                                                       C *lq0, C *lamJ, Geom g, C gamma, C inv_dx, C w, C wdt,
+                                                       int first, const C *W, const C *J, int chunk)
 {
-    const unsigned t = blockIdx.x * 128u + threadIdx.x, line = t / (unsigned)g.nx, i = t - line * (unsigned)g.nx;
-    if (line >= (unsigned)(D == 1 ? g.nz : g.ny)) return;
-    const int n = D == 1 ? g.ny : g.nz, blo = D == 1 ? g.bc[2] : g.bc[4], bhi = D == 1 ? g.bc[3] : g.bc[5];
+    const unsigned t = blockIdx.x * 128u + threadIdx.x, line = D == 0 ? t : t / (unsigned)g.nx,
+                   i = D == 0 ? 0u : t - line * (unsigned)g.nx;
+    if (line >= (unsigned)(D == 0 ? (idx)g.ny * (idx)g.nz : D == 1 ? g.nz : g.ny)) return;
+    const int n = D == 0 ? g.nx : D == 1 ? g.ny : g.nz, blo = g.bc[2 * D], bhi = g.bc[2 * D + 1];
     const bool per = blo == BC_PERIODIC, jet = D == 2 && blo == BC_INFLOW;
-    const idx step = D == 1 ? (idx)g.nx : (idx)g.plane;
+    const idx step = D == 0 ? 1u : D == 1 ? (idx)g.nx : (idx)g.plane;
     const idx base = (idx)line * (D == 1 ? (idx)g.plane : (idx)g.nx) + (idx)i;
     const int c0 = blockIdx.y * chunk, c1 = min(n, c0 + chunk);
     const int f0 = per ? c0 - 2 : max(0, c0 - 2), f1 = per ? c1 + 2 : min(n, c1 + 2);
@@ -2987,7 +2991,11 @@ __global__ void __launch_bounds__(128) k_adj_rhs_march(const S *q, const S *sig,
         const bool mine = c >= c0 && c < c1;
         const idx at = mine ? cell(c) : 0;
 #pragma unroll
-        for (int u = 0; u < 5; u++) v[u] = mine ? lqs[ckl((size_t)u * (size_t)g.n + at, 5 * g.n)] : C(0);
+        for (int u = 0; u < 5; u++) {
+            const size_t a = ckl((size_t)u * (size_t)g.n + at, 5 * g.n);
+            v[u] = !mine ? C(0) : D == 0 ? w * lout[a] : lqs[a];
+            if (D == 0 && mine) lq0[a] = first ? (C(1) - w) * lout[a] : lq0[a] + (C(1) - w) * lout[a];
+        }
         v[5] = mine ? lsig[at] : C(0);
     };
     auto write = [&](int c, const C (&v)[6]) {
@@ -3867,14 +3875,26 @@ cudaError_t launch_adj_rhs(const Geom &g, const Phys &p, const Inflow &in, const
     const C gamma = C(p.gamma), inv_dx = C(1.0 / p.dx), wdt = C(w) * C(dt);
     const long long rows = (long long)g.ny * g.nz;
     const int nseg = g.bc[0] == BC_PERIODIC ? (g.nx + XCELLS - 1) / XCELLS : (g.nx + 6 + XCELLS - 1) / XCELLS;
-    k_adj_rhs_x<<<(unsigned)((rows * nseg + XWARPS - 1) / XWARPS), 32 * XWARPS, 0, st>>>(
-        q, s, lo, (C *)lqs, (C *)lq0, (C *)lsig, g, gamma, inv_dx, C(w), wdt, first, nseg);
+    // FP64 rows of up to 12 cells: a warp of the gather has 32 faces' worth of FP64
+    // instructions for n + 1 (6 x 300 x 300, one step: 25.0 ms against 20.0 marching;
+    // 12 x 200 x 200: 12.6 and 11.4; 20 x 200 x 200: 15.1 and 15.5; in FP32 the march
+    // gains 6% at 6 cells and loses from 8)
+    bool thin = false;
+    if constexpr (sizeof(C) == 8) {
+        thin = g.nx <= 12;
+        if (thin)
+            k_adj_rhs_march<0><<<(unsigned)((rows + 127) / 128), 128, 0, st>>>(
+                q, s, lo, (C *)lqs, (C *)lsig, (C *)lq0, (C *)lamJ, g, gamma, inv_dx, C(w), wdt, first, W, J, g.nx);
+    }
+    if (!thin)
+        k_adj_rhs_x<<<(unsigned)((rows * nseg + XWARPS - 1) / XWARPS), 32 * XWARPS, 0, st>>>(
+            q, s, lo, (C *)lqs, (C *)lq0, (C *)lsig, g, gamma, inv_dx, C(w), wdt, first, nseg);
     const long long by = ((long long)g.nx * g.nz + 127) / 128, bz = (g.plane + 127) / 128;
     const int cy = march_chunk(by, g.ny), cz = march_chunk(bz, g.nz);
     k_adj_rhs_march<1><<<dim3((unsigned)by, (g.ny + cy - 1) / cy), 128, 0, st>>>(
-        q, s, lo, (C *)lqs, (C *)lsig, (C *)lamJ, g, gamma, inv_dx, wdt, W, J, cy);
+        q, s, lo, (C *)lqs, (C *)lsig, (C *)lq0, (C *)lamJ, g, gamma, inv_dx, C(w), wdt, first, W, J, cy);
     k_adj_rhs_march<2><<<dim3((unsigned)bz, (g.nz + cz - 1) / cz), 128, 0, st>>>(
-        q, s, lo, (C *)lqs, (C *)lsig, (C *)lamJ, g, gamma, inv_dx, wdt, W, J, cz);
+        q, s, lo, (C *)lqs, (C *)lsig, (C *)lq0, (C *)lamJ, g, gamma, inv_dx, C(w), wdt, first, W, J, cz);
     return cudaGetLastError();
 }
 
