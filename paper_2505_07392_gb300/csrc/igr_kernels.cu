@@ -2499,12 +2499,14 @@ __global__ void __launch_bounds__(DIAG_NT) k_diag(const QB *__restrict__ q, cons
 //            FP32 arithmetic without jets.
 //   scatter  one thread per face or cell adds to the cells it read by atomics
 //            (36 per face and 36 per cell of the source). Kept in FP32
-//            arithmetic with jets, where it is 3.9 times slower (128^3, four
-//            jets: 10.0 ms against 2.6 for the step): a jet's gradient is a
-//            double summed from these FP32 values with cancellation, so
-//            another order of addition moves it by 1e-7, beyond what two runs
-//            of the scatter differ by (4e-8; near the inflow face its order
-//            hardly varies).
+//            arithmetic with jets, where it takes 9.3 ms for a step of 128^3
+//            and four jets: its order of additions is not fixed, and dJ/dw, a
+//            double summed from these FP32 values with cancellation, moves with
+//            it, by 1e-8 to 1.3e-7 between two runs (median 3e-8) and by up to
+//            8e-8 in the mean between two allocations of the same buffers. The
+//            gather (2.6 ms) repeats its bits but moves dJ/dw by 0.6e-7 to
+//            2.5e-7 and is less exact for some states (against FP64 3.3e-7 where
+//            the scatter has 2.2e-7, 1.1e-7 where it has 0.5e-7).
 // The reversed sweeps gather in both. Adjoint values are in the arithmetic
 // type C. Non-smooth points follow the forward's branch: the LF speed
 // max(aL, aR) sends its adjoint to the side the forward took (aR on a tie),
@@ -3445,8 +3447,10 @@ template <class K> cudaError_t allow_smem(K kern, int bytes)
 constexpr int kRows = sizeof(S) == 2 ? 2 : 1;  // rows per thread of form 3
 // Kernel form of a source or sweep launch: 2 full quad tiles, 1 fitted quad
 // tiles, 0 pairs; a sweep's form 3: full tiles with two rows per thread
-// (16-bit storage; from 16M cells: FP16, 512 x 512 x 128: 73 us against 79
-// with one; 256 x 256 x 192: 32 against 29.5). Its grid and block.
+// (16-bit storage, from 2M cells, where the tiles of one row fill the SMs more than
+// once; FP16, two rows against one: 128^3 7.0 and 7.3 us, 256 x 256 x 128 20.4 and
+// 22.7, 256 x 256 x 192 29.4 and 32.6, 512 x 512 x 128 73 and 80, 512^3 262 and 295;
+// 128 x 128 x 64 6.9 and 6.1). Its grid and block.
 int quad_form(const Geom &g, const Tiles &t, int vec)
 {
     if (t.elem || vec == 0 || g.nx % VX != 0) return 0;
@@ -3456,10 +3460,11 @@ int source_form(const Geom &g, const Tiles &t) { return quad_form(g, t, t.vec_so
 int sweep_form(const Geom &g, const Tiles &t)
 {
     const int form = quad_form(g, t, t.vec_jacobi);
-    return form == 2 && sizeof(S) == 2 && g.ny % (2 * FR) == 0 && g.n >= (1 << 24) ? 3 : form;
+    return form == 2 && sizeof(S) == 2 && g.ny % (2 * FR) == 0 && g.n >= (1 << 21) ? 3 : form;
 }
-// the source takes the compiled-in tile in the 16-bit forms only (FP32, 256^3:
-// 90.8 us against 72.2 with the tile's shape at run time)
+// the source takes the compiled-in tile in the 16-bit forms only (FP16, compiled in
+// against shape at run time: 128^3 7.7 and 8.7 us, 512 x 512 x 128 114 and 164; FP32:
+// 9.5 and 9.9, 171 and 138, 256 x 128 x 128 27.1 and 22.5)
 bool source_full(int form) { return form == 2 && sizeof(S) == 2; }
 dim3 quad_grid(const Geom &g, int form, int zc)
 {
