@@ -1112,15 +1112,15 @@ template <typename F> static igr_status time_launches(igr_ctx *c, int reps, F fn
     return IGR_OK;
 }
 
-extern "C" {
-
-// Sweeps on stored coefficients have neither chunk nor form: theirs are left alone.
-igr_status igr_autotune(igr_ctx *c, int reps)
+// igr_autotune; forms: both forms are tried (an instance of a batch keeps its own: the
+// faster form alone may take it out of the launch that it shares). Sweeps on stored
+// coefficients have neither chunk nor form: theirs are left alone.
+static igr_status tune(igr_ctx *c, int reps, bool forms)
 {
     if (!c || reps < 1) return fail(c, IGR_ERR_INVALID_ARG, "ctx and reps >= 1 are required");
     if (c->profiling) return fail(c, IGR_ERR_INVALID_ARG, "disable profiling before tuning");
     // the default shape and chunks of 4..128 planes, pairs and, where rows allow, quads
-    const int nforms = c->g.nx % 4 == 0 ? 2 : 1;
+    const int nforms = forms && c->g.nx % 4 == 0 ? 2 : 1;
     const bool sweeps = !c->own_sweeps;
     const Tiles dflt = default_tiles(c->g, c->ops);
     const int cand[] = {0, 4, 8, 16, 32, 64, 128};
@@ -1140,12 +1140,13 @@ igr_status igr_autotune(igr_ctx *c, int reps)
         igr_status s;
         // each kernel class writes only scratch: b, the other Sigma buffer, the stage-1 output
         for (int v = 0; v < nforms; v++) {
-            t.vec_source = t.vec_jacobi = v;
+            t.vec_source = forms ? v : c->tiles.vec_source;
+            t.vec_jacobi = forms ? v : c->tiles.vec_jacobi;
             s = time_launches(c, reps, [&] {
                 return c->ops->source(c->g, c->p, t, inflow_of(c), c->q[0], nullptr, c->b, c->rho16, c->st);
             }, &ms);
             if (s != IGR_OK) return s;
-            if (ms < tbest[0]) { tbest[0] = ms; best.zc_source = t.zc_source; best.vec_source = v; }
+            if (ms < tbest[0]) { tbest[0] = ms; best.zc_source = t.zc_source; best.vec_source = t.vec_source; }
             if (!sweeps) continue;
             s = time_launches(c, reps, [&] {
                 // red-black: a half-sweep in place on a copy of Sigma in the stage-1 output buffer
@@ -1155,7 +1156,7 @@ igr_status igr_autotune(igr_ctx *c, int reps)
                            : c->ops->jacobi(c->g, c->p, t, qj, c->b, sig, scratch, -1, c->st);
             }, &ms);
             if (s != IGR_OK) return s;
-            if (ms < tbest[1]) { tbest[1] = ms; best.zc_jacobi = t.zc_jacobi; best.vec_jacobi = v; }
+            if (ms < tbest[1]) { tbest[1] = ms; best.zc_jacobi = t.zc_jacobi; best.vec_jacobi = t.vec_jacobi; }
         }
         s = time_launches(c, reps, [&] {
             return c->ops->flux(c->g, c->p, t, inflow_of(c), FLUX_STAGE1, c->q[0], nullptr, sig, c->q[0], c->q[1],
@@ -1167,6 +1168,10 @@ igr_status igr_autotune(igr_ctx *c, int reps)
     c->tiles = best;
     return IGR_OK;
 }
+
+extern "C" {
+
+igr_status igr_autotune(igr_ctx *c, int reps) { return tune(c, reps, true); }
 
 // ------------------------------------------------------------ batches
 
@@ -1503,7 +1508,7 @@ igr_status igr_autotune_batch(igr_batch *b, int reps)
             c->tiles = b->inst[same]->tiles;
             continue;
         }
-        igr_status s = igr_autotune(c, reps);
+        igr_status s = tune(c, reps, false);
         if (s != IGR_OK) return bfail(b, s, igr_last_error(c));
     }
     // 2. the batch together: per kernel class, every instance's z-chunk
