@@ -145,10 +145,10 @@ struct QBOut { QB *p[5]; };                       // a new state q^n+1
 // ------------------------------------------------------------ load/store
 // Read-only (non-coherent) loads, for kernels that are launched plainly. A kernel
 // that begins with launched() is resident while its predecessor writes, so it
-// takes ordinary loads (ldr, ld4r, cp.async) and no __restrict__ pointers, and the
-// writes that it waited for are visible to them. They cost nothing: every case
-// within 0.5% of the read-only loads' time (plume 1024 x 1024 x 512, FP16
-// increments: 140.0 ms before, 139.7 now; ten steps at 32^3: 1200 and 1194 us).
+// takes ordinary loads (ldv, ldr, ld4r, cp.async) and no __restrict__ pointers, and
+// the writes that it waited for are visible to them. They cost next to nothing
+// (plume 1024 x 1024 x 512, FP16 increments: 140.0 ms before, 139.7 now; two steps
+// of 512 x 512 x 128: FP16 8.43 and 8.39 ms, FP32 9.58 and 9.64, BF16 8.42 and 8.78).
 __device__ __forceinline__ double ldc(const double *p) { return __ldg(p); }
 __device__ __forceinline__ float ldc(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ldc(const __half *p) { return __half2float(__ldg(p)); }
@@ -157,7 +157,25 @@ __device__ __forceinline__ float ldc(const __nv_bfloat16 *p) { return __bfloat16
 // Raw (ordinary) loads for prefetching: the value stays in its storage type until it is
 // used, so no instruction waits on the load before then (a conversion right
 // after the load would stall there and hide nothing).
-__device__ __forceinline__ S ldr(const S *p) { return *p; }
+// An ordinary load in the order of the source: the compiler may not move it over
+// the wait, and the element loads of a plane stay together (as plain reads, which it
+// moves between the stores, two FP16 steps of 512 x 512 x 128 took 8.51 ms against
+// 8.39, the right-hand side with FP16 increments 818 us against 785).
+__device__ __forceinline__ double ldv(const double *p) { return *p; }
+__device__ __forceinline__ float ldv(const float *p)
+{
+    float r;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(r) : "l"(p));
+    return r;
+}
+template <class H> __device__ __forceinline__ H ldv(const H *p)
+{
+    static_assert(sizeof(H) == 2, "16-bit types");
+    unsigned short r;
+    asm volatile("ld.global.b16 %0, [%1];" : "=h"(r) : "l"(p));
+    return *reinterpret_cast<H *>(&r);
+}
+__device__ __forceinline__ S ldr(const S *p) { return ldv(p); }
 __device__ __forceinline__ double cv(double v) { return v; }
 __device__ __forceinline__ float cv(float v) { return v; }
 __device__ __forceinline__ float cv(__half v) { return __half2float(v); }
@@ -190,7 +208,7 @@ template <> struct StateIO<true> {
     template <bool HASD> static __device__ __forceinline__ QRawInc ld(const QIn &q, int u, idx c)
     {
         QRawInc r;
-        r.b = q.b[0][u * q.fs + c];
+        r.b = ldv(q.b[0] + u * q.fs + c);
         r.d = HASD ? ldr(q.d[0] + u * q.fs + c) : S(0.0f);
         return r;
     }
@@ -1973,7 +1991,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *sig, const QBI
     auto ldq_raw = [&](int u, idx c) -> QRaw {
         if constexpr (kInc) {
             QRawInc r;
-            r.b = qb0[u * fs + c];
+            r.b = ldv(qb0 + u * fs + c);
             r.d = HASD ? ldr(qd0 + u * fs + c) : S(0.0f);
             return *reinterpret_cast<QRaw *>(&r);
         } else {
@@ -2230,7 +2248,7 @@ __device__ __forceinline__ void flux_body(const QIn qin, const S *sig, const QBI
                 if (k >= k0 && (mode == FLUX_STAGE2 || mode == FLUX_STAGE3)) {
                     idx c = ck((idx)k * pl + own, g.n);
 #pragma unroll
-                    for (int u = 0; u < 5; u++) qnv[u] = kInc ? qn0[u * fs + c] : qn.p[u][c];
+                    for (int u = 0; u < 5; u++) qnv[u] = ldv(kInc ? qn0 + u * fs + c : qn.p[u] + c);
                 }
             }
             Fzm = Fzp;
