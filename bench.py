@@ -50,15 +50,15 @@ FALLBACK_HBM_GBS = 6800.0
 # Both from ncu captures of the flux kernel on the 512 x 512 x 128 plume,
 # mean of the three stage launches of one step.
 NCU_INSTR = {
-    "flux_f16inc": {"warp_instr_per_cell": 20.142, "src": "ed6d2d52d92802c7"},
-    "flux_f16": {"warp_instr_per_cell": 21.409, "src": "ed6d2d52d92802c7"},
-    "flux_f32": {"warp_instr_per_cell": 18.333, "src": "ed6d2d52d92802c7"},
+    "flux_f16inc": {"warp_instr_per_cell": 19.943, "src": "5b7794e850f179b4"},
+    "flux_f16": {"warp_instr_per_cell": 21.198, "src": "5b7794e850f179b4"},
+    "flux_f32": {"warp_instr_per_cell": 18.314, "src": "5b7794e850f179b4"},
 }
 
 NCU_TRAFFIC = {
-    "flux_f16inc": {"bytes_per_cell": 42.831, "src": "ed6d2d52d92802c7"},
-    "flux_f16": {"bytes_per_cell": 28.632, "src": "ed6d2d52d92802c7"},
-    "flux_f32": {"bytes_per_cell": 57.610, "src": "ed6d2d52d92802c7"},
+    "flux_f16inc": {"bytes_per_cell": 42.861, "src": "5b7794e850f179b4"},
+    "flux_f16": {"bytes_per_cell": 28.640, "src": "5b7794e850f179b4"},
+    "flux_f32": {"bytes_per_cell": 57.605, "src": "5b7794e850f179b4"},
 }
 
 

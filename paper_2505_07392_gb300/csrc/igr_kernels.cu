@@ -1953,9 +1953,8 @@ constexpr int FLUX_MAXREG = sizeof(C) == 8 ? 224 : 128;
 // global memory once per block; nothing relies on the L1 cache.
 //
 // What bounds it is the latency of 16 warps' shared loads, MUFU operations
-// and dependent arithmetic (issue slots 57% busy, shared-memory bandwidth
-// 42%, no pipe above 45%): the face flux is packed by variable pairs and the
-// face buffers hold quads (FP16 increments, stage 2: 695 -> 604 instructions
+// and dependent arithmetic (issue slots 56-68% busy, no pipe above 35%): the face flux is packed by variable pairs and the
+// face buffers hold quads (FP16 increments, stage 2: 695 -> 657 instructions
 // per cell), and the prologue's planes are loaded three at a time. Per launch,
 // stages 1 to 3: FP16 increments 1024 x 1024 x 256 7.26 -> 7.02 ms, FP32
 // 512 x 512 x 256 1.96 -> 1.78 ms, 32^3 18.6 -> 16.8 us. Measured and not
